@@ -239,9 +239,11 @@ def mrr_work(n: int, N: int) -> dict:
     special prime and n RNS digits, rescale) at n data limbs and degree N:
     n^2 + 5n + 2 transforms of (N/2) log2 N butterflies; N (2n^2 + 16n - 4)
     further modular products (tensor 4n, key products 2n(n+1), d P 2n,
-    mod-down 2n + 2n centred reductions, rescale 2(n-1) + 2(n-1)); HBM bytes:
-    the two input ciphertexts read and the output written once (the
-    resident key is not counted)."""
+    mod-down 2n + 2n centred reductions, rescale 2(n-1) + 2(n-1)): the method
+    as written, one transform per limb and division; the kernels share one
+    between the two divisions and run n^2 + 3n + 2. HBM bytes: the two input
+    ciphertexts read and the output written once (the resident key is not
+    counted)."""
     log_n = N.bit_length() - 1
     return {"bfly": (n * n + 5 * n + 2) * (N // 2) * log_n, "products": N * (2 * n * n + 16 * n - 4),
             "bytes": (4 * n + 2 * (n - 1)) * N * 8}

@@ -203,6 +203,7 @@ struct he_ntt_tables {
     ulonglong2 *d_fwd = nullptr;  // [K][N] (W, W')
     ulonglong2 *d_inv = nullptr;
     he::PrimeConst *d_pc = nullptr;
+    std::vector<he::PrimeConst> h_pc;   // host copy of d_pc
 };
 
 // the lazy butterfly ranges need 2^30 <= q < 2^60 (Sec. III-A-1: below 60 bits)
@@ -292,6 +293,7 @@ extern "C" he_status he_ntt_tables_create(uint32_t N, uint32_t limbs, const uint
         free_tables(t);
         return cuda_fail(e, "upload twiddle tables");
     }
+    t->h_pc = std::move(pcs);
     *out = t;
     return HE_OK;
 }
@@ -592,6 +594,7 @@ struct he_context {
     u64 P = 0;
     he_ntt_tables *tables = nullptr;   // primes q_0..q_L, P
     u64 *d_cst = nullptr;
+    he::PrimeConst *d_pc_lift = nullptr;
     std::atomic<int> eval_log_e{4};    // words per thread of the evaluation kernels
 };
 
@@ -629,7 +632,8 @@ extern "C" he_status he_context_create(uint32_t N, uint32_t n_data, const uint64
         delete c;
         return s;
     }
-    std::vector<u64> cst(3 * (size_t)n_data + 3 * (size_t)n_data * n_data + n_data, 0);
+    std::vector<u64> cst(4 * (size_t)n_data + 6 * (size_t)n_data * n_data, 0);
+    std::vector<he::PrimeConst> lift(n_data + 1);
     for (u32 i = 0; i < n_data; i++) {
         const u64 q = all[i];
         cst[3 * i + 0] = h_inv(special_modulus % q, q);
@@ -644,12 +648,30 @@ extern "C" he_status he_context_create(uint32_t N, uint32_t n_data, const uint64
             d[0] = h_inv(ql % q, q);
             d[1] = shoup(d[0], q);
             d[2] = ql % q;
+            u64 *r = &cst[n_data * (4 + 3 * (size_t)n_data) + 3 * ((size_t)l * n_data + i)];
+            const u64 Pql = h_mul(special_modulus % q, ql % q, q);   // never 0: the primes differ
+            r[0] = h_inv(Pql, q);
+            r[1] = shoup(r[0], q);
+            r[2] = q - Pql;
         }
+    for (u32 i = 0; i <= n_data; i++) {
+        he::PrimeConst &k = lift[i];
+        k = c->tables->h_pc[i];
+        if (i == n_data) continue;
+        k.ninv = h_mul(k.ninv, cst[3 * i], k.p);
+        k.ninv_sh = shoup(k.ninv, k.p);
+        k.w1ninv = h_mul(k.w1ninv, cst[3 * i], k.p);
+        k.w1ninv_sh = shoup(k.w1ninv, k.p);
+    }
     cudaError_t e = cudaMalloc(&c->d_cst, cst.size() * sizeof(u64));
     if (e == cudaSuccess) e = cudaMemcpy(c->d_cst, cst.data(), cst.size() * sizeof(u64), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&c->d_pc_lift, lift.size() * sizeof(lift[0]));
+    if (e == cudaSuccess)
+        e = cudaMemcpy(c->d_pc_lift, lift.data(), lift.size() * sizeof(lift[0]), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
         he_ntt_tables_destroy(c->tables);
         cudaFree(c->d_cst);
+        cudaFree(c->d_pc_lift);
         delete c;
         return cuda_fail(e, "context constants");
     }
@@ -672,6 +694,7 @@ extern "C" he_status he_context_destroy(he_context *ctx)
         cudaDeviceSynchronize();
         he_ntt_tables_destroy(ctx->tables);
         cudaFree(ctx->d_cst);
+        cudaFree(ctx->d_pc_lift);
         delete ctx;
     }
     return HE_OK;
@@ -726,6 +749,7 @@ static he::DevCtx dev_ctx(const he_context *c)
     d.tw_fwd = c->tables->d_fwd;
     d.tw_inv = c->tables->d_inv;
     d.pc = c->tables->d_pc;
+    d.pc_lift = c->d_pc_lift;
     d.cst = c->d_cst;
     d.N = c->N;
     d.n_data = c->n_data;
@@ -822,9 +846,10 @@ static he_status plift_intt(const he_context *ctx, u64 *plift, u32 limbs, cudaSt
 // With room for the expanded buffer (x_words at xbuf, at least one
 // ciphertext's (n + 1) n N words) the transforms run as independent plain-
 // size launches (k_ks_expand), the key products as an elementwise pass
-// (k_ks_mac) and the special prime's accumulators go through the inverse
-// transform in place; the buffer takes groups of up to kModupGroup
-// ciphertexts. Otherwise the fused k_ks_modup runs.
+// (k_ks_mac); the buffer takes groups of up to kModupGroup ciphertexts, and
+// the special prime's accumulators in plift are left in the NTT domain
+// (*special_ntt = true). Otherwise the fused k_ks_modup runs, which also takes
+// them through the inverse transform.
 // The tiled key multiply-accumulate's shared memory, 2 n MAC_TILE key pairs
 // (64 KB at the largest chain, n = 32), above the default 48 KB limit.
 static cudaError_t mac_tiled_smem_attr()
@@ -839,11 +864,12 @@ static cudaError_t mac_tiled_smem_attr()
 }
 
 static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64 *xbuf, size_t x_words,
-                          cudaStream_t s)
+                          bool *special_ntt, cudaStream_t s)
 {
     const u32 n = a.n;
     const size_t per = (size_t)(n + 1) * n * ctx->N;
     const u32 group = (u32)std::min<size_t>({(size_t)kModupGroup, (size_t)count, xbuf ? x_words / per : 0});
+    *special_ntt = group > 0;
     if (group == 0) return run_eval(ctx, he::EK_KS_MODUP, a, count * (n + 1), s);
     a.mx = xbuf;
     for (u32 c0 = 0; c0 < count; c0 += group) {
@@ -863,7 +889,7 @@ static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64
     }
     a.mx = nullptr;
     a.c_first = 0;
-    return plift_intt(ctx, a.plift, 2 * count, s);
+    return HE_OK;
 }
 
 extern "C" he_status he_relin(uint64_t *ct_out2, const uint64_t *ct_in3, const he_relin_key *key,
@@ -891,7 +917,10 @@ extern "C" he_status he_relin(uint64_t *ct_out2, const uint64_t *ct_in3, const h
     u64 *xbuf = (u64 *)scratch + relin_words(ctx, n);
     const size_t x_words = scratch_bytes / 8 - relin_words(ctx, n);
     if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, n, s)) return r;
-    if (he_status r = ks_modup(ctx, a, 1, xbuf, x_words, s)) return r;
+    bool special_ntt = false;
+    if (he_status r = ks_modup(ctx, a, 1, xbuf, x_words, &special_ntt, s)) return r;
+    if (special_ntt)
+        if (he_status r = plift_intt(ctx, a.plift, 2, s)) return r;
     return run_eval(ctx, he::EK_KS_MODDOWN, a, 2 * n, s);
 }
 
@@ -955,11 +984,15 @@ static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const
     u64 *xbuf = (u64 *)scratch + base_words;
     const size_t x_words = scratch_bytes / 8 - base_words;
     if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, count * n, s)) return r;
-    if (he_status r = ks_modup(ctx, a, count, xbuf, x_words, s)) return r;
-    if (!rescale) return run_eval(ctx, he::EK_KS_MODDOWN, a, count * 2 * n, s);
-    if (he_status r = run_eval(ctx, he::EK_MRR_LAST, a, count * 2, s)) return r;
-    if (he_status r = run_eval(ctx, he::EK_MRR_REST_Z, a, count * 2 * level, s)) return r;
-    return run_eval(ctx, he::EK_MRR_REST_OUT, a, count * 2 * level, s);
+    bool special_ntt = false;
+    if (he_status r = ks_modup(ctx, a, count, xbuf, x_words, &special_ntt, s)) return r;
+    if (!rescale) {
+        if (special_ntt)
+            if (he_status r = plift_intt(ctx, a.plift, 2 * count, s)) return r;
+        return run_eval(ctx, he::EK_KS_MODDOWN, a, count * 2 * n, s);
+    }
+    if (he_status r = run_eval(ctx, he::EK_MRR_LIFT, a, count * (special_ntt ? 4 : 2), s)) return r;
+    return run_eval(ctx, he::EK_MRR_REST, a, count * 2 * level, s);
 }
 
 extern "C" he_status he_mul_relin_rescale(uint64_t *ct_out, const uint64_t *ct_a, const uint64_t *ct_b,
@@ -1052,7 +1085,7 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
         E.evk = key->d_evk;
         E.ctx = dev_ctx(ctx);
         const u64 items[he::JS_COUNT] = {(u64)c * n, (u64)c * (n + 1) * n,
-                                         (u64)(c + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (ctx->N / 2), 2ull * c,
+                                         (u64)(c + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (ctx->N / 2), 4ull * c,
                                          2ull * c * (n - 1)};
         for (int st = 0; st < he::JS_COUNT; st++) {
             if (tot[st] + items[st] > 0x7fffffffull) return fail(HE_EINVAL, "batch too large");
@@ -1071,10 +1104,8 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
     if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, (u32)tot[he::JS_EXPAND], s, &t)) return r;
     he::k_ks_mac<true><<<stream_grid(tot[he::JS_MAC], 256), 256, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
-    if (he_status r = plift_intt(ctx, plift, 2 * pairs, s)) return r;
-    if (he_status r = run_eval(ctx, he::EK_MRR_LAST, a, (u32)tot[he::JS_LAST], s, &t)) return r;
-    if (he_status r = run_eval(ctx, he::EK_MRR_REST_Z, a, (u32)tot[he::JS_REST], s, &t)) return r;
-    return run_eval(ctx, he::EK_MRR_REST_OUT, a, (u32)tot[he::JS_REST], s, &t);
+    if (he_status r = run_eval(ctx, he::EK_MRR_LIFT, a, (u32)tot[he::JS_LIFT], s, &t)) return r;
+    return run_eval(ctx, he::EK_MRR_REST, a, (u32)tot[he::JS_REST], s, &t);
 }
 
 extern "C" he_status he_mul_relin_rescale_batch(const he_mrr_job *jobs_host, uint32_t n_jobs,
@@ -1957,9 +1988,8 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
         cnt[he::JS_DIGITS] = units((u64)c * n);
         cnt[he::JS_EXPAND] = units((u64)c * n * n);
         cnt[he::JS_MAC] = (u64)(c + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (N / 2);
-        cnt[he::JS_LAST] = units(2ull * c);
+        cnt[he::JS_LIFT] = units(4ull * c);
         cnt[he::JS_REST] = units(2ull * c * (n - 1));
-        cnt[he::JS_PLIFT] = units(2ull * c);
         for (int st = 0; st < he::JS_COUNT; st++) {
             if (tot[st] + cnt[st] > 0x0fffffffull) return fail(HE_EINVAL, "batch too large");
             E.begin[st] = (u32)tot[st];
@@ -1974,10 +2004,8 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
     HE_CUDA(he::launch_mrr_multi(he::MS_EXPAND, a, t, (u32)tot[he::JS_EXPAND], s));
     he::k_ks_mac<true><<<stream_grid(tot[he::JS_MAC], 256), 256, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
-    HE_CUDA(he::launch_mrr_multi(he::MS_PLIFT, a, t, (u32)tot[he::JS_PLIFT], s));
-    HE_CUDA(he::launch_mrr_multi(he::MS_LAST, a, t, (u32)tot[he::JS_LAST], s));
-    HE_CUDA(he::launch_mrr_multi(he::MS_REST_Z, a, t, (u32)tot[he::JS_REST], s));
-    HE_CUDA(he::launch_mrr_multi(he::MS_REST_OUT, a, t, (u32)tot[he::JS_REST], s));
+    HE_CUDA(he::launch_mrr_multi(he::MS_LIFT, a, t, (u32)tot[he::JS_LIFT], s));
+    HE_CUDA(he::launch_mrr_multi(he::MS_REST, a, t, (u32)tot[he::JS_REST], s));
     return HE_OK;
 }
 

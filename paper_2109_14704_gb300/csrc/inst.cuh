@@ -148,9 +148,8 @@ struct ShapeOps {
             HE_EVAL_CASE(EK_KS_MODDOWN, k_ks_moddown, sm1)
             HE_EVAL_CASE(EK_RS_LIFT, k_rs_lift, sm1)
             HE_EVAL_CASE(EK_RS, k_rs, sm1)
-            HE_EVAL_CASE_J(EK_MRR_LAST, k_mrr_last, sm1)
-            HE_EVAL_CASE_J(EK_MRR_REST_Z, k_mrr_rest_z, sm1)
-            HE_EVAL_CASE_J(EK_MRR_REST_OUT, k_mrr_rest_out, sm1)
+            HE_EVAL_CASE_J(EK_MRR_LIFT, k_mrr_lift, sm1)
+            HE_EVAL_CASE_J(EK_MRR_REST, k_mrr_rest, sm1)
 #undef HE_EVAL_CASE_J
 #undef HE_EVAL_CASE
         default:

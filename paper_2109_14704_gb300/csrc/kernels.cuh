@@ -628,9 +628,8 @@ __global__ void k_enc_combine(u64 *ct, const u64 *noise, const u64 *pt, const u6
 //                 r_k the centred lift of y_k                        (2n NTT)
 // RS (Sec. II-A): k_rs_lift brings c_k[q_l] to the coefficient domain
 // (2 INTT), k_rs combines (c_k[q_i] - NTT(r mod q_i)) q_l^-1 (2(n-1) NTT).
-// MulLinRS fuses Mul into the loads and the mod-down of limb q_l with RS's
-// INTT (k_mrr_last), and mod-down with RS for the other limbs (k_mrr_rest_z,
-// k_mrr_rest_out).
+// MulLinRS fuses Mul into the loads and the two divisions into one transform
+// per remaining limb (k_mrr_lift, k_mrr_rest).
 
 // Centred residue of y in [0, m) (|r| <= (m-1)/2) reduced mod q:
 // y mod q, or y mod q - m mod q when y > (m-1)/2 (any word y).
@@ -1194,142 +1193,126 @@ k_rs(EvalArgs a)
     store_run<Sh>(out, x, m, tid);
 }
 
-// MulLinRS, limb q_l: relin output c_k[q_l] = d_k[l] + (acc - NTT(r)) P^-1,
-// then straight into INTT_{q_l} (values stay in registers) -> lift2;
-// item = 2 c + k.
-template <class Sh>
-__device__ __forceinline__ void mrr_last_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
-{
-    extern __shared__ __align__(16) u64 smem[];
-    const u32 tid = threadIdx.x;
-    const u32 n = a.n, l = n - 1;
-    const u32 c = item / 2, k = item % 2;
-    const PrimeConst pc = a.ctx.pc[l];
-    const PrimeConst pP = a.ctx.pc[a.ctx.n_data];
-    const u64 *cst = a.ctx.cst + 3 * l;
-    const u64 half_P = (pP.p - 1) / 2;
-    const u64 *y = a.plift + ((size_t)c * 2 + k) * Sh::N;
-    u64 x[Sh::E];
-    auto ld = [&](u32 P) -> u64 { return centred_mod(rd(y + P), half_P, cst[2], pc); };
-    auto nost = [&](u32, u64) {};
-    ntt_fwd_block<Sh, false>(smem, m, rbase, a.ctx.tw_fwd + (size_t)l * Sh::N, pc, ld, nost, x);
-    const u64 *accp = a.accq + (((size_t)c * 2 + k) * n + l) * Sh::N;
-    sub_scale_run<Sh>(x, accp, cst[0], cst[1], pc, m, tid);   // acc holds d P
-    u64 *dst = a.lift2 + ((size_t)c * 2 + k) * Sh::N;
-    auto st = [&](u32 P, u64 v) {
-        if (valid) dst[P] = v;
-    };
-    auto nold = [&](u32) -> u64 { return 0; };
-    ntt_inv_block<Sh, true>(smem, m, rbase, a.ctx.tw_inv + (size_t)l * Sh::N, pc, nold, st, x);
-}
+// MulLinRS after the mod-up: mod-down by P and rescale by q_l. The transform
+// is linear, so both divisions of limb i < l share one:
+//   out_i = ((acc_i - NTT_i(r_P)) P^-1 - NTT_i(r_l)) q_l^-1
+//         = (acc_i - NTT_i(r_P + P r_l)) (P q_l)^-1      (mod q_i)
+// with acc the stored d P + acc, r_P the centred residue of y_P = INTT_P(acc)
+// and r_l that of the relinearised limb q_l, which is needed in the
+// coefficient domain only:
+//   y_l = INTT_l((acc_l - NTT_l(r_P)) P^-1) = INTT_l(acc_l) P^-1 - r_P P^-1.
+// So limb q_l takes one inverse transform like the special prime (both in
+// k_mrr_lift; P^-1 is folded into its N^-1 constants), and the 2 (n - 1)
+// forward transforms of k_mrr_rest form r_P + P r_l on their loads. Against
+// a forward and an inverse transform for limb q_l and two forward transforms
+// for every other limb this leaves 2 + 2 + 2 (n - 1) transforms of
+// 2 + 4 + 4 (n - 1). The outputs are canonical, so they are the same words.
+// Measured (one context with 7 + 1 primes at N = 2^14, level 6): 64 pairs
+// 1157 -> 1005 us, one pair 104 -> 75 us.
 
-template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
-__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
-k_mrr_last(EvalArgs a0, JobsArg<JOBS> tab)
-{
-    EvalArgs a = a0;
-    using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
-    const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
-    u32 item = blockIdx.x >> LOG_C;
-    if constexpr (JOBS) item = bind_job(a, tab, JS_LAST, item);
-    mrr_last_body<Sh>(a, item, m, 0, true);
-}
+// r_P + P r_l mod q_i as a transform input below 7 q_i, from y_P and
+// a_l = INTT_l(acc_l) P^-1 (both canonical): with b_P, b_l the flags of the
+// residues above half,
+//   y_l = a_l - y_P P^-1 + b_P (mod q_l),
+//   r_P + P r_l = y_P + P (y_l - b_P) - b_l P q_l.
+struct RestLift {
+    u64 half_P, half_l, ql;
+    u64 Pinv_l, Pinv_l_sh;   // P^-1 mod q_l
+    u64 P_i, P_i_sh;         // P mod q_i
+    u64 minus_Pql;           // q_i - (P q_l mod q_i)
+    __device__ __forceinline__ u64 operator()(u64 yP, u64 al, const PrimeConst &pc) const
+    {
+        const u64 bP = yP > half_P ? 1u : 0u;
+        const u64 yl = reduce_once(sub_mod(al, mul_shoup(yP, Pinv_l, Pinv_l_sh, ql), ql) + bP, ql);
+        const u64 t0 = reduce_once(reduce_word(yP, pc), pc.two_p);                      // below 2 q_i
+        const u64 t1 = mul_shoup_lazy4_asm(yl + pc.p - bP, P_i, P_i_sh, pc.neg_p);      // below 4 q_i
+        return t0 + t1 + (yl > half_l ? minus_Pql : 0);
+    }
+};
 
-// MulLinRS, limbs i < l: mod-down by P, then rescale by q_l, as two launches
-// of one transform each (plain transform size and register budget; one
-// fused kernel holding the first result across the second transform needs
-// twice the registers):
-//   k_mrr_rest_z:   z_k[i] = d_k[i] + (acc_k[i] - NTT_i([y_k]_P)) P^-1
-//                          = (stored acc - NTT_i([y_k]_P)) P^-1 (the mod-up
-//                   stores d_k P + acc_k), written over the accumulator (each
-//                   thread rewrites only the positions it read);
-//   k_mrr_rest_out: out[c][k][i] = (z_k[i] - NTT_i([y2_k]_{q_l})) q_l^-1.
-// Both transforms are left lazy (their outputs only enter Shoup products).
 // item = 2 l c + l k + i (ciphertext c, component k, limb i < l).
 template <class Sh>
-__device__ __forceinline__ void mrr_rest_z_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
+__device__ __forceinline__ void mrr_rest_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
 {
     extern __shared__ __align__(16) u64 smem[];
     const u32 tid = threadIdx.x;
-    const u32 n = a.n, l = n - 1;
+    const u32 n = a.n, l = n - 1, nd = a.ctx.n_data;
     const u32 c = item / (2 * l), k = (item / l) % 2, i = item % l;
     const PrimeConst pc = a.ctx.pc[i];
-    const u64 *cP = a.ctx.cst + 3 * i;
-    const u64 half_P = (a.ctx.pc[a.ctx.n_data].p - 1) / 2;
-    const u64 P_mod_q = cP[2];
-    const u64 *y = a.plift + ((size_t)c * 2 + k) * Sh::N;
+    const u64 *cPl = a.ctx.cst + rest_index(a.ctx, l, i);   // (P q_l)^-1, its Shoup quotient, -P q_l (mod q_i)
+    RestLift lift;
+    lift.half_P = (a.ctx.pc[nd].p - 1) / 2;
+    lift.ql = a.ctx.pc[l].p;
+    lift.half_l = (lift.ql - 1) / 2;
+    lift.Pinv_l = a.ctx.cst[3 * l];
+    lift.Pinv_l_sh = a.ctx.cst[3 * l + 1];
+    lift.P_i = a.ctx.cst[3 * i + 2];
+    lift.P_i_sh = a.ctx.cst[p_shoup_index(a.ctx, i)];
+    lift.minus_Pql = cPl[2];
+    const u64 *yP = a.plift + ((size_t)c * 2 + k) * Sh::N;
+    const u64 *al = a.lift2 + ((size_t)c * 2 + k) * Sh::N;
     u64 x[Sh::E];
     auto nost = [&](u32, u64) {};
-    auto ld = [&](int P) -> u64 { return centred_mod(rd(y + P), half_P, P_mod_q, pc); };
+    auto ld = [&](int P) -> u64 { return lift(rd(yP + P), rd(al + P), pc); };
     ntt_fwd_block<Sh, false>(smem, m, rbase, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, nost, x);
-    u64 *accp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
-    sub_scale_run<Sh>(x, accp, cP[0], cP[1], pc, m, tid);
-    if (valid) store_run<Sh>(accp, x, m, tid);
-}
-
-template <class Sh>
-__device__ __forceinline__ void mrr_rest_out_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
-{
-    extern __shared__ __align__(16) u64 smem[];
-    const u32 tid = threadIdx.x;
-    const u32 n = a.n, l = n - 1;
-    const u32 c = item / (2 * l), k = (item / l) % 2, i = item % l;
-    const PrimeConst pc = a.ctx.pc[i];
-    const u64 *cl = a.ctx.cst + 3 * a.ctx.n_data + 3 * ((size_t)l * a.ctx.n_data + i);
-    const u64 half_l = (a.ctx.pc[l].p - 1) / 2;
-    const u64 ql_mod_q = cl[2];
-    const u64 *y2 = a.lift2 + ((size_t)c * 2 + k) * Sh::N;
-    u64 x[Sh::E];
-    auto nost = [&](u32, u64) {};
-    auto ld = [&](int P) -> u64 { return centred_mod(rd(y2 + P), half_l, ql_mod_q, pc); };
-    ntt_fwd_block<Sh, false>(smem, m, rbase, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, nost, x);
-    const u64 *zp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
+    const u64 *accp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
     u64 *out = a.out + (((size_t)c * 2 + k) * l + i) * Sh::N;
-    sub_scale_run<Sh>(x, zp, cl[0], cl[1], pc, m, tid);
+    sub_scale_run<Sh>(x, accp, cPl[0], cPl[1], pc, m, tid);
     if (valid) store_run<Sh>(out, x, m, tid);
 }
 
-// Inverse transform of one special-prime accumulator row of plift in place
-// (row = 2 c + k; inputs in [0, 4P), the key multiply-accumulate's range).
-// Every load precedes the cluster barrier before the cross-CTA stages (or,
-// in one CTA, the barrier of the first round exchange) and every store
-// follows it, so the rows can be transformed in place.
+// Inverse transforms before the rest: items below 2 count take accq's limb l
+// of row item = 2 c + k to lift2, times P^-1 (the lift constants); the next
+// 2 count take the special-prime rows of plift in place (inputs in [0, 4P),
+// the key multiply-accumulate's range; not launched after the fused mod-up,
+// which leaves them transformed). Every load precedes the cluster barrier
+// before the cross-CTA stages (or, in one CTA, the barrier of the first
+// round exchange) and every store follows it, so a row can be transformed in
+// place.
 template <class Sh>
-__device__ __forceinline__ void plift_intt_body(const EvalArgs &a, u32 row, u32 m, u32 rbase, bool valid)
+__device__ __forceinline__ void mrr_lift_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
 {
     extern __shared__ __align__(16) u64 smem[];
-    const u32 tp = a.ctx.n_data;
-    u64 *y = a.plift + (size_t)row * Sh::N;
+    const u32 n = a.n, l = n - 1;
+    const bool special = item >= 2 * a.count;
+    const u32 row = special ? item - 2 * a.count : item;
+    const u32 pr = special ? a.ctx.n_data : l;
+    const PrimeConst pc = a.ctx.pc_lift[pr];
+    const u64 *src = special ? a.plift + (size_t)row * Sh::N : a.accq + ((size_t)row * n + l) * Sh::N;
+    u64 *dst = (special ? a.plift : a.lift2) + (size_t)row * Sh::N;
+    const u32 tid = threadIdx.x;
     u64 x[Sh::E];
-    auto ld = [&](u32 P) -> u64 { return rd(y + P); };
+#pragma unroll
+    for (int e = 0; e < Sh::E; e += 4) ld4(src + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+    auto nold = [&](u32) -> u64 { return 0; };
     auto st = [&](u32 P, u64 v) {
-        if (valid) y[P] = v;
+        if (valid) dst[P] = v;
     };
-    ntt_inv_block<Sh, false>(smem, m, rbase, a.ctx.tw_inv + (size_t)tp * Sh::N, a.ctx.pc[tp], ld, st, x);
+    ntt_inv_block<Sh, true>(smem, m, rbase, a.ctx.tw_inv + (size_t)pr * Sh::N, pc, nold, st, x);
 }
 
 template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
-k_mrr_rest_z(EvalArgs a0, JobsArg<JOBS> tab)
+k_mrr_lift(EvalArgs a0, JobsArg<JOBS> tab)
+{
+    EvalArgs a = a0;
+    using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
+    const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
+    u32 item = blockIdx.x >> LOG_C;
+    if constexpr (JOBS) item = bind_job(a, tab, JS_LIFT, item);
+    mrr_lift_body<Sh>(a, item, m, 0, true);
+}
+
+template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
+k_mrr_rest(EvalArgs a0, JobsArg<JOBS> tab)
 {
     EvalArgs a = a0;
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
     u32 item = blockIdx.x >> LOG_C;
     if constexpr (JOBS) item = bind_job(a, tab, JS_REST, item);
-    mrr_rest_z_body<Sh>(a, item, m, 0, true);
-}
-
-template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
-__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
-k_mrr_rest_out(EvalArgs a0, JobsArg<JOBS> tab)
-{
-    EvalArgs a = a0;
-    using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
-    const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
-    u32 item = blockIdx.x >> LOG_C;
-    if constexpr (JOBS) item = bind_job(a, tab, JS_REST, item);
-    mrr_rest_out_body<Sh>(a, item, m, 0, true);
+    mrr_rest_body<Sh>(a, item, m, 0, true);
 }
 
 }  // namespace he

@@ -73,16 +73,24 @@ struct DevCtx {
     const ulonglong2 *tw_fwd;   // [n_data + 1][N]
     const ulonglong2 *tw_inv;
     const PrimeConst *pc;       // [n_data + 1]
+    const PrimeConst *pc_lift;  // pc, the data primes' last inverse stage also multiplying by P^-1
     // cst[3 i + {0,1,2}] = P^-1 mod q_i, its Shoup quotient, P mod q_i;
     // cst[3 n_data + 3 (l n_data + i) + {0,1,2}] = q_l^-1 mod q_i, Shoup,
     // q_l mod q_i (rescale from level l, i < l);
-    // cst[3 n_data + 3 n_data^2 + i] = Shoup quotient of P mod q_i.
+    // cst[3 n_data + 3 n_data^2 + i] = Shoup quotient of P mod q_i;
+    // cst[4 n_data + 3 n_data^2 + 3 (l n_data + i) + {0,1,2}] =
+    // (P q_l)^-1 mod q_i, its Shoup quotient, -P q_l mod q_i (i < l).
     const u64 *cst;
     u32 N;
     u32 n_data;
 };
 
 __host__ __device__ inline u32 p_shoup_index(const DevCtx &c, u32 i) { return 3 * c.n_data * (1 + c.n_data) + i; }
+
+__host__ __device__ inline u32 rest_index(const DevCtx &c, u32 l, u32 i)
+{
+    return c.n_data * (4 + 3 * c.n_data) + 3 * (l * c.n_data + i);
+}
 
 struct EvalArgs {
     const u64 *ct_a, *ct_b;     // [count][2][n][N] (fused Mul) or null
@@ -106,9 +114,8 @@ struct EvalArgs {
 // covers every job; job i's items in stage S start at job[i].begin[S].
 // Multi-degree batches (a context and key per job, degrees 2^12 .. 2^15):
 // the transform stages count units (clusters of 8 CTAs, each running 8 >> c
-// items of degree 2^(12 + c) side by side) instead of items, and the special
-// prime's inverse transforms are a stage of their own (JS_PLIFT).
-enum JobStage { JS_DIGITS = 0, JS_EXPAND, JS_MAC, JS_LAST, JS_REST, JS_PLIFT, JS_COUNT };
+// items of degree 2^(12 + c) side by side) instead of items.
+enum JobStage { JS_DIGITS = 0, JS_EXPAND, JS_MAC, JS_LIFT, JS_REST, JS_COUNT };
 constexpr u32 kMaxJobs = 16;
 struct EvalJob {
     const u64 *ct_a, *ct_b;     // [count][2][n][N]
@@ -129,8 +136,8 @@ using JobsArg = typename std::conditional<JOBS, JobTable, NoJobs>::type;
 
 // Stages of the multi-degree MulLinRS pipeline (multi.cu), one launch each
 // over `units` clusters; the key multiply-accumulate between the expansion
-// and the special-prime transforms is k_ks_mac over the same job table.
-enum MultiStage { MS_DIGITS = 0, MS_EXPAND, MS_PLIFT, MS_LAST, MS_REST_Z, MS_REST_OUT, MS_COUNT };
+// and the lifts is k_ks_mac over the same job table.
+enum MultiStage { MS_DIGITS = 0, MS_EXPAND, MS_LIFT, MS_REST, MS_COUNT };
 cudaError_t launch_mrr_multi(MultiStage stage, const EvalArgs &a, const JobTable &t, u32 units, cudaStream_t s);
 
 enum EvalKernel {
@@ -140,9 +147,8 @@ enum EvalKernel {
     EK_KS_MODDOWN,
     EK_RS_LIFT,
     EK_RS,
-    EK_MRR_LAST,
-    EK_MRR_REST_Z,
-    EK_MRR_REST_OUT,
+    EK_MRR_LIFT,
+    EK_MRR_REST,
     EK_COUNT
 };
 

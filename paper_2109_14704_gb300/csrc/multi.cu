@@ -25,8 +25,7 @@ __device__ __forceinline__ int multi_slot(MultiStage S)
     switch (S) {
     case MS_DIGITS: return JS_DIGITS;
     case MS_EXPAND: return JS_EXPAND;
-    case MS_PLIFT: return JS_PLIFT;
-    case MS_LAST: return JS_LAST;
+    case MS_LIFT: return JS_LIFT;
     default: return JS_REST;
     }
 }
@@ -37,7 +36,7 @@ __device__ __forceinline__ u32 multi_items(const EvalArgs &a)
 {
     if constexpr (S == MS_DIGITS) return a.count * a.n;
     if constexpr (S == MS_EXPAND) return a.count * a.n * a.n;   // off-diagonal (target, digit) pairs
-    if constexpr (S == MS_PLIFT || S == MS_LAST) return 2 * a.count;
+    if constexpr (S == MS_LIFT) return 4 * a.count;
     return 2 * a.count * (a.n - 1);
 }
 
@@ -63,21 +62,15 @@ __device__ __noinline__ void multi_item(const EvalArgs &a, u32 item, u32 m, u32 
             j = r - n * (n - 1);
         }
         ks_expand_body<Sh>(a, g, t, j, m, rbase, valid);
-    } else if constexpr (S == MS_PLIFT) {
-        plift_intt_body<Sh>(a, item, m, rbase, valid);
-    } else if constexpr (S == MS_LAST) {
-        mrr_last_body<Sh>(a, item, m, rbase, valid);
-    } else if constexpr (S == MS_REST_Z) {
-        mrr_rest_z_body<Sh>(a, item, m, rbase, valid);
+    } else if constexpr (S == MS_LIFT) {
+        mrr_lift_body<Sh>(a, item, m, rbase, valid);
     } else {
-        mrr_rest_out_body<Sh>(a, item, m, rbase, valid);
+        mrr_rest_body<Sh>(a, item, m, rbase, valid);
     }
 }
 
-// The forward-and-inverse stage keeps more state: the evaluation kernels'
-// 128-register budget (two CTAs per SM), the others the transform's 64.
 template <MultiStage S>
-__global__ void __launch_bounds__(256, S == MS_LAST ? 2 : 4) k_mrr_multi(EvalArgs a0, JobTable t)
+__global__ void __launch_bounds__(256, 4) k_mrr_multi(EvalArgs a0, JobTable t)
 {
     EvalArgs a = a0;
     const u32 rank = cluster_ctarank();
@@ -127,10 +120,8 @@ cudaError_t launch_mrr_multi(MultiStage stage, const EvalArgs &a, const JobTable
     switch (stage) {
     case MS_DIGITS: return launch_stage<MS_DIGITS>(a, t, units, s);
     case MS_EXPAND: return launch_stage<MS_EXPAND>(a, t, units, s);
-    case MS_PLIFT: return launch_stage<MS_PLIFT>(a, t, units, s);
-    case MS_LAST: return launch_stage<MS_LAST>(a, t, units, s);
-    case MS_REST_Z: return launch_stage<MS_REST_Z>(a, t, units, s);
-    case MS_REST_OUT: return launch_stage<MS_REST_OUT>(a, t, units, s);
+    case MS_LIFT: return launch_stage<MS_LIFT>(a, t, units, s);
+    case MS_REST: return launch_stage<MS_REST>(a, t, units, s);
     default: return cudaErrorInvalidValue;
     }
 }

@@ -155,3 +155,34 @@ def test_sign_tested_comparison():
     for x in vals:
         for m in (0, 1, x, (1 << 63) - 1, rnd.randrange(1 << 63)):
             assert reduce_once(x, m) == (x - m if x >= m else x)
+
+
+@pytest.mark.parametrize("P_bits,ql_bits,qi_bits", [(60, 60, 60), (60, 40, 31), (31, 60, 60), (31, 31, 60), (60, 31, 50)])
+def test_shared_division_input(P_bits, ql_bits, qi_bits):
+    """The rest stage's transform input: from y_P and a_l = [acc_l P^-1] it is
+    congruent to r_P + P r_l mod q_i (both residues centred, r_l that of
+    (acc_l - r_P) P^-1) and below 7 q_i, at the edges of every range."""
+    N = 1024
+    primes = []
+    for b in (P_bits, ql_bits, qi_bits):
+        primes.append(next(q for q in oracle.find_primes(b, 2 * N, 3) if q not in primes))
+    P, ql, qi = primes
+    half_P, half_l = (P - 1) // 2, (ql - 1) // 2
+    Pinv = pow(P, -1, ql)
+    r = random.Random(P_bits * 7 + ql_bits)
+    edges = lambda m: [0, 1, m // 2 - 1, m // 2, m // 2 + 1, m - 2, m - 1] + [r.randrange(m) for _ in range(40)]
+    for yP in edges(P):
+        for al in edges(ql):
+            bP = int(yP > half_P)
+            s = lazy4(yP, Pinv, shoup_pre(Pinv, ql), ql)          # the exact quotient gives [0, 2 q_l)
+            s = s % ql
+            yl = reduce_once(sub_mod(al, s, ql) + bP, ql)
+            t0 = reduce_once(lazy4(yP, 1, shoup_pre(1, qi), qi), 2 * qi)
+            Pi = P % qi
+            t1 = lazy4(yl + qi - bP, Pi, shoup_pre(Pi, qi), qi)
+            v = t0 + t1 + (qi - P * ql % qi if yl > half_l else 0)
+            rP = yP - P if yP > half_P else yP
+            want_l = (al - rP * Pinv) % ql
+            rl = want_l - ql if want_l > half_l else want_l
+            assert yl == want_l
+            assert v < 7 * qi and (v - (rP + P * rl)) % qi == 0
