@@ -192,6 +192,9 @@ static he::PrimeConst prime_const(u64 q, u32 N, u64 w1)
     c.w1ninv = h_mul(w1, c.ninv, q);
     c.w1ninv_sh = shoup(c.w1ninv, q);
     c.one_sh = shoup(1, q);
+    u64 inv = q;   // q^-1 mod 2^64 by Newton's iteration, 3 bits to start (q odd)
+    for (int i = 0; i < 5; i++) inv *= 2 - q * inv;
+    c.mneg = 0 - inv;
     return c;
 }
 
@@ -593,15 +596,35 @@ struct he_context {
     std::vector<u64> data;
     u64 P = 0;
     he_ntt_tables *tables = nullptr;   // primes q_0..q_L, P
-    u64 *d_cst = nullptr;
+    he::LimbConst *d_limb = nullptr;
+    he::DropConst *d_drop = nullptr;
     he::PrimeConst *d_pc_lift = nullptr;
+    u64 R_special = 0;                 // 2^64 mod P
     std::atomic<int> eval_log_e{4};    // words per thread of the evaluation kernels
 };
 
 struct he_relin_key {
     const he_context *ctx = nullptr;
-    ulonglong2 *d_evk = nullptr;
+    ulonglong2 *d_evk = nullptr;       // (word, Shoup quotient): the fused mod-up
+    u64 *d_mac = nullptr;              // the multiply-accumulate's words
 };
+
+template <class T>
+static cudaError_t upload(T **dst, const std::vector<T> &v)
+{
+    cudaError_t e = cudaMalloc(dst, std::max<size_t>(v.size(), 1) * sizeof(T));
+    if (e == cudaSuccess && !v.empty()) e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
+    return e;
+}
+
+static void free_context(he_context *c)
+{
+    he_ntt_tables_destroy(c->tables);
+    cudaFree(c->d_limb);
+    cudaFree(c->d_drop);
+    cudaFree(c->d_pc_lift);
+    delete c;
+}
 
 extern "C" he_status he_context_create(uint32_t N, uint32_t n_data, const uint64_t *data_moduli_host,
                                        uint64_t special_modulus, he_context **out)
@@ -632,47 +655,33 @@ extern "C" he_status he_context_create(uint32_t N, uint32_t n_data, const uint64
         delete c;
         return s;
     }
-    std::vector<u64> cst(4 * (size_t)n_data + 6 * (size_t)n_data * n_data, 0);
-    std::vector<he::PrimeConst> lift(n_data + 1);
+    std::vector<he::LimbConst> limb(n_data);
+    std::vector<he::DropConst> drop((size_t)n_data * n_data);
+    std::vector<he::PrimeConst> lift(c->tables->h_pc);   // the special prime's as it is
     for (u32 i = 0; i < n_data; i++) {
         const u64 q = all[i];
-        cst[3 * i + 0] = h_inv(special_modulus % q, q);
-        cst[3 * i + 1] = shoup(cst[3 * i + 0], q);
-        cst[3 * i + 2] = special_modulus % q;
-        cst[3 * (size_t)n_data * (1 + n_data) + i] = shoup(special_modulus % q, q);
-    }
-    for (u32 l = 1; l < n_data; l++)
-        for (u32 i = 0; i < l; i++) {
-            const u64 q = all[i], ql = all[l];
-            u64 *d = &cst[3 * n_data + 3 * ((size_t)l * n_data + i)];
-            d[0] = h_inv(ql % q, q);
-            d[1] = shoup(d[0], q);
-            d[2] = ql % q;
-            u64 *r = &cst[n_data * (4 + 3 * (size_t)n_data) + 3 * ((size_t)l * n_data + i)];
-            const u64 Pql = h_mul(special_modulus % q, ql % q, q);   // never 0: the primes differ
-            r[0] = h_inv(Pql, q);
-            r[1] = shoup(r[0], q);
-            r[2] = q - Pql;
+        he::LimbConst &k = limb[i];
+        auto put = [&](u64 v, u64 &w, u64 &w_sh) { w = v, w_sh = shoup(v, q); };
+        put(h_inv(special_modulus % q, q), k.Pinv, k.Pinv_sh);
+        put((u64)(((u128)1 << 64) % q), k.R, k.R_sh);
+        put(h_inv(k.R, q), k.k2, k.k2_sh);
+        put(h_mul(k.Pinv, k.k2, q), k.k1, k.k1_sh);
+        put(h_mul(lift[i].ninv, k.R, q), lift[i].ninv, lift[i].ninv_sh);
+        put(h_mul(lift[i].w1ninv, k.R, q), lift[i].w1ninv, lift[i].w1ninv_sh);
+        for (u32 l = i + 1; l < n_data; l++) {
+            he::DropConst &d = drop[(size_t)l * n_data + i];
+            d.ql = all[l] % q;
+            put(h_inv(d.ql, q), d.ql_inv, d.ql_inv_sh);
+            put(h_mul(k.R, d.ql_inv, q), d.R_ql_inv, d.R_ql_inv_sh);
+            d.minus_ql_k2 = q - h_mul(d.ql, k.k2, q);
         }
-    for (u32 i = 0; i <= n_data; i++) {
-        he::PrimeConst &k = lift[i];
-        k = c->tables->h_pc[i];
-        if (i == n_data) continue;
-        k.ninv = h_mul(k.ninv, cst[3 * i], k.p);
-        k.ninv_sh = shoup(k.ninv, k.p);
-        k.w1ninv = h_mul(k.w1ninv, cst[3 * i], k.p);
-        k.w1ninv_sh = shoup(k.w1ninv, k.p);
     }
-    cudaError_t e = cudaMalloc(&c->d_cst, cst.size() * sizeof(u64));
-    if (e == cudaSuccess) e = cudaMemcpy(c->d_cst, cst.data(), cst.size() * sizeof(u64), cudaMemcpyHostToDevice);
-    if (e == cudaSuccess) e = cudaMalloc(&c->d_pc_lift, lift.size() * sizeof(lift[0]));
-    if (e == cudaSuccess)
-        e = cudaMemcpy(c->d_pc_lift, lift.data(), lift.size() * sizeof(lift[0]), cudaMemcpyHostToDevice);
+    c->R_special = (u64)(((u128)1 << 64) % special_modulus);
+    cudaError_t e = upload(&c->d_limb, limb);
+    if (e == cudaSuccess) e = upload(&c->d_drop, drop);
+    if (e == cudaSuccess) e = upload(&c->d_pc_lift, lift);
     if (e != cudaSuccess) {
-        he_ntt_tables_destroy(c->tables);
-        cudaFree(c->d_cst);
-        cudaFree(c->d_pc_lift);
-        delete c;
+        free_context(c);
         return cuda_fail(e, "context constants");
     }
     *out = c;
@@ -692,10 +701,7 @@ extern "C" he_status he_context_destroy(he_context *ctx)
 {
     if (ctx) {
         cudaDeviceSynchronize();
-        he_ntt_tables_destroy(ctx->tables);
-        cudaFree(ctx->d_cst);
-        cudaFree(ctx->d_pc_lift);
-        delete ctx;
+        free_context(ctx);
     }
     return HE_OK;
 }
@@ -706,25 +712,34 @@ extern "C" he_status he_relin_key_upload(const he_context *ctx, const uint64_t *
     *out = nullptr;
     if (!ctx || !evk_host) return fail(HE_EINVAL, "context or key is NULL");
     const u32 nd = ctx->n_data, N = ctx->N;
-    const size_t words = (size_t)nd * 2 * (nd + 1) * N;
-    std::vector<ulonglong2> dev(words);
-    for (u32 j = 0; j < nd; j++)
-        for (u32 k = 0; k < 2; k++)
-            for (u32 t = 0; t <= nd; t++) {
-                const u64 q = ctx->tables->moduli[t];
-                const size_t base = (((size_t)j * 2 + k) * (nd + 1) + t) * N;
-                for (u32 i = 0; i < N; i++) {
-                    const u64 w = evk_host[base + i];
-                    if (w >= q) return fail(HE_EINVAL, "key word %zu is not reduced mod its prime", base + i);
-                    dev[base + i] = make_ulonglong2(w, shoup(w, q));
-                }
-            }
+    const size_t rows = (size_t)nd * 2 * (nd + 1), words = rows * N;
+    for (size_t r = 0; r < rows; r++) {
+        const u64 q = ctx->tables->moduli[r % (nd + 1)];
+        const u64 *w = evk_host + r * N;
+        bool ok = true;
+        for (u32 i = 0; i < N; i++) ok &= w[i] < q;
+        if (ok) continue;
+        u32 i = 0;
+        while (w[i] < q) i++;
+        return fail(HE_EINVAL, "key word %zu is not reduced mod its prime", r * N + i);
+    }
     he_relin_key *key = new he_relin_key;
     key->ctx = ctx;
+    u64 *raw = nullptr;
     cudaError_t e = cudaMalloc(&key->d_evk, words * sizeof(ulonglong2));
-    if (e == cudaSuccess) e = cudaMemcpy(key->d_evk, dev.data(), words * sizeof(ulonglong2), cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) e = cudaMalloc(&key->d_mac, words * 8);
+    if (e == cudaSuccess) e = cudaMalloc(&raw, words * 8);
+    if (e == cudaSuccess) e = cudaMemcpy(raw, evk_host, words * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess) {
+        he::k_key_prepare<<<stream_grid(words, 256), 256>>>(key->d_evk, key->d_mac, raw, words, (u32)ctx->log_n, nd,
+                                                            ctx->tables->d_pc, ctx->d_limb, ctx->R_special);
+        e = cudaGetLastError();
+        if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
+    }
+    cudaFree(raw);
     if (e != cudaSuccess) {
         cudaFree(key->d_evk);
+        cudaFree(key->d_mac);
         delete key;
         return fail(e == cudaErrorMemoryAllocation ? HE_ENOMEM : HE_ECUDA, "relin key upload: %s",
                     cudaGetErrorString(e));
@@ -738,6 +753,7 @@ extern "C" he_status he_relin_key_destroy(he_relin_key *key)
     if (key) {
         cudaDeviceSynchronize();
         cudaFree(key->d_evk);
+        cudaFree(key->d_mac);
         delete key;
     }
     return HE_OK;
@@ -750,7 +766,8 @@ static he::DevCtx dev_ctx(const he_context *c)
     d.tw_inv = c->tables->d_inv;
     d.pc = c->tables->d_pc;
     d.pc_lift = c->d_pc_lift;
-    d.cst = c->d_cst;
+    d.limb = c->d_limb;
+    d.drop = c->d_drop;
     d.N = c->N;
     d.n_data = c->n_data;
     return d;
@@ -841,6 +858,9 @@ static he_status plift_intt(const he_context *ctx, u64 *plift, u32 limbs, cudaSt
     return ntt_launch(L, ctx->log_n, true, s);
 }
 
+// CTAs of the per-tile key multiply-accumulate: one a tile up to 16 an SM
+static u32 mac_grid(u64 tiles) { return (u32)std::max<u64>(1, std::min<u64>(tiles, (u64)num_sms() * 16)); }
+
 // Mod-up of key switching for `count` ciphertexts (a.c2 holds their
 // coefficient-domain digits): accq and plift as k_ks_modup leaves them.
 // With room for the expanded buffer (x_words at xbuf, at least one
@@ -850,19 +870,6 @@ static he_status plift_intt(const he_context *ctx, u64 *plift, u32 limbs, cudaSt
 // the special prime's accumulators in plift are left in the NTT domain
 // (*special_ntt = true). Otherwise the fused k_ks_modup runs, which also takes
 // them through the inverse transform.
-// The tiled key multiply-accumulate's shared memory, 2 n MAC_TILE key pairs
-// (64 KB at the largest chain, n = 32), above the default 48 KB limit.
-static cudaError_t mac_tiled_smem_attr()
-{
-    static std::once_flag once;
-    static cudaError_t e = cudaSuccess;
-    std::call_once(once, [] {
-        e = cudaFuncSetAttribute(he::k_ks_mac_tiled, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                 (int)(2 * 32 * he::MAC_TILE * sizeof(ulonglong2)));
-    });
-    return e;
-}
-
 static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64 *xbuf, size_t x_words,
                           bool *special_ntt, cudaStream_t s)
 {
@@ -876,14 +883,13 @@ static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64
         const u32 gs = std::min(group, count - c0);
         a.c_first = c0;
         if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, gs * (n + 1) * n, s)) return r;
-        if (gs >= 8) {   // every ciphertext lane of the tiled kernel busy
+        if (gs >= 8) {   // a warp per ciphertext: all of them busy
             const u32 blocks = (n + 1) * (ctx->N / he::MAC_TILE) * ((gs + he::MAC_CHUNK - 1) / he::MAC_CHUNK);
-            const u32 smem = n * 2 * he::MAC_TILE * (u32)sizeof(ulonglong2);
-            if (cudaError_t e = mac_tiled_smem_attr()) return cuda_fail(e, "k_ks_mac_tiled attribute");
+            const u32 smem = n * 2 * he::MAC_TILE * 8;   // 32 KB at the longest chain
             he::k_ks_mac_tiled<<<blocks, 256, smem, s>>>(a, gs);
         } else {
-            const u32 total = (u32)((gs + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (ctx->N / 2));
-            he::k_ks_mac<false><<<stream_grid(total, 256), 256, 0, s>>>(a, gs, total, he::NoJobs{});
+            const u32 tiles = gs * (n + 1) * (ctx->N / he::MAC_BLOCK);
+            he::k_ks_mac<false><<<mac_grid(tiles), he::MAC_BLOCK / 2, 0, s>>>(a, gs, tiles, he::NoJobs{});
         }
         HE_CUDA(cudaGetLastError());
     }
@@ -910,6 +916,7 @@ extern "C" he_status he_relin(uint64_t *ct_out2, const uint64_t *ct_in3, const h
     a.accq = a.c2 + (size_t)n * ctx->N;
     a.plift = a.accq + (size_t)2 * n * ctx->N;
     a.evk = key->d_evk;
+    a.evk_mac = key->d_mac;
     a.n = n;
     a.count = 1;
     a.ctx = dev_ctx(ctx);
@@ -977,6 +984,7 @@ static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const
     a.plift = a.accq + (size_t)count * 2 * n * ctx->N;
     a.lift2 = rescale ? a.plift + (size_t)count * 2 * ctx->N : nullptr;
     a.evk = key->d_evk;
+    a.evk_mac = key->d_mac;
     a.n = n;
     a.count = count;
     a.ctx = dev_ctx(ctx);
@@ -1082,10 +1090,10 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
         w = E.mx + (size_t)c * (n + 1) * n * ctx->N;
         E.plift = pl;
         pl += (size_t)c * 2 * ctx->N;
-        E.evk = key->d_evk;
+        E.evk_mac = key->d_mac;
         E.ctx = dev_ctx(ctx);
         const u64 items[he::JS_COUNT] = {(u64)c * n, (u64)c * (n + 1) * n,
-                                         (u64)(c + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (ctx->N / 2), 4ull * c,
+                                         (u64)c * (n + 1) * (ctx->N / he::MAC_BLOCK), 4ull * c,
                                          2ull * c * (n - 1)};
         for (int st = 0; st < he::JS_COUNT; st++) {
             if (tot[st] + items[st] > 0x7fffffffull) return fail(HE_EINVAL, "batch too large");
@@ -1097,12 +1105,11 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
     for (int st = 0; st < he::JS_COUNT; st++) grid_items = std::max<u64>(grid_items, tot[st]);
     if (grid_items * 8 > 0x7fffffffull) return fail(HE_EINVAL, "batch too large");
     he::EvalArgs a = {};
-    a.evk = key->d_evk;
     a.ctx = dev_ctx(ctx);
     a.n = t.job[0].n;   // unused with a job table; kept valid
     if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, (u32)tot[he::JS_DIGITS], s, &t)) return r;
     if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, (u32)tot[he::JS_EXPAND], s, &t)) return r;
-    he::k_ks_mac<true><<<stream_grid(tot[he::JS_MAC], 256), 256, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
+    he::k_ks_mac<true><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
     if (he_status r = run_eval(ctx, he::EK_MRR_LIFT, a, (u32)tot[he::JS_LIFT], s, &t)) return r;
     return run_eval(ctx, he::EK_MRR_REST, a, (u32)tot[he::JS_REST], s, &t);
@@ -1678,14 +1685,6 @@ extern "C" he_status he_plan_destroy(he_plan *plan)
     return HE_OK;
 }
 
-template <class T>
-static cudaError_t upload(T **dst, const std::vector<T> &v)
-{
-    cudaError_t e = cudaMalloc(dst, std::max<size_t>(v.size(), 1) * sizeof(T));
-    if (e == cudaSuccess && !v.empty()) e = cudaMemcpy(*dst, v.data(), v.size() * sizeof(T), cudaMemcpyHostToDevice);
-    return e;
-}
-
 extern "C" he_status he_ntt_plan_create(const he_poly_desc *descs_host, uint32_t count,
                                         const he_ntt_shape *shapes_host, uint32_t n_shapes, he_plan **out)
 {
@@ -1974,7 +1973,7 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
         E.out = J.ct_out;
         E.n = n;
         E.count = c;
-        E.evk = J.key->d_evk;
+        E.evk_mac = J.key->d_mac;
         E.ctx = dev_ctx(ctx);
         E.c2 = w;
         E.accq = E.c2 + (size_t)c * n * N;
@@ -1987,7 +1986,7 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
         u64 cnt[he::JS_COUNT] = {};
         cnt[he::JS_DIGITS] = units((u64)c * n);
         cnt[he::JS_EXPAND] = units((u64)c * n * n);
-        cnt[he::JS_MAC] = (u64)(c + he::MAC_CTS - 1) / he::MAC_CTS * (n + 1) * (N / 2);
+        cnt[he::JS_MAC] = (u64)c * (n + 1) * (N / he::MAC_BLOCK);
         cnt[he::JS_LIFT] = units(4ull * c);
         cnt[he::JS_REST] = units(2ull * c * (n - 1));
         for (int st = 0; st < he::JS_COUNT; st++) {
@@ -1997,12 +1996,12 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
         }
     }
     he::EvalArgs a = {};
-    a.evk = t.job[0].evk;   // every stage binds its job's own context and key
+    a.evk_mac = t.job[0].evk_mac;   // every stage binds its job's own context and key
     a.ctx = t.job[0].ctx;
     a.n = t.job[0].n;
     HE_CUDA(he::launch_mrr_multi(he::MS_DIGITS, a, t, (u32)tot[he::JS_DIGITS], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_EXPAND, a, t, (u32)tot[he::JS_EXPAND], s));
-    he::k_ks_mac<true><<<stream_grid(tot[he::JS_MAC], 256), 256, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
+    he::k_ks_mac<true><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
     HE_CUDA(he::launch_mrr_multi(he::MS_LIFT, a, t, (u32)tot[he::JS_LIFT], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_REST, a, t, (u32)tot[he::JS_REST], s));

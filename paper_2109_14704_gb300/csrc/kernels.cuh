@@ -621,10 +621,10 @@ __global__ void k_enc_combine(u64 *ct, const u64 *noise, const u64 *pt, const u6
 //                 (for t = q_j the NTT-domain c[2]_j is used as is); on P the
 //                 accumulators are brought back by INTT_P and kept as the
 //                 coefficient-domain residues y_k = [x_k]_P          (2 INTT);
-//                 on the data primes the stored accumulator already holds
-//                 d_k P + acc_k, so that the mod-down needs no d_k:
+//                 on the data primes the stored accumulator is already
+//                 (acc_k P^-1 + d_k) 2^-64, so that the mod-down needs no d_k:
 //   k_ks_moddown  out_k[i] = d_k[i] + (acc_k[q_i] - NTT(r_k mod q_i)) P^-1
-//                          = (stored acc - NTT(r_k mod q_i)) P^-1,
+//                          = (stored acc - NTT(r_k P^-1 2^-64 mod q_i)) 2^64,
 //                 r_k the centred lift of y_k                        (2n NTT)
 // RS (Sec. II-A): k_rs_lift brings c_k[q_l] to the coefficient domain
 // (2 INTT), k_rs combines (c_k[q_i] - NTT(r mod q_i)) q_l^-1 (2(n-1) NTT).
@@ -697,7 +697,7 @@ __device__ __forceinline__ u32 bind_job(EvalArgs &a, const JobTable &t, int S, u
     a.plift = J.plift;
     a.lift2 = J.lift2;
     a.mx = J.mx;
-    a.evk = J.evk;
+    a.evk_mac = J.evk_mac;
     a.ctx = J.ctx;
     a.n = J.n;
     a.count = J.count;
@@ -715,52 +715,6 @@ struct DSource {
         if (k == 0) return mul_mod(rd(ct_a + off), rd(ct_b + off), pc);
         if (k == 1) return mad2_mod(rd(ct_a + off), rd(ct_b + per + off), rd(ct_a + per + off), rd(ct_b + off), pc);
         return mul_mod(rd(ct_a + per + off), rd(ct_b + per + off), pc);
-    }
-    // d_k at the two positions P, P + 1 (P even), from 16-byte loads.
-    __device__ __forceinline__ ulonglong2 d2(int k, u32 limb, u32 log_n, u32 P, const PrimeConst &pc) const
-    {
-        const size_t off = ((size_t)limb << log_n) + P;
-        auto ld = [](const u64 *q) { return __ldg(reinterpret_cast<const ulonglong2 *>(q)); };
-        if (ct3) return ld(ct3 + k * per + off);
-        ulonglong2 r;
-        if (k == 1) {
-            const ulonglong2 a0 = ld(ct_a + off), a1 = ld(ct_a + per + off);
-            const ulonglong2 b0 = ld(ct_b + off), b1 = ld(ct_b + per + off);
-            r.x = mad2_mod(a0.x, b1.x, a1.x, b0.x, pc);
-            r.y = mad2_mod(a0.y, b1.y, a1.y, b0.y, pc);
-            return r;
-        }
-        const size_t o = (k == 0) ? off : per + off;
-        const ulonglong2 a = ld(ct_a + o), b = ld(ct_b + o);
-        r.x = mul_mod(a.x, b.x, pc);
-        r.y = mul_mod(a.y, b.y, pc);
-        return r;
-    }
-    // d_k at the four positions P .. P + 3 (P = 0 mod 4) into r[0..3], from
-    // 32-byte loads.
-    __device__ __forceinline__ void d4(int k, u32 limb, u32 log_n, u32 P, const PrimeConst &pc, u64 *r) const
-    {
-        const size_t off = ((size_t)limb << log_n) + P;
-        if (ct3) {
-            ld4_nc(ct3 + k * per + off, r[0], r[1], r[2], r[3]);
-            return;
-        }
-        u64 a[4], b[4];
-        if (k == 1) {
-            u64 a1[4], b1[4];
-            ld4_nc(ct_a + off, a[0], a[1], a[2], a[3]);
-            ld4_nc(ct_b + per + off, b1[0], b1[1], b1[2], b1[3]);
-            ld4_nc(ct_a + per + off, a1[0], a1[1], a1[2], a1[3]);
-            ld4_nc(ct_b + off, b[0], b[1], b[2], b[3]);
-#pragma unroll
-            for (int i = 0; i < 4; i++) r[i] = mad2_mod(a[i], b1[i], a1[i], b[i], pc);
-            return;
-        }
-        const size_t o = (k == 0) ? off : per + off;
-        ld4_nc(ct_a + o, a[0], a[1], a[2], a[3]);
-        ld4_nc(ct_b + o, b[0], b[1], b[2], b[3]);
-#pragma unroll
-        for (int i = 0; i < 4; i++) r[i] = mul_mod(a[i], b[i], pc);
     }
 };
 
@@ -787,14 +741,30 @@ __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 
 {
     extern __shared__ __align__(16) u64 smem[];
     const u32 c = item / a.n, j = item % a.n;
-    const PrimeConst pc = a.ctx.pc[j];
     const DSource ds = dsource(a, c);
+    const PrimeConst pc = ds.ct3 ? a.ctx.pc[j] : a.ctx.pc_lift[j];
     u64 *out = a.c2 + ((size_t)c * a.n + j) * Sh::N;
     const u32 tid = threadIdx.x;
     u64 x[Sh::E];
-    // d2 at the thread's inverse-input positions (consecutive quarters)
+    // the thread's inverse-input positions (consecutive quarters): the given
+    // third component, or a1 b1 as Montgomery products, below 2 q_j and
+    // scaled by 2^-64, which the lift constants' last stage takes off
+    const size_t off = ds.per + (size_t)j * Sh::N;
+    if (ds.ct3) {
+        const u64 *d = ds.ct3 + ds.per + off;
 #pragma unroll
-    for (int e = 0; e < Sh::E; e += 4) ds.d4(2, j, Sh::LOG_N, (u32)last_pos<Sh>(m, tid, e), pc, x + e);
+        for (int e = 0; e < Sh::E; e += 4) ld4_nc(d + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+    } else {
+#pragma unroll
+        for (int e = 0; e < Sh::E; e += 4) {
+            const int P = last_pos<Sh>(m, tid, e);
+            u64 b[4];
+            ld4_nc(ds.ct_a + off + P, x[e], x[e + 1], x[e + 2], x[e + 3]);
+            ld4_nc(ds.ct_b + off + P, b[0], b[1], b[2], b[3]);
+#pragma unroll
+            for (int i = 0; i < 4; i++) x[e + i] = mul_mont(x[e + i], b[i], pc);
+        }
+    }
     auto nold = [&](u32) -> u64 { return 0; };
     auto st = [&](u32 P, u64 v) {
         if (valid) out[P] = v;
@@ -866,15 +836,17 @@ k_ks_modup(EvalArgs a)
         }
     }
     if (t < n) {
-        const u64 P_mod_q = a.ctx.cst[3 * t + 2], P_mod_q_sh = a.ctx.cst[p_shoup_index(a.ctx, t)];
+        // (acc_k P^-1 + d_k) 2^-64, below 4 q_t
+        const LimbConst lc = a.ctx.limb[t];
 #pragma unroll
         for (int k = 0; k < 2; k++) {
             u64 *dst = a.accq + (((size_t)c * 2 + k) * n + t) * Sh::N;
 #pragma unroll
             for (int e = 0; e < Sh::E; e++) {
                 const int P = last_pos<Sh>(m, tid, e);
-                const u64 s = reduce_once(reduce_once(acc[(k * Sh::E + e) * Sh::T + tid], pc.two_p), pc.p);
-                dst[P] = add_mod(s, mul_shoup(ds.d(k, t, Sh::LOG_N, (u32)P, pc), P_mod_q, P_mod_q_sh, pc.p), pc.p);
+                const u64 s = mul_shoup_lazy4_asm(acc[(k * Sh::E + e) * Sh::T + tid], lc.k1, lc.k1_sh, pc.neg_p);
+                const u64 d = mul_shoup_lazy4_asm(ds.d(k, t, Sh::LOG_N, (u32)P, pc), lc.k2, lc.k2_sh, pc.neg_p);
+                dst[P] = reduce_once(s + d, pc.four_p);
             }
         }
     } else {
@@ -899,7 +871,7 @@ k_ks_modup(EvalArgs a)
 // left in the lazy range [0, 12t) (it only feeds Shoup products). The same
 // transforms as k_ks_modup, but as independent launches of the plain
 // transform's size and register budget instead of a sequence inside one
-// accumulating cluster; k_ks_mac then accumulates them with the key.
+// accumulating cluster; k_ks_mac or k_ks_mac_tiled then accumulates them.
 // Clusters of the diagonal (j = t) exit at once: there the digit is already
 // in the NTT domain.
 // One transform of the expanded mod-up: X[g][t][j] = NTT_t(c2_j mod t),
@@ -947,99 +919,187 @@ k_ks_expand(EvalArgs a0, JobsArg<JOBS> tab)
 }
 
 #ifdef HE_MISC_KERNELS
-// Expanded mod-up, second half (elementwise):
-//   acc_k[t] = sum_j X[g][t][j] * evk[j][k][t]   (j = t: the NTT-domain
-//   digit d2_t itself), lazy products in [0, 4t), sums kept in [0, 4t);
-// d_k P + acc_k, canonical, into accq for data targets (as k_ks_modup),
-// acc_k left in [0, 4P) in plift for the special prime (the inverse
-// transform that follows accepts that range).
-// A thread takes two positions of one target for MAC_CTS ciphertexts of the
-// group, so each key word it loads serves MAC_CTS products; two ciphertexts
-// under a 64-register bound (four blocks of 256 per SM) measured fastest
-// (one: fewer key reuses; four: too few warps to cover the loads).
-constexpr u32 MAC_CTS = 2;
+// Expanded mod-up, second half (elementwise): for target t and component k
+//   acc_k = sum_j X[g][t][j] * evk[j][k][t]   (j = t: the NTT-domain digit
+// d2_t itself). The sums are 128-bit integers (Sum128) reduced once by
+// Montgomery's 2^-64, with the factors the division needs folded into the
+// uploaded key words: on the data primes P^-1, so that the tensor terms d_k
+// (products of two canonical words) join the same sum, giving
+// (acc_k P^-1 + d_k) 2^-64 in accq; on the special prime 2^64, giving acc_k in
+// plift. The diagonal digit enters as a Montgomery product, whose 2^-64 its
+// key words take off. All results in [0, 4 p).
+// Bounds: x is brought below 4 p + 2^32 <= 8 p (2^30 <= p < 2^60), so 32
+// digits and two tensor products sum to less than 2^128, and the reduced sum
+// is below 10 p.
 
-// One item of k_ks_mac: two positions of one target for up to MAC_CTS
-// ciphertexts of the group (item q of the group's chunks x targets x pairs).
-__device__ __forceinline__ void ks_mac_item(const EvalArgs &a, u32 groups, u32 q)
-{
-    const u32 n = a.n, N = a.ctx.N, nd1 = a.ctx.n_data + 1;
-    const u32 log_n = 31 - __clz(N);
-    const size_t key_j = (size_t)2 * nd1 * N, key_k = (size_t)nd1 * N;   // evk [j][k][target][N]
-    const size_t mx_g = (size_t)(n + 1) * n * N;                          // mx [g][target][j][N]
-    const u32 P = (q & ((N >> 1) - 1)) * 2;
-    const u32 r = q >> (log_n - 1);
-    const u32 t = r % (n + 1), g0 = (r / (n + 1)) * MAC_CTS;
-    const u32 ng = min(MAC_CTS, groups - g0);
-    const u32 tp = (t == n) ? a.ctx.n_data : t;
-    const PrimeConst pc = a.ctx.pc[tp];
-    const ulonglong2 *key = a.evk + (size_t)tp * N + P;                  // digit 0, k = 0
-    const u64 *mx = a.mx + ((size_t)g0 * (n + 1) + t) * n * N + P;      // ciphertext g0, digit 0
-    u64 acc[MAC_CTS][2][2];
-    for (u32 j = 0; j < n; j++, key += key_j, mx += N) {
-        ulonglong2 w[2][2];
-#pragma unroll
-        for (int k = 0; k < 2; k++) ld_tw2(key + k * key_k, 0, w[k][0], w[k][1]);   // positions P, P + 1
-#pragma unroll
-        for (u32 gi = 0; gi < MAC_CTS; gi++) {
-            if (gi >= ng) break;
-            ulonglong2 v;
-            if (j == t)
-                v = dsource(a, a.c_first + g0 + gi).d2(2, j, log_n, P, pc);
-            else
-                v = __ldg(reinterpret_cast<const ulonglong2 *>(mx + gi * mx_g));
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const u64 p0 = mul_shoup_lazy4_asm(v.x, w[k][0].x, w[k][0].y, pc.neg_p);
-                const u64 p1 = mul_shoup_lazy4_asm(v.y, w[k][1].x, w[k][1].y, pc.neg_p);
-                acc[gi][k][0] = j == 0 ? p0 : reduce_once(acc[gi][k][0] + p0, pc.four_p);
-                acc[gi][k][1] = j == 0 ? p1 : reduce_once(acc[gi][k][1] + p1, pc.four_p);
-            }
-        }
+// Words at two neighbouring positions.
+struct MacVec {
+    u64 v[2];
+    __device__ __forceinline__ static MacVec load(const u64 *p)
+    {
+        const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2 *>(p));
+        return {{t.x, t.y}};
     }
+    __device__ __forceinline__ static MacVec shared(const u64 *p)
+    {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+        return {{t.x, t.y}};
+    }
+    __device__ __forceinline__ void store(u64 *p) const
+    {
+        *reinterpret_cast<ulonglong2 *>(p) = make_ulonglong2(v[0], v[1]);
+    }
+};
+
+// The sums at positions P, P + 1 of one target for one ciphertext.
+struct MacSums {
+    using Vec = MacVec;
+    Sum128 s[2][2];   // [component][position]
+
+    __device__ __forceinline__ void add(const Vec &x, int k, const Vec &w)
+    {
 #pragma unroll
-    for (u32 gi = 0; gi < MAC_CTS; gi++) {
-        if (gi >= ng) break;
-        const u32 c = a.c_first + g0 + gi;
-        const DSource ds = dsource(a, c);
+        for (int i = 0; i < 2; i++) s[k][i].mac(x.v[i], w.v[i]);
+    }
+    // a transformed digit: the lazy output below 8 p + 2^32 to below 4 p + 2^32
+    __device__ __forceinline__ void digit(Vec x, const Vec &w0, const Vec &w1, const PrimeConst &pc)
+    {
+#pragma unroll
+        for (int i = 0; i < 2; i++)
+            if ((u32)(x.v[i] >> 32) >= pc.h4) x.v[i] -= pc.four_p;
+        add(x, 0, w0);
+        add(x, 1, w1);
+    }
+    // the tensor terms and the diagonal digit, whose key words are w0, w1
+    // (none on the special prime)
+    __device__ __forceinline__ void begin(const DSource &ds, u32 t, u32 n, u32 log_n, u32 P, const PrimeConst &pc,
+                                          const Vec &w0, const Vec &w1, const LimbConst *limb)
+    {
+#pragma unroll
+        for (int k = 0; k < 2; k++)
+#pragma unroll
+            for (int i = 0; i < 2; i++) s[k][i].clear();
+        if (t == n) return;
+        const size_t off = ((size_t)t << log_n) + P;
+        Vec d;
+        if (ds.ct3) {
+            const LimbConst &lc = limb[t];
+            d = Vec::load(ds.ct3 + 2 * ds.per + off);
+#pragma unroll
+            for (int i = 0; i < 2; i++) d.v[i] = mul_shoup_lazy4_asm(d.v[i], lc.k2, lc.k2_sh, pc.neg_p);
+        } else {
+            const Vec a0 = Vec::load(ds.ct_a + off), a1 = Vec::load(ds.ct_a + ds.per + off);
+            const Vec b0 = Vec::load(ds.ct_b + off), b1 = Vec::load(ds.ct_b + ds.per + off);
+            add(a0, 0, b0);
+            add(a0, 1, b1);
+            add(a1, 1, b0);
+#pragma unroll
+            for (int i = 0; i < 2; i++) d.v[i] = mul_mont(a1.v[i], b1.v[i], pc);
+        }
+        add(d, 0, w0);
+        add(d, 1, w1);
+    }
+    __device__ __forceinline__ void finish(const EvalArgs &a, const DSource &ds, u32 c, u32 t, u32 log_n, u32 P,
+                                           const PrimeConst &pc) const
+    {
+        const u32 n = a.n, N = a.ctx.N;
 #pragma unroll
         for (int k = 0; k < 2; k++) {
-            ulonglong2 o;
+            Vec o;
+#pragma unroll
+            for (int i = 0; i < 2; i++) o.v[i] = s[k][i].redc(pc);
+            u64 *dst;
             if (t < n) {
-                // stored as d_k P + acc_k (see the mod-down)
-                const u64 P_mod_q = a.ctx.cst[3 * t + 2], P_mod_q_sh = a.ctx.cst[p_shoup_index(a.ctx, t)];
-                const u64 s0 = reduce_once(reduce_once(acc[gi][k][0], pc.two_p), pc.p);
-                const u64 s1 = reduce_once(reduce_once(acc[gi][k][1], pc.two_p), pc.p);
-                const ulonglong2 dv = ds.d2(k, t, log_n, P, pc);
-                o.x = add_mod(s0, mul_shoup(dv.x, P_mod_q, P_mod_q_sh, pc.p), pc.p);
-                o.y = add_mod(s1, mul_shoup(dv.y, P_mod_q, P_mod_q_sh, pc.p), pc.p);
-                *reinterpret_cast<ulonglong2 *>(a.accq + (((size_t)c * 2 + k) * n + t) * N + P) = o;
+                if (ds.ct3) {
+                    const LimbConst &lc = a.ctx.limb[t];
+                    const Vec d = Vec::load(ds.ct3 + k * ds.per + ((size_t)t << log_n) + P);
+#pragma unroll
+                    for (int i = 0; i < 2; i++) o.v[i] += mul_shoup_lazy4_asm(d.v[i], lc.k2, lc.k2_sh, pc.neg_p);
+                }
+                dst = a.accq + (((size_t)c * 2 + k) * n + t) * N + P;
             } else {
-                o.x = acc[gi][k][0];
-                o.y = acc[gi][k][1];
-                *reinterpret_cast<ulonglong2 *>(a.plift + ((size_t)c * 2 + k) * N + P) = o;
+                dst = a.plift + ((size_t)c * 2 + k) * N + P;
             }
+#pragma unroll
+            for (int i = 0; i < 2; i++) o.v[i] = reduce_once(reduce_once(o.v[i], pc.four_p << 1), pc.four_p);
+            o.store(dst);
+        }
+    }
+};
+
+// One tile: MAC_BLOCK positions of one target for one ciphertext of the
+// group, two to a thread; the ciphertexts of a group are neighbouring
+// tiles, so that they find each other's key words in L2. The next digit's
+// words are loaded while the current products run.
+constexpr u32 MAC_BLOCK = 512;
+
+__device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 tile)
+{
+    using Vec = MacVec;
+    const u32 n = a.n, N = a.ctx.N, nd1 = a.ctx.n_data + 1;
+    const u32 log_n = 31 - __clz(N), per = N / MAC_BLOCK;
+    const u32 g = tile % groups, r = tile / groups;
+    const u32 P = (r % per) * MAC_BLOCK + threadIdx.x * 2, t = r / per;
+    const u32 tp = (t == n) ? a.ctx.n_data : t;
+    const PrimeConst pc = a.ctx.pc[tp];
+    const u32 c = a.c_first + g;
+    const DSource ds = dsource(a, c);
+    const size_t key_k = (size_t)nd1 * N, key_j = 2 * key_k;             // evk [j][k][target][N]
+    const u64 *key = a.evk_mac + (size_t)tp * N + P;
+    const u64 *mx = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;        // mx [g][target][j][N]
+    const u64 *kt = key + (t < n ? t : 0) * key_j;
+    MacSums acc;
+    acc.begin(ds, t, n, log_n, P, pc, Vec::load(kt), Vec::load(kt + key_k), a.ctx.limb);
+    // the digits j != t: n of them on the special prime, n - 1 otherwise
+    const u32 terms = t < n ? n - 1 : n;
+    u32 j = t == 0 ? 1u : 0u;
+    Vec v, w0, w1;
+    if (terms) v = Vec::load(mx + (size_t)j * N), w0 = Vec::load(key + j * key_j), w1 = Vec::load(key + j * key_j + key_k);
+    for (u32 i = 0; i < terms; i++) {
+        const Vec x = v, k0 = w0, k1 = w1;
+        if (i + 1 < terms) {
+            j += j + 1 == t ? 2u : 1u;
+            v = Vec::load(mx + (size_t)j * N), w0 = Vec::load(key + j * key_j), w1 = Vec::load(key + j * key_j + key_k);
+        }
+        acc.digit(x, k0, k1, pc);
+    }
+    acc.finish(a, ds, c, t, log_n, P, pc);
+}
+
+// Tiles of a uniform group (groups x (n + 1) targets x N / MAC_BLOCK), or
+// those of every job of a table back to back (each job one group of all its
+// ciphertexts).
+template <bool JOBS = false>
+__global__ void __launch_bounds__(MAC_BLOCK / 2, 4) k_ks_mac(EvalArgs a0, u32 groups, u32 total, JobsArg<JOBS> tab)
+{
+    for (u32 q = blockIdx.x; q < total; q += gridDim.x) {
+        if constexpr (JOBS) {
+            EvalArgs a = a0;
+            const u32 local = bind_job(a, tab, JS_MAC, q);
+            ks_mac_tile(a, a.count, local);
+        } else {
+            ks_mac_tile(a0, groups, q);
         }
     }
 }
 
-// Tiled form of the key multiply-accumulate for a uniform group of at
-// least 8 ciphertexts: one CTA per (target t, tile of MAC_TILE positions,
-// chunk of MAC_CHUNK ciphertexts). The tile's key pairs for every digit and
-// component are staged in shared memory once ([2 j + k][position], 2 n
-// MAC_TILE pairs) and serve every ciphertext of the chunk; each warp covers
-// 4 position pairs for 8 ciphertexts (its key reads are broadcasts), each
-// thread 2 positions of one ciphertext at a time, the next digit's values
-// loaded while the current ones' products run. With its few registers the
-// kernel runs six CTAs per SM: the per-thread form above is bound by the
-// latency of its loads at four (measured: the MulLinRS batch at N = 2^14,
-// 64 pairs, 1.203 -> 1.166 ms). Same products, same sums mod p: the outputs
-// are those of k_ks_mac.
+// Form for a uniform group of at least 8 ciphertexts: one CTA per (target t,
+// tile of MAC_TILE positions, chunk of MAC_CHUNK ciphertexts), a warp per
+// ciphertext at a time. The tile's key words for every digit and component
+// are staged in shared memory once ([2 j + k][position]) and serve every
+// ciphertext of the chunk. Same sums, so the outputs are those of k_ks_mac.
+// Bound by the multiply pipe (69 % busy) with HBM at 60 %: at N = 2^14, n = 7,
+// 64 ciphertexts (470 MB of digits, 780 MB in all) 257 us with a lazy Shoup
+// product per term and a separate d_k P, 183 us with the sums. Four CTAs an SM
+// (64 registers): three or five 5 to 6 % slower on the whole batch, one
+// position a thread at six 4 % slower, a shared-memory queue of asynchronous
+// copies 4 % slower (more instructions; the loads are not what it waits for).
 constexpr u32 MAC_TILE = 64, MAC_CHUNK = 32;
 
-__global__ void __launch_bounds__(256, 6) k_ks_mac_tiled(EvalArgs a, u32 groups)
+__global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
 {
-    extern __shared__ __align__(16) ulonglong2 key_tile[];   // [2 n][MAC_TILE]
+    using Vec = MacVec;
+    extern __shared__ __align__(16) u64 key_tile[];   // [2 n][MAC_TILE]
     const u32 n = a.n, N = a.ctx.N, nd1 = a.ctx.n_data + 1;
     const u32 tiles = N / MAC_TILE, chunks = (groups + MAC_CHUNK - 1) / MAC_CHUNK;
     const u32 b = blockIdx.x;
@@ -1047,80 +1107,78 @@ __global__ void __launch_bounds__(256, 6) k_ks_mac_tiled(EvalArgs a, u32 groups)
     const u32 tp = (t == n) ? a.ctx.n_data : t;
     const PrimeConst pc = a.ctx.pc[tp];
     const u32 P0 = tile * MAC_TILE;
-    for (u32 i = threadIdx.x; i < n * 2 * MAC_TILE; i += blockDim.x) {
+    for (u32 i = 2 * threadIdx.x; i < n * 2 * MAC_TILE; i += 2 * blockDim.x) {
         const u32 row = i / MAC_TILE, col = i % MAC_TILE;   // row 2 j + k: evk [j][k][target][N]
-        key_tile[i] = __ldg(a.evk + ((size_t)row * nd1 + tp) * N + P0 + col);
+        MacVec::load(a.evk_mac + ((size_t)row * nd1 + tp) * N + P0 + col).store(key_tile + i);
     }
     __syncthreads();
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const u32 pp = warp * 4 + (lane & 3);
-    const u32 P = P0 + 2 * pp;
+    const u32 P = P0 + 2 * lane;
     const u32 log_n = 31 - __clz(N);
     const u32 gend = min(groups, (chunk + 1) * MAC_CHUNK);
-    for (u32 g = chunk * MAC_CHUNK + (lane >> 2); g < gend; g += 8) {
-        const u64 *mxp = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;   // mx [g][target][j][N]
-        auto load_v = [&](u32 j) -> ulonglong2 {
-            if (j == t) return dsource(a, a.c_first + g).d2(2, j, log_n, P, pc);
-            return __ldg(reinterpret_cast<const ulonglong2 *>(mxp + (size_t)j * N));
-        };
-        u64 acc[2][2];
-        ulonglong2 vn = load_v(0);
-        for (u32 j = 0; j < n; j++) {
-            const ulonglong2 v = vn;
-            if (j + 1 < n) vn = load_v(j + 1);
-#pragma unroll
-            for (int k = 0; k < 2; k++) {
-                const ulonglong2 w0 = key_tile[(2 * j + k) * MAC_TILE + 2 * pp];
-                const ulonglong2 w1 = key_tile[(2 * j + k) * MAC_TILE + 2 * pp + 1];
-                const u64 p0 = mul_shoup_lazy4_asm(v.x, w0.x, w0.y, pc.neg_p);
-                const u64 p1 = mul_shoup_lazy4_asm(v.y, w1.x, w1.y, pc.neg_p);
-                acc[k][0] = j == 0 ? p0 : reduce_once(acc[k][0] + p0, pc.four_p);
-                acc[k][1] = j == 0 ? p1 : reduce_once(acc[k][1] + p1, pc.four_p);
-            }
-        }
+    const u64 *kl = key_tile + 2 * lane;
+    for (u32 g = chunk * MAC_CHUNK + warp; g < gend; g += 8) {
+        const u64 *mx = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;   // mx [g][target][j][N]
         const u32 c = a.c_first + g;
         const DSource ds = dsource(a, c);
-#pragma unroll
-        for (int k = 0; k < 2; k++) {
-            ulonglong2 o;
-            if (t < n) {
-                // stored as d_k P + acc_k (see the mod-down)
-                const u64 P_mod_q = a.ctx.cst[3 * t + 2], P_mod_q_sh = a.ctx.cst[p_shoup_index(a.ctx, t)];
-                const u64 s0 = reduce_once(reduce_once(acc[k][0], pc.two_p), pc.p);
-                const u64 s1 = reduce_once(reduce_once(acc[k][1], pc.two_p), pc.p);
-                const ulonglong2 dv = ds.d2(k, t, log_n, P, pc);
-                o.x = add_mod(s0, mul_shoup(dv.x, P_mod_q, P_mod_q_sh, pc.p), pc.p);
-                o.y = add_mod(s1, mul_shoup(dv.y, P_mod_q, P_mod_q_sh, pc.p), pc.p);
-                *reinterpret_cast<ulonglong2 *>(a.accq + (((size_t)c * 2 + k) * n + t) * N + P) = o;
-            } else {
-                o.x = acc[k][0];
-                o.y = acc[k][1];
-                *reinterpret_cast<ulonglong2 *>(a.plift + ((size_t)c * 2 + k) * N + P) = o;
+        const u32 terms = t < n ? n - 1 : n, jt = t < n ? t : 0;
+        u32 j = t == 0 ? 1u : 0u;
+        Vec v;
+        if (terms) v = Vec::load(mx + (size_t)j * N);
+        MacSums acc;
+        acc.begin(ds, t, n, log_n, P, pc, Vec::shared(kl + 2 * jt * MAC_TILE),
+                  Vec::shared(kl + (2 * jt + 1) * MAC_TILE), a.ctx.limb);
+        for (u32 i = 0; i < terms; i++) {
+            const Vec x = v;
+            const u64 *w = kl + 2 * j * MAC_TILE;
+            if (i + 1 < terms) {
+                j += j + 1 == t ? 2u : 1u;
+                v = Vec::load(mx + (size_t)j * N);
             }
+            acc.digit(x, Vec::shared(w), Vec::shared(w + MAC_TILE), pc);
         }
+        acc.finish(a, ds, c, t, log_n, P, pc);
     }
 }
 
-// Items: for a uniform group, (groups / MAC_CTS rounded up) x (n + 1)
-// targets x N / 2 position pairs; for a job table, those of every job back
-// to back (each job one group of all its ciphertexts). `total` is below 2^32
-// for every accepted size (64 ciphertexts per group, 33 targets, 2^15 pairs).
-template <bool JOBS = false>
-__global__ void __launch_bounds__(256, 4) k_ks_mac(EvalArgs a0, u32 groups, u32 total, JobsArg<JOBS> tab)
+// Device words of an uploaded key, [nd][2][nd + 1][N] canonical words raw:
+// evk = (word, Shoup quotient), evk_mac = the multiply-accumulate's word. The
+// quotient floor(w 2^64 / p) comes in two steps of 32 bits: with mu =
+// floor(2^(2b+2) / p) and r < p < 2^b, r mu / 2^(2b-30) is r 2^32 / p less
+// below one, so its floor is short by at most two.
+__device__ __forceinline__ u64 shoup_step(u64 &r, const PrimeConst &c)
 {
-    for (u32 q = blockIdx.x * blockDim.x + threadIdx.x; q < total; q += gridDim.x * blockDim.x) {
-        if constexpr (JOBS) {
-            EvalArgs a = a0;
-            const u32 local = bind_job(a, tab, JS_MAC, q);
-            ks_mac_item(a, a.count, local);
-        } else {
-            ks_mac_item(a0, groups, q);
-        }
+    u64 hi, lo;
+    mul_wide(r, c.mu, hi, lo);
+    const u32 s = 2 * c.bits - 30;               // 32 .. 90
+    u64 q = s < 64 ? (hi << (64 - s)) | (lo >> s) : hi >> (s - 64);
+    r = (r << 32) - q * c.p;                     // below 3 p
+    while (r >= c.p) r -= c.p, q++;
+    return q;
+}
+
+__global__ void k_key_prepare(ulonglong2 *evk, u64 *evk_mac, const u64 *raw, u64 words, u32 log_n, u32 nd,
+                              const PrimeConst *pcs, const LimbConst *limb, u64 R_special)
+{
+    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
+        const u32 t = (u32)((e >> log_n) % (nd + 1));
+        const PrimeConst pc = pcs[t];
+        const u64 w = raw[e];
+        u64 r = w;
+        const u64 qh = shoup_step(r, pc);
+        const u64 ql = shoup_step(r, pc);
+        evk[e] = make_ulonglong2(w, (qh << 32) + ql);
+        const u32 j = (u32)((e >> log_n) / (2 * (nd + 1)));
+        u64 f = R_special;
+        if (t < nd) f = j == t ? mul_mod(limb[t].Pinv, limb[t].R, pc) : limb[t].Pinv;
+        evk_mac[e] = mul_mod(w, f, pc);
     }
 }
 #endif  // HE_MISC_KERNELS
 
-// Relin mod-down (no rescale): out[c][k][i] = d_k[i] + (acc - NTT(r)) P^-1.
+// Relin mod-down (no rescale): out[c][k][i] = d_k[i] + (acc - NTT(r)) P^-1,
+// at the accumulator's scale: (stored acc - NTT(r P^-1 2^-64)) 2^64, with
+// r P^-1 = y P^-1 - 1 where y is above half.
 template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
 k_ks_moddown(EvalArgs a)
@@ -1134,16 +1192,19 @@ k_ks_moddown(EvalArgs a)
     const u32 c = item / (2 * n), k = (item / n) % 2, i = item % n;
     const PrimeConst pc = a.ctx.pc[i];
     const PrimeConst pP = a.ctx.pc[a.ctx.n_data];
-    const u64 *cst = a.ctx.cst + 3 * i;         // P^-1, Shoup, P mod q_i
-    const u64 half_P = (pP.p - 1) / 2;
+    const LimbConst lc = a.ctx.limb[i];
+    const u64 half_P = (pP.p - 1) / 2, minus_k2 = pc.p - lc.k2;
     const u64 *y = a.plift + ((size_t)c * 2 + k) * Sh::N;
     u64 x[Sh::E];
-    auto ld = [&](u32 P) -> u64 { return centred_mod(rd(y + P), half_P, cst[2], pc); };
+    auto ld = [&](u32 P) -> u64 {   // below 5 q_i
+        const u64 v = rd(y + P);
+        return mul_shoup_lazy4_asm(v, lc.k1, lc.k1_sh, pc.neg_p) + (v > half_P ? minus_k2 : 0);
+    };
     auto st = [&](u32, u64) {};
     ntt_fwd_block<Sh, false>(smem, m, 0, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, st, x);
     const u64 *accp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
     u64 *out = a.out + (((size_t)c * 2 + k) * n + i) * Sh::N;
-    sub_scale_run<Sh>(x, accp, cst[0], cst[1], pc, m, tid);   // acc holds d P
+    sub_scale_run<Sh>(x, accp, lc.R, lc.R_sh, pc, m, tid);
     store_run<Sh>(out, x, m, tid);
 }
 
@@ -1180,53 +1241,53 @@ k_rs(EvalArgs a)
     const u32 n = a.n, l = n - 1;
     const u32 c = item / (2 * l), k = (item / l) % 2, i = item % l;
     const PrimeConst pc = a.ctx.pc[i];
-    const u64 *cst = a.ctx.cst + 3 * a.ctx.n_data + 3 * ((size_t)l * a.ctx.n_data + i);
+    const DropConst dc = a.ctx.drop[(size_t)l * a.ctx.n_data + i];
     const u64 half_l = (a.ctx.pc[l].p - 1) / 2;
     const u64 *y = a.lift2 + ((size_t)c * 2 + k) * Sh::N;
     u64 x[Sh::E];
-    auto ld = [&](u32 P) -> u64 { return centred_mod(rd(y + P), half_l, cst[2], pc); };
+    auto ld = [&](u32 P) -> u64 { return centred_mod(rd(y + P), half_l, dc.ql, pc); };
     auto st = [&](u32, u64) {};
     ntt_fwd_block<Sh, false>(smem, m, 0, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, st, x);
     const u64 *src = a.ct2 + (((size_t)c * 2 + k) * n + i) * Sh::N;
     u64 *out = a.out + (((size_t)c * 2 + k) * l + i) * Sh::N;
-    sub_scale_run<Sh>(x, src, cst[0], cst[1], pc, m, tid);
+    sub_scale_run<Sh>(x, src, dc.ql_inv, dc.ql_inv_sh, pc, m, tid);
     store_run<Sh>(out, x, m, tid);
 }
 
 // MulLinRS after the mod-up: mod-down by P and rescale by q_l. The transform
 // is linear, so both divisions of limb i < l share one:
-//   out_i = ((acc_i - NTT_i(r_P)) P^-1 - NTT_i(r_l)) q_l^-1
-//         = (acc_i - NTT_i(r_P + P r_l)) (P q_l)^-1      (mod q_i)
-// with acc the stored d P + acc, r_P the centred residue of y_P = INTT_P(acc)
-// and r_l that of the relinearised limb q_l, which is needed in the
-// coefficient domain only:
-//   y_l = INTT_l((acc_l - NTT_l(r_P)) P^-1) = INTT_l(acc_l) P^-1 - r_P P^-1.
+//   out_i = (d + (acc_i - NTT_i(r_P)) P^-1 - NTT_i(r_l)) q_l^-1
+//         = (s_i - NTT_i((r_P P^-1 + r_l) 2^-64)) 2^64 q_l^-1    (mod q_i)
+// with s the stored (acc P^-1 + d) 2^-64, r_P the centred residue of y_P =
+// INTT_P(acc) and r_l that of the relinearised limb q_l, which is needed in
+// the coefficient domain only:
+//   y_l = INTT_l(d + (acc_l - NTT_l(r_P)) P^-1) = INTT_l(2^64 s_l) - r_P P^-1.
 // So limb q_l takes one inverse transform like the special prime (both in
-// k_mrr_lift; P^-1 is folded into its N^-1 constants), and the 2 (n - 1)
-// forward transforms of k_mrr_rest form r_P + P r_l on their loads. Against
+// k_mrr_lift; 2^64 is folded into its N^-1 constants), and the 2 (n - 1)
+// forward transforms of k_mrr_rest form r_P P^-1 + r_l on their loads. Against
 // a forward and an inverse transform for limb q_l and two forward transforms
 // for every other limb this leaves 2 + 2 + 2 (n - 1) transforms of
 // 2 + 4 + 4 (n - 1). The outputs are canonical, so they are the same words.
-// Measured (one context with 7 + 1 primes at N = 2^14, level 6): 64 pairs
-// 1157 -> 1005 us, one pair 104 -> 75 us.
+// Measured by itself (one context with 7 + 1 primes at N = 2^14, level 6): 64
+// pairs 1157 -> 1005 us, one pair 104 -> 75 us.
 
-// r_P + P r_l mod q_i as a transform input below 7 q_i, from y_P and
-// a_l = INTT_l(acc_l) P^-1 (both canonical): with b_P, b_l the flags of the
+// (r_P P^-1 + r_l) 2^-64 mod q_i as a transform input below 7 q_i, from y_P
+// and a_l = INTT_l(2^64 s_l) (both canonical): with b_P, b_l the flags of the
 // residues above half,
 //   y_l = a_l - y_P P^-1 + b_P (mod q_l),
-//   r_P + P r_l = y_P + P (y_l - b_P) - b_l P q_l.
+//   r_P P^-1 + r_l = y_P P^-1 + (y_l - b_P) - b_l q_l (mod q_i).
 struct RestLift {
     u64 half_P, half_l, ql;
     u64 Pinv_l, Pinv_l_sh;   // P^-1 mod q_l
-    u64 P_i, P_i_sh;         // P mod q_i
-    u64 minus_Pql;           // q_i - (P q_l mod q_i)
+    u64 k1, k1_sh, k2, k2_sh;
+    u64 minus_ql_k2;
     __device__ __forceinline__ u64 operator()(u64 yP, u64 al, const PrimeConst &pc) const
     {
         const u64 bP = yP > half_P ? 1u : 0u;
         const u64 yl = reduce_once(sub_mod(al, mul_shoup(yP, Pinv_l, Pinv_l_sh, ql), ql) + bP, ql);
-        const u64 t0 = reduce_once(reduce_word(yP, pc), pc.two_p);                      // below 2 q_i
-        const u64 t1 = mul_shoup_lazy4_asm(yl + pc.p - bP, P_i, P_i_sh, pc.neg_p);      // below 4 q_i
-        return t0 + t1 + (yl > half_l ? minus_Pql : 0);
+        const u64 t0 = reduce_once(mul_shoup_lazy4_asm(yP, k1, k1_sh, pc.neg_p), pc.two_p);   // below 2 q_i
+        const u64 t1 = mul_shoup_lazy4_asm(yl + pc.p - bP, k2, k2_sh, pc.neg_p);              // below 4 q_i
+        return t0 + t1 + (yl > half_l ? minus_ql_k2 : 0);
     }
 };
 
@@ -1239,16 +1300,20 @@ __device__ __forceinline__ void mrr_rest_body(const EvalArgs &a, u32 item, u32 m
     const u32 n = a.n, l = n - 1, nd = a.ctx.n_data;
     const u32 c = item / (2 * l), k = (item / l) % 2, i = item % l;
     const PrimeConst pc = a.ctx.pc[i];
-    const u64 *cPl = a.ctx.cst + rest_index(a.ctx, l, i);   // (P q_l)^-1, its Shoup quotient, -P q_l (mod q_i)
+    const DropConst &dc = a.ctx.drop[(size_t)l * nd + i];
+    const LimbConst &lc = a.ctx.limb[i];
     RestLift lift;
     lift.half_P = (a.ctx.pc[nd].p - 1) / 2;
     lift.ql = a.ctx.pc[l].p;
     lift.half_l = (lift.ql - 1) / 2;
-    lift.Pinv_l = a.ctx.cst[3 * l];
-    lift.Pinv_l_sh = a.ctx.cst[3 * l + 1];
-    lift.P_i = a.ctx.cst[3 * i + 2];
-    lift.P_i_sh = a.ctx.cst[p_shoup_index(a.ctx, i)];
-    lift.minus_Pql = cPl[2];
+    lift.Pinv_l = a.ctx.limb[l].Pinv;
+    lift.Pinv_l_sh = a.ctx.limb[l].Pinv_sh;
+    lift.k1 = lc.k1;
+    lift.k1_sh = lc.k1_sh;
+    lift.k2 = lc.k2;
+    lift.k2_sh = lc.k2_sh;
+    lift.minus_ql_k2 = dc.minus_ql_k2;
+    const u64 C = dc.R_ql_inv, C_sh = dc.R_ql_inv_sh;
     const u64 *yP = a.plift + ((size_t)c * 2 + k) * Sh::N;
     const u64 *al = a.lift2 + ((size_t)c * 2 + k) * Sh::N;
     u64 x[Sh::E];
@@ -1257,12 +1322,12 @@ __device__ __forceinline__ void mrr_rest_body(const EvalArgs &a, u32 item, u32 m
     ntt_fwd_block<Sh, false>(smem, m, rbase, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, nost, x);
     const u64 *accp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
     u64 *out = a.out + (((size_t)c * 2 + k) * l + i) * Sh::N;
-    sub_scale_run<Sh>(x, accp, cPl[0], cPl[1], pc, m, tid);
+    sub_scale_run<Sh>(x, accp, C, C_sh, pc, m, tid);
     if (valid) store_run<Sh>(out, x, m, tid);
 }
 
 // Inverse transforms before the rest: items below 2 count take accq's limb l
-// of row item = 2 c + k to lift2, times P^-1 (the lift constants); the next
+// of row item = 2 c + k to lift2, times 2^64 (the lift constants); the next
 // 2 count take the special-prime rows of plift in place (inputs in [0, 4P),
 // the key multiply-accumulate's range; not launched after the fused mod-up,
 // which leaves them transformed). Every load precedes the cluster barrier

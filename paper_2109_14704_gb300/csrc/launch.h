@@ -68,29 +68,35 @@ struct MixedUnit {
 cudaError_t launch_ntt_mixed(const MixedUnit *units, u32 n_units, const LimbJob *jobs, bool inverse, u32 clusters,
                              cudaStream_t s);
 
+// Constants of data prime q_i for the divisions. The mod-up leaves its
+// accumulators on the data primes divided by P, with d_k added, and scaled by
+// 2^-64 (the Montgomery reduction of its sums): k1 and k2 bring the lift of
+// the special prime's rows to that scale, R takes it off again.
+struct LimbConst {
+    u64 Pinv, Pinv_sh;   // P^-1 mod q_i
+    u64 k1, k1_sh;       // P^-1 2^-64
+    u64 k2, k2_sh;       // 2^-64
+    u64 R, R_sh;         // 2^64
+};
+// Constants of dropping q_l, for the remaining limb q_i.
+struct DropConst {
+    u64 ql_inv, ql_inv_sh;   // q_l^-1 mod q_i
+    u64 ql;                  // q_l mod q_i
+    u64 R_ql_inv, R_ql_inv_sh;   // 2^64 q_l^-1
+    u64 minus_ql_k2;         // -q_l 2^-64
+};
+
 // Device view of a modulus chain (q_0..q_{n_data-1}, then P at n_data).
 struct DevCtx {
     const ulonglong2 *tw_fwd;   // [n_data + 1][N]
     const ulonglong2 *tw_inv;
     const PrimeConst *pc;       // [n_data + 1]
-    const PrimeConst *pc_lift;  // pc, the data primes' last inverse stage also multiplying by P^-1
-    // cst[3 i + {0,1,2}] = P^-1 mod q_i, its Shoup quotient, P mod q_i;
-    // cst[3 n_data + 3 (l n_data + i) + {0,1,2}] = q_l^-1 mod q_i, Shoup,
-    // q_l mod q_i (rescale from level l, i < l);
-    // cst[3 n_data + 3 n_data^2 + i] = Shoup quotient of P mod q_i;
-    // cst[4 n_data + 3 n_data^2 + 3 (l n_data + i) + {0,1,2}] =
-    // (P q_l)^-1 mod q_i, its Shoup quotient, -P q_l mod q_i (i < l).
-    const u64 *cst;
+    const PrimeConst *pc_lift;  // pc, the data primes' last inverse stage also multiplying by 2^64
+    const LimbConst *limb;      // [n_data]
+    const DropConst *drop;      // [l][n_data], i < l
     u32 N;
     u32 n_data;
 };
-
-__host__ __device__ inline u32 p_shoup_index(const DevCtx &c, u32 i) { return 3 * c.n_data * (1 + c.n_data) + i; }
-
-__host__ __device__ inline u32 rest_index(const DevCtx &c, u32 l, u32 i)
-{
-    return c.n_data * (4 + 3 * c.n_data) + 3 * (l * c.n_data + i);
-}
 
 struct EvalArgs {
     const u64 *ct_a, *ct_b;     // [count][2][n][N] (fused Mul) or null
@@ -101,7 +107,8 @@ struct EvalArgs {
     u64 *accq;                  // scratch [count][2][n][N]
     u64 *plift;                 // scratch [count][2][N]
     u64 *lift2;                 // scratch [count][2][N]
-    const ulonglong2 *evk;      // [n_data][2][n_data + 1][N] (value, Shoup)
+    const ulonglong2 *evk;      // [n_data][2][n_data + 1][N] (value, Shoup quotient)
+    const u64 *evk_mac;         // same order: value P^-1 mod q_i (2^64 P^-1 for digit j = i), value 2^64 mod P on the special prime
     u64 *mx;                    // expanded mod-up scratch [group][n + 1][n][N]
     u32 n;                      // limbs at the current level
     u32 count;
@@ -114,14 +121,15 @@ struct EvalArgs {
 // covers every job; job i's items in stage S start at job[i].begin[S].
 // Multi-degree batches (a context and key per job, degrees 2^12 .. 2^15):
 // the transform stages count units (clusters of 8 CTAs, each running 8 >> c
-// items of degree 2^(12 + c) side by side) instead of items.
+// items of degree 2^(12 + c) side by side) instead of items. JS_MAC counts
+// tiles of MAC_BLOCK positions.
 enum JobStage { JS_DIGITS = 0, JS_EXPAND, JS_MAC, JS_LIFT, JS_REST, JS_COUNT };
 constexpr u32 kMaxJobs = 16;
 struct EvalJob {
     const u64 *ct_a, *ct_b;     // [count][2][n][N]
     u64 *out;                   // [count][2][n - 1][N]
     u64 *c2, *accq, *plift, *lift2, *mx;   // the job's scratch regions
-    const ulonglong2 *evk;      // the job's key
+    const u64 *evk_mac;         // the job's key
     DevCtx ctx;                 // the job's context
     u32 n, count;
     u32 begin[JS_COUNT];

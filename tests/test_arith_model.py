@@ -159,9 +159,9 @@ def test_sign_tested_comparison():
 
 @pytest.mark.parametrize("P_bits,ql_bits,qi_bits", [(60, 60, 60), (60, 40, 31), (31, 60, 60), (31, 31, 60), (60, 31, 50)])
 def test_shared_division_input(P_bits, ql_bits, qi_bits):
-    """The rest stage's transform input: from y_P and a_l = [acc_l P^-1] it is
-    congruent to r_P + P r_l mod q_i (both residues centred, r_l that of
-    (acc_l - r_P) P^-1) and below 7 q_i, at the edges of every range."""
+    """The rest stage's transform input: from y_P and a_l = [2^64 s_l] it is
+    congruent to (r_P P^-1 + r_l) 2^-64 mod q_i (both residues centred, r_l
+    that of a_l - r_P P^-1) and below 7 q_i, at the edges of every range."""
     N = 1024
     primes = []
     for b in (P_bits, ql_bits, qi_bits):
@@ -169,20 +169,56 @@ def test_shared_division_input(P_bits, ql_bits, qi_bits):
     P, ql, qi = primes
     half_P, half_l = (P - 1) // 2, (ql - 1) // 2
     Pinv = pow(P, -1, ql)
+    k2 = pow(1 << 64, -1, qi)
+    k1 = pow(P, -1, qi) * k2 % qi
     r = random.Random(P_bits * 7 + ql_bits)
     edges = lambda m: [0, 1, m // 2 - 1, m // 2, m // 2 + 1, m - 2, m - 1] + [r.randrange(m) for _ in range(40)]
     for yP in edges(P):
         for al in edges(ql):
             bP = int(yP > half_P)
-            s = lazy4(yP, Pinv, shoup_pre(Pinv, ql), ql)          # the exact quotient gives [0, 2 q_l)
-            s = s % ql
-            yl = reduce_once(sub_mod(al, s, ql) + bP, ql)
-            t0 = reduce_once(lazy4(yP, 1, shoup_pre(1, qi), qi), 2 * qi)
-            Pi = P % qi
-            t1 = lazy4(yl + qi - bP, Pi, shoup_pre(Pi, qi), qi)
-            v = t0 + t1 + (qi - P * ql % qi if yl > half_l else 0)
+            yl = reduce_once(sub_mod(al, yP * Pinv % ql, ql) + bP, ql)
+            t0 = reduce_once(lazy4(yP, k1, shoup_pre(k1, qi), qi), 2 * qi)
+            t1 = lazy4(yl + qi - bP, k2, shoup_pre(k2, qi), qi)
+            v = t0 + t1 + (qi - ql * k2 % qi if yl > half_l else 0)
             rP = yP - P if yP > half_P else yP
             want_l = (al - rP * Pinv) % ql
             rl = want_l - ql if want_l > half_l else want_l
             assert yl == want_l
-            assert v < 7 * qi and (v - (rP + P * rl)) % qi == 0
+            assert v < 7 * qi and (v * P * (1 << 64) - (rP + P * rl)) % qi == 0
+
+
+@pytest.mark.parametrize("bits", [31, 40, 50, 60])
+def test_key_sum_bounds(bits):
+    """The key multiply-accumulate's sum of 32 digits below 4 p + 2^32 and two
+    tensor products stays below 2^128, and its Montgomery reduction is
+    congruent to the sum times 2^-64 and below 10 p."""
+    p = oracle.find_primes(bits, 2048, 1)[0]
+    mneg = -pow(p, -1, 1 << 64) % (1 << 64)
+    r = random.Random(bits)
+    top = 4 * p + (1 << 32) - 1
+    for trial in range(60):
+        pick = (lambda m: m) if trial == 0 else (lambda m: r.choice([0, 1, m, m - 1, r.randrange(m)]))
+        s = sum(pick(top) * pick(p - 1) for _ in range(32)) + 2 * pick(p - 1) * pick(p - 1)
+        assert s < 1 << 128
+        lo, hi = s & M64, s >> 64
+        m = lo * mneg & M64
+        v = hi + (m * p >> 64) + (1 if lo else 0)
+        assert v < 10 * p and (v * (1 << 64) - s) % p == 0
+
+
+@pytest.mark.parametrize("bits", [31, 32, 40, 47, 48, 60])
+def test_shoup_quotient_in_two_steps(bits):
+    """floor(w 2^64 / p) from two 32-bit steps, each short by at most two."""
+    p = oracle.find_primes(bits, 2048, 1)[0]
+    mu = (1 << (2 * bits + 2)) // p
+    r0 = random.Random(bits)
+    for w in [0, 1, p - 1, p // 2] + [r0.randrange(p) for _ in range(300)]:
+        r, q = w, 0
+        for _ in range(2):
+            qs = r * mu >> (2 * bits - 30)
+            rest = (r << 32) - qs * p
+            assert 0 <= rest < 3 * p
+            qs, r = qs + rest // p, rest % p
+            assert qs < 1 << 32
+            q = (q << 32) + qs
+        assert q == (w << 64) // p
