@@ -870,6 +870,34 @@ static u32 mac_grid(u64 tiles) { return (u32)std::max<u64>(1, std::min<u64>(tile
 // the special prime's accumulators in plift are left in the NTT domain
 // (*special_ntt = true). Otherwise the fused k_ks_modup runs, which also takes
 // them through the inverse transform.
+// The key multiply-accumulate of a uniform group of gs ciphertexts.
+template <int KIND>
+static he_status ks_mac(const he_context *ctx, const he::EvalArgs &a, u32 gs, cudaStream_t s)
+{
+    const u32 n = a.n;
+    if (gs >= 8) {   // a warp per ciphertext: all of them busy
+        const u32 blocks = (n + 1) * (ctx->N / he::MAC_TILE) * ((gs + he::MAC_CHUNK - 1) / he::MAC_CHUNK);
+        const u32 smem = n * 2 * he::MAC_TILE * 8;   // 32 KB at the longest chain
+        he::k_ks_mac_tiled<KIND><<<blocks, 256, smem, s>>>(a, gs);
+    } else {
+        const u32 tiles = gs * (n + 1) * (ctx->N / he::MAC_BLOCK);
+        he::k_ks_mac<false, KIND><<<mac_grid(tiles), he::MAC_BLOCK / 2, 0, s>>>(a, gs, tiles, he::NoJobs{});
+    }
+    HE_CUDA(cudaGetLastError());
+    return HE_OK;
+}
+
+static he::SourceKind source_kind(const he::EvalArgs &a)
+{
+    return !a.ct3 ? he::SRC_PAIR : (a.galois ? he::SRC_ROTATE : he::SRC_THREE);
+}
+
+static he::EvalKernel digits_kernel(const he::EvalArgs &a)
+{
+    const he::SourceKind k = source_kind(a);
+    return k == he::SRC_PAIR ? he::EK_KS_DIGITS : (k == he::SRC_THREE ? he::EK_KS_DIGITS_THREE : he::EK_KS_DIGITS_ROTATE);
+}
+
 static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64 *xbuf, size_t x_words,
                           bool *special_ntt, cudaStream_t s)
 {
@@ -883,15 +911,11 @@ static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64
         const u32 gs = std::min(group, count - c0);
         a.c_first = c0;
         if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, gs * (n + 1) * n, s)) return r;
-        if (gs >= 8) {   // a warp per ciphertext: all of them busy
-            const u32 blocks = (n + 1) * (ctx->N / he::MAC_TILE) * ((gs + he::MAC_CHUNK - 1) / he::MAC_CHUNK);
-            const u32 smem = n * 2 * he::MAC_TILE * 8;   // 32 KB at the longest chain
-            he::k_ks_mac_tiled<<<blocks, 256, smem, s>>>(a, gs);
-        } else {
-            const u32 tiles = gs * (n + 1) * (ctx->N / he::MAC_BLOCK);
-            he::k_ks_mac<false><<<mac_grid(tiles), he::MAC_BLOCK / 2, 0, s>>>(a, gs, tiles, he::NoJobs{});
-        }
-        HE_CUDA(cudaGetLastError());
+        const he::SourceKind kind = source_kind(a);
+        he_status r = kind == he::SRC_PAIR    ? ks_mac<he::SRC_PAIR>(ctx, a, gs, s)
+                      : kind == he::SRC_THREE ? ks_mac<he::SRC_THREE>(ctx, a, gs, s)
+                                              : ks_mac<he::SRC_ROTATE>(ctx, a, gs, s);
+        if (r) return r;
     }
     a.mx = nullptr;
     a.c_first = 0;
@@ -923,7 +947,7 @@ extern "C" he_status he_relin(uint64_t *ct_out2, const uint64_t *ct_in3, const h
     cudaStream_t s = (cudaStream_t)stream;
     u64 *xbuf = (u64 *)scratch + relin_words(ctx, n);
     const size_t x_words = scratch_bytes / 8 - relin_words(ctx, n);
-    if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, n, s)) return r;
+    if (he_status r = run_eval(ctx, digits_kernel(a), a, n, s)) return r;
     bool special_ntt = false;
     if (he_status r = ks_modup(ctx, a, 1, xbuf, x_words, &special_ntt, s)) return r;
     if (special_ntt)
@@ -952,12 +976,14 @@ extern "C" he_status he_rescale(uint64_t *ct_out, const uint64_t *ct_in, const h
 }
 
 // Key switching of `count` ciphertexts whose third component is given either
-// as the tensor of a pair (ct_a, ct_b: Mul fused into the loads) or as a
-// three-component input ct3, then (rescale = true) RS by q_l (MulLinRS
+// as the tensor of a pair (ct_a, ct_b: Mul fused into the loads), as a
+// three-component input ct3, or (galois nonzero) as the rotation (sigma(c0), 0,
+// sigma(c1)) of two-component inputs ct3, gathered on the loads; then (rescale = true) RS by q_l (MulLinRS
 // kernels) or (rescale = false) the mod-down only (MulLin / Relin).
 static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const uint64_t *ct_b, const uint64_t *ct3,
                                    uint32_t count, const he_relin_key *key, const he_context *ctx, uint32_t level,
-                                   void *scratch, size_t scratch_bytes, he_stream_t stream, bool rescale)
+                                   void *scratch, size_t scratch_bytes, he_stream_t stream, bool rescale,
+                                   uint32_t galois = 0)
 {
     if (he_status s = check_level(ctx, level, rescale)) return s;
     if (!key || key->ctx != ctx) return fail(HE_EINVAL, "relin key is NULL or belongs to another context");
@@ -978,6 +1004,7 @@ static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const
     a.ct_a = ct3 ? nullptr : ct_a;
     a.ct_b = ct3 ? nullptr : ct_b;
     a.ct3 = ct3;
+    a.galois = galois;
     a.out = ct_out;
     a.c2 = (u64 *)scratch;
     a.accq = a.c2 + (size_t)count * n * ctx->N;
@@ -991,7 +1018,7 @@ static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const
     cudaStream_t s = (cudaStream_t)stream;
     u64 *xbuf = (u64 *)scratch + base_words;
     const size_t x_words = scratch_bytes / 8 - base_words;
-    if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, count * n, s)) return r;
+    if (he_status r = run_eval(ctx, digits_kernel(a), a, count * n, s)) return r;
     bool special_ntt = false;
     if (he_status r = ks_modup(ctx, a, count, xbuf, x_words, &special_ntt, s)) return r;
     if (!rescale) {
@@ -1109,7 +1136,7 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
     a.n = t.job[0].n;   // unused with a job table; kept valid
     if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, (u32)tot[he::JS_DIGITS], s, &t)) return r;
     if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, (u32)tot[he::JS_EXPAND], s, &t)) return r;
-    he::k_ks_mac<true><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
+    he::k_ks_mac<true, he::SRC_PAIR><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
     if (he_status r = run_eval(ctx, he::EK_MRR_LIFT, a, (u32)tot[he::JS_LIFT], s, &t)) return r;
     return run_eval(ctx, he::EK_MRR_REST, a, (u32)tot[he::JS_REST], s, &t);
@@ -1190,8 +1217,9 @@ extern "C" he_status he_ct_automorph(uint64_t *ct_out, const uint64_t *ct_in, ui
     return HE_OK;
 }
 
-// Rotate scratch: the three-component input (sigma(c0), 0, sigma(c1)) of the
-// key switch, then the key switch's own scratch (with the expanded mod-up).
+// Rotate scratch: room for the three-component input of the key switch
+// (callers size their buffers by it; the rotation is gathered on the loads and
+// the key switch takes the whole buffer), and the key switch's own scratch.
 static size_t rotate_c3_words(const he_context *c, u32 n, u32 count) { return (size_t)3 * n * c->N * count; }
 
 extern "C" size_t he_rotate_scratch_bytes(const he_context *ctx, uint32_t level, uint32_t count)
@@ -1213,19 +1241,8 @@ extern "C" he_status he_rotate(uint64_t *ct_out, const uint64_t *ct_in, uint32_t
     const u32 n = level + 1;
     const size_t c3_words = rotate_c3_words(ctx, n, count);
     if (scratch_bytes < (c3_words + relin_words(ctx, n) * count) * 8) return fail(HE_EINVAL, "scratch too small");
-    u64 *c3 = (u64 *)scratch;
-    const size_t comp = (size_t)n * ctx->N;
-    cudaStream_t s = (cudaStream_t)stream;
-    // (sigma(c0), 0, sigma(c1)) per ciphertext
-    for (u32 c = 0; c < count; c++) {
-        if (he_status r = he_ct_automorph(c3 + (size_t)c * 3 * comp, ct_in + (size_t)c * 2 * comp, 1, 1, galois_elt,
-                                          ctx, level, stream)) return r;
-        HE_CUDA(cudaMemsetAsync(c3 + ((size_t)c * 3 + 1) * comp, 0, comp * 8, s));
-        if (he_status r = he_ct_automorph(c3 + ((size_t)c * 3 + 2) * comp, ct_in + ((size_t)c * 2 + 1) * comp, 1, 1,
-                                          galois_elt, ctx, level, stream)) return r;
-    }
-    return key_switch_common(ct_out, nullptr, nullptr, c3, count, galois_key, ctx, level, c3 + c3_words,
-                             scratch_bytes - c3_words * 8, stream, false);
+    return key_switch_common(ct_out, nullptr, nullptr, ct_in, count, galois_key, ctx, level, scratch, scratch_bytes,
+                             stream, false, galois_elt);
 }
 
 extern "C" he_status he_ct_matmul_tensor(uint64_t *t_out, const uint64_t *a, const uint64_t *b, uint32_t m,
@@ -2001,7 +2018,7 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
     a.n = t.job[0].n;
     HE_CUDA(he::launch_mrr_multi(he::MS_DIGITS, a, t, (u32)tot[he::JS_DIGITS], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_EXPAND, a, t, (u32)tot[he::JS_EXPAND], s));
-    he::k_ks_mac<true><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
+    he::k_ks_mac<true, he::SRC_PAIR><<<mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, s>>>(a, 0, (u32)tot[he::JS_MAC], t);
     HE_CUDA(cudaGetLastError());
     HE_CUDA(he::launch_mrr_multi(he::MS_LIFT, a, t, (u32)tot[he::JS_LIFT], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_REST, a, t, (u32)tot[he::JS_REST], s));

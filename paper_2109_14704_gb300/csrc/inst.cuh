@@ -115,6 +115,16 @@ struct ShapeOps {
         return n;
     }
 
+    template <int KIND>
+    static cudaError_t digits_of(const EvalArgs &a, u32 grid, const JobTable *jobs, cudaStream_t s)
+    {
+        if (jobs) return cudaErrorInvalidValue;
+        static std::once_flag f;
+        static cudaError_t e = cudaSuccess;
+        if (cudaError_t r = smem_attr(k_ks_digits_of<LOG_B, LOG_C, LOG_E, KIND>, Sh::SMEM_BYTES, f, e)) return r;
+        return launch_k(k_ks_digits_of<LOG_B, LOG_C, LOG_E, KIND>, grid, Sh::T, Sh::SMEM_BYTES, Sh::C, s, a);
+    }
+
     static cudaError_t eval(EvalKernel k, const EvalArgs &a, u32 items, const JobTable *jobs, cudaStream_t s)
     {
         const u32 grid = items * Sh::C;
@@ -143,6 +153,8 @@ struct ShapeOps {
         return launch_k(KERNEL<LOG_B, LOG_C, LOG_E, false>, grid, Sh::T, SMEM, Sh::C, s, a, NoJobs{});      \
     }
             HE_EVAL_CASE_J(EK_KS_DIGITS, k_ks_digits, sm1)
+        case EK_KS_DIGITS_THREE: return digits_of<SRC_THREE>(a, grid, jobs, s);
+        case EK_KS_DIGITS_ROTATE: return digits_of<SRC_ROTATE>(a, grid, jobs, s);
             HE_EVAL_CASE(EK_KS_MODUP, k_ks_modup, sm3)
             HE_EVAL_CASE_J(EK_KS_EXPAND, k_ks_expand, sm1)
             HE_EVAL_CASE(EK_KS_MODDOWN, k_ks_moddown, sm1)

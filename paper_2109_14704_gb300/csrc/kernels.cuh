@@ -268,6 +268,19 @@ k_negacyclic(NegaLaunch a)
     ntt_inv_block<Sh, true>(smem, m, 0, twi, pc, nold, st, x);
 }
 
+// Word of an NTT-domain polynomial that X -> X^g brings to index i. Index i
+// holds a(psi^(2 brv(i) + 1)) (the order of he_ntt_fwd), so the image
+// sigma(a)(psi^(2 brv(i) + 1)) = a(psi^(g (2 brv(i) + 1))) is the input word at
+// index brv((g (2 brv(i) + 1) mod 2N - 1) / 2). The low k bits of i are the
+// high k bits of brv(i), which only reach the high k bits of the product: an
+// aligned run of 2^k words comes from an aligned run of 2^k words.
+__device__ __forceinline__ u32 automorph_index(u32 i, u32 log_n, u32 g)
+{
+    const u32 mask2 = (2u << log_n) - 1, sh = 32 - log_n;
+    const u32 t = (g * (2 * (__brev(i) >> sh) + 1)) & mask2;   // mod 2^32 is enough: 2N divides it
+    return __brev((t - 1) >> 1) >> sh;
+}
+
 #ifdef HE_MISC_KERNELS  // defined by the one translation unit that owns them
 // ======================================================== naive radix-2 ====
 // The baseline of Sec. III-B: one launch per stage, each thread one
@@ -384,20 +397,14 @@ __global__ void k_ct_add(u64 *out, const u64 *a, const u64 *b, u64 words, u32 lo
 }
 
 // The automorphism X -> X^g (g odd) on NTT-domain polynomials of 2^log_n
-// words (any number of them, back to back). Output index i holds
-// a(psi^(2 brv(i) + 1)) (the order of he_ntt_fwd), so the image
-// sigma(a)(psi^(2 brv(i) + 1)) = a(psi^(g (2 brv(i) + 1))) is the input
-// word at index brv((g (2 brv(i) + 1) mod 2N - 1) / 2): a gather within
-// each polynomial, the same for every limb.
+// words (any number of them, back to back): a gather within each polynomial,
+// the same for every limb (automorph_index).
 __global__ void k_ct_automorph(u64 *out, const u64 *in, u64 words, u32 log_n, u32 g)
 {
-    const u32 N = 1u << log_n, mask2 = 2 * N - 1, sh = 32 - log_n;
+    const u32 N = 1u << log_n;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u32 i = (u32)e & (N - 1);
-        const u32 r = __brev(i) >> sh;
-        const u32 t = (u32)(((u64)g * (2 * r + 1)) & mask2);
-        const u32 src = __brev((t - 1) >> 1) >> sh;
-        out[e] = __ldg(reinterpret_cast<const unsigned long long *>(in + (e - i) + src));
+        out[e] = __ldg(reinterpret_cast<const unsigned long long *>(in + (e - i) + automorph_index(i, log_n, g)));
     }
 }
 
@@ -691,6 +698,7 @@ __device__ __forceinline__ u32 bind_job(EvalArgs &a, const JobTable &t, int S, u
     a.ct_a = J.ct_a;
     a.ct_b = J.ct_b;
     a.ct3 = nullptr;
+    a.galois = 0;
     a.out = J.out;
     a.c2 = J.c2;
     a.accq = J.accq;
@@ -708,23 +716,44 @@ __device__ __forceinline__ u32 bind_job(EvalArgs &a, const JobTable &t, int S, u
 struct DSource {
     const u64 *ct_a, *ct_b, *ct3;  // per-ciphertext bases
     size_t per;                    // n * N words per component
+    u32 galois;                    // nonzero: ct3 = (c0, c1), read as (sigma(c0), 0, sigma(c1))
+    // the third component, and its word at position P of a limb
+    __device__ __forceinline__ const u64 *third() const { return ct3 + (galois ? per : 2 * per); }
     __device__ __forceinline__ u64 d(int k, u32 limb, u32 log_n, u32 P, const PrimeConst &pc) const
     {
+        if (galois) {
+            if (k == 1) return 0;
+            return rd(ct3 + (k ? per : 0) + ((size_t)limb << log_n) + automorph_index(P, log_n, galois));
+        }
         const size_t off = ((size_t)limb << log_n) + P;
         if (ct3) return rd(ct3 + k * per + off);
         if (k == 0) return mul_mod(rd(ct_a + off), rd(ct_b + off), pc);
         if (k == 1) return mad2_mod(rd(ct_a + off), rd(ct_b + per + off), rd(ct_a + per + off), rd(ct_b + off), pc);
         return mul_mod(rd(ct_a + per + off), rd(ct_b + per + off), pc);
     }
+    // words P, P + 1 (P even) of a limb row `row` of ct3, through sigma if set:
+    // the pair comes from a pair, in either order
+    __device__ __forceinline__ ulonglong2 pair(const u64 *row, u32 log_n, u32 P) const
+    {
+        const u32 src = galois ? automorph_index(P, log_n, galois) : P;
+        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(row + (src & ~1u)));
+        return (src & 1u) ? make_ulonglong2(v.y, v.x) : v;
+    }
 };
 
+// KIND: the input known at compile time (a kernel that tells them apart at run
+// time holds the registers of all three), or SRC_ANY.
+template <int KIND = SRC_ANY>
 __device__ __forceinline__ DSource dsource(const EvalArgs &a, u32 c)
 {
     DSource s;
     s.per = (size_t)a.n * a.ctx.N;
-    s.ct3 = a.ct3 ? a.ct3 + (size_t)c * 3 * s.per : nullptr;
+    s.galois = (KIND == SRC_ROTATE || KIND == SRC_ANY) ? a.galois : 0;
+    s.ct3 = (KIND == SRC_PAIR || !a.ct3) ? nullptr : a.ct3 + (size_t)c * (s.galois ? 2 : 3) * s.per;
     s.ct_a = a.ct_a ? a.ct_a + (size_t)c * 2 * s.per : nullptr;
     s.ct_b = a.ct_b ? a.ct_b + (size_t)c * 2 * s.per : nullptr;
+    if (KIND == SRC_THREE || KIND == SRC_ROTATE) __builtin_assume(s.ct3 != nullptr);
+    if (KIND == SRC_ROTATE) __builtin_assume(s.galois != 0);
     return s;
 }
 
@@ -736,12 +765,12 @@ __device__ __forceinline__ DSource dsource(const EvalArgs &a, u32 c)
 // all CTAs of the cluster pass the same cluster barriers).
 
 // Digit INTT: c2[c][j] = INTT_{q_j}(d2[c][j]), item = c n + j.
-template <class Sh>
+template <class Sh, int KIND = SRC_PAIR>
 __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 m, u32 rbase, bool valid)
 {
     extern __shared__ __align__(16) u64 smem[];
     const u32 c = item / a.n, j = item % a.n;
-    const DSource ds = dsource(a, c);
+    const DSource ds = dsource<KIND>(a, c);
     const PrimeConst pc = ds.ct3 ? a.ctx.pc[j] : a.ctx.pc_lift[j];
     u64 *out = a.c2 + ((size_t)c * a.n + j) * Sh::N;
     const u32 tid = threadIdx.x;
@@ -749,12 +778,29 @@ __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 
     // the thread's inverse-input positions (consecutive quarters): the given
     // third component, or a1 b1 as Montgomery products, below 2 q_j and
     // scaled by 2^-64, which the lift constants' last stage takes off
-    const size_t off = ds.per + (size_t)j * Sh::N;
     if (ds.ct3) {
-        const u64 *d = ds.ct3 + ds.per + off;
+        const u64 *d = ds.third() + (size_t)j * Sh::N;
+        if (ds.galois) {
+            // four words come from an aligned run of four, in some order
 #pragma unroll
-        for (int e = 0; e < Sh::E; e += 4) ld4_nc(d + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+            for (int e = 0; e < Sh::E; e += 4) {
+                const u32 P = (u32)last_pos<Sh>(m, tid, e);
+                const u32 src = automorph_index(P, Sh::LOG_N, ds.galois);
+                u64 v[4];
+                ld4_nc(d + (src & ~3u), v[0], v[1], v[2], v[3]);
+#pragma unroll
+                for (u32 i = 0; i < 4; i++) {
+                    const u32 o = (i ? automorph_index(P + i, Sh::LOG_N, ds.galois) : src) & 3u;
+                    x[e + i] = (o & 2u) ? ((o & 1u) ? v[3] : v[2]) : ((o & 1u) ? v[1] : v[0]);
+                }
+            }
+        } else {
+#pragma unroll
+            for (int e = 0; e < Sh::E; e += 4)
+                ld4_nc(d + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+        }
     } else {
+        const size_t off = ds.per + (size_t)j * Sh::N;
 #pragma unroll
         for (int e = 0; e < Sh::E; e += 4) {
             const int P = last_pos<Sh>(m, tid, e);
@@ -782,6 +828,15 @@ k_ks_digits(EvalArgs a0, JobsArg<JOBS> tab)
     u32 item = blockIdx.x >> LOG_C;
     if constexpr (JOBS) item = bind_job(a, tab, JS_DIGITS, item);
     ks_digits_body<Sh>(a, item, m, 0, true);
+}
+
+// The same for given three-component inputs and for rotations.
+template <int LOG_B, int LOG_C, int LOG_E, int KIND>
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
+k_ks_digits_of(EvalArgs a)
+{
+    const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
+    ks_digits_body<NttShape<LOG_B, LOG_C, LOG_E>, KIND>(a, blockIdx.x >> LOG_C, m, 0, true);
 }
 
 template <int LOG_B, int LOG_C, int LOG_E>
@@ -940,6 +995,7 @@ struct MacVec {
         const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2 *>(p));
         return {{t.x, t.y}};
     }
+    __device__ __forceinline__ static MacVec of(ulonglong2 t) { return {{t.x, t.y}}; }
     __device__ __forceinline__ static MacVec shared(const u64 *p)
     {
         const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
@@ -980,14 +1036,14 @@ struct MacSums {
 #pragma unroll
             for (int i = 0; i < 2; i++) s[k][i].clear();
         if (t == n) return;
-        const size_t off = ((size_t)t << log_n) + P;
         Vec d;
         if (ds.ct3) {
             const LimbConst &lc = limb[t];
-            d = Vec::load(ds.ct3 + 2 * ds.per + off);
+            d = Vec::of(ds.pair(ds.third() + ((size_t)t << log_n), log_n, P));
 #pragma unroll
             for (int i = 0; i < 2; i++) d.v[i] = mul_shoup_lazy4_asm(d.v[i], lc.k2, lc.k2_sh, pc.neg_p);
         } else {
+            const size_t off = ((size_t)t << log_n) + P;
             const Vec a0 = Vec::load(ds.ct_a + off), a1 = Vec::load(ds.ct_a + ds.per + off);
             const Vec b0 = Vec::load(ds.ct_b + off), b1 = Vec::load(ds.ct_b + ds.per + off);
             add(a0, 0, b0);
@@ -1010,9 +1066,9 @@ struct MacSums {
             for (int i = 0; i < 2; i++) o.v[i] = s[k][i].redc(pc);
             u64 *dst;
             if (t < n) {
-                if (ds.ct3) {
+                if (ds.ct3 && !(k == 1 && ds.galois)) {
                     const LimbConst &lc = a.ctx.limb[t];
-                    const Vec d = Vec::load(ds.ct3 + k * ds.per + ((size_t)t << log_n) + P);
+                    const Vec d = Vec::of(ds.pair(ds.ct3 + k * ds.per + ((size_t)t << log_n), log_n, P));
 #pragma unroll
                     for (int i = 0; i < 2; i++) o.v[i] += mul_shoup_lazy4_asm(d.v[i], lc.k2, lc.k2_sh, pc.neg_p);
                 }
@@ -1033,6 +1089,7 @@ struct MacSums {
 // words are loaded while the current products run.
 constexpr u32 MAC_BLOCK = 512;
 
+template <int KIND>
 __device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 tile)
 {
     using Vec = MacVec;
@@ -1043,7 +1100,7 @@ __device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 t
     const u32 tp = (t == n) ? a.ctx.n_data : t;
     const PrimeConst pc = a.ctx.pc[tp];
     const u32 c = a.c_first + g;
-    const DSource ds = dsource(a, c);
+    const DSource ds = dsource<KIND>(a, c);
     const size_t key_k = (size_t)nd1 * N, key_j = 2 * key_k;             // evk [j][k][target][N]
     const u64 *key = a.evk_mac + (size_t)tp * N + P;
     const u64 *mx = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;        // mx [g][target][j][N]
@@ -1069,16 +1126,16 @@ __device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 t
 // Tiles of a uniform group (groups x (n + 1) targets x N / MAC_BLOCK), or
 // those of every job of a table back to back (each job one group of all its
 // ciphertexts).
-template <bool JOBS = false>
+template <bool JOBS, int KIND>
 __global__ void __launch_bounds__(MAC_BLOCK / 2, 4) k_ks_mac(EvalArgs a0, u32 groups, u32 total, JobsArg<JOBS> tab)
 {
     for (u32 q = blockIdx.x; q < total; q += gridDim.x) {
         if constexpr (JOBS) {
             EvalArgs a = a0;
             const u32 local = bind_job(a, tab, JS_MAC, q);
-            ks_mac_tile(a, a.count, local);
+            ks_mac_tile<KIND>(a, a.count, local);
         } else {
-            ks_mac_tile(a0, groups, q);
+            ks_mac_tile<KIND>(a0, groups, q);
         }
     }
 }
@@ -1096,6 +1153,7 @@ __global__ void __launch_bounds__(MAC_BLOCK / 2, 4) k_ks_mac(EvalArgs a0, u32 gr
 // copies 4 % slower (more instructions; the loads are not what it waits for).
 constexpr u32 MAC_TILE = 64, MAC_CHUNK = 32;
 
+template <int KIND>
 __global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
 {
     using Vec = MacVec;
@@ -1120,7 +1178,7 @@ __global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
     for (u32 g = chunk * MAC_CHUNK + warp; g < gend; g += 8) {
         const u64 *mx = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;   // mx [g][target][j][N]
         const u32 c = a.c_first + g;
-        const DSource ds = dsource(a, c);
+        const DSource ds = dsource<KIND>(a, c);
         const u32 terms = t < n ? n - 1 : n, jt = t < n ? t : 0;
         u32 j = t == 0 ? 1u : 0u;
         Vec v;
@@ -1179,8 +1237,11 @@ __global__ void k_key_prepare(ulonglong2 *evk, u64 *evk_mac, const u64 *raw, u64
 // Relin mod-down (no rescale): out[c][k][i] = d_k[i] + (acc - NTT(r)) P^-1,
 // at the accumulator's scale: (stored acc - NTT(r P^-1 2^-64)) 2^64, with
 // r P^-1 = y P^-1 - 1 where y is above half.
+// One transform a limb at the plain transform's register budget (at 126
+// registers, two CTAs of 256 an SM, 126 us for 256 limbs of 2^15 words; at 64
+// 98 us).
 template <int LOG_B, int LOG_C, int LOG_E>
-__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_ks_moddown(EvalArgs a)
 {
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
@@ -1210,7 +1271,7 @@ k_ks_moddown(EvalArgs a)
 
 // RS, first half: y_k = INTT_{q_l}(c_k[q_l]) -> lift2 (coefficient domain).
 template <int LOG_B, int LOG_C, int LOG_E>
-__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_rs_lift(EvalArgs a)
 {
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
@@ -1230,7 +1291,7 @@ k_rs_lift(EvalArgs a)
 
 // RS, second half: out[c][k][i] = (c_k[q_i] - NTT(r mod q_i)) q_l^-1, i < l.
 template <int LOG_B, int LOG_C, int LOG_E>
-__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_rs(EvalArgs a)
 {
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;

@@ -98,9 +98,13 @@ struct DevCtx {
     u32 n_data;
 };
 
+// Input of a key switch: a pair of ciphertexts to multiply, a three-component
+// ciphertext, or a rotation.
+enum SourceKind { SRC_PAIR = 0, SRC_THREE, SRC_ROTATE, SRC_ANY };
+
 struct EvalArgs {
     const u64 *ct_a, *ct_b;     // [count][2][n][N] (fused Mul) or null
-    const u64 *ct3;             // [count][3][n][N] or null
+    const u64 *ct3;             // [count][3][n][N] or null; with galois, [count][2][n][N]
     const u64 *ct2;             // [count][2][n][N] rescale input
     u64 *out;
     u64 *c2;                    // scratch [count][n][N]
@@ -113,7 +117,7 @@ struct EvalArgs {
     u32 n;                      // limbs at the current level
     u32 count;
     u32 c_first;                // first ciphertext of the expanded mod-up group
-    u32 pad;
+    u32 galois;                 // nonzero: the input is (sigma(c0), 0, sigma(c1)), sigma: X -> X^galois
     DevCtx ctx;
 };
 
@@ -149,7 +153,9 @@ enum MultiStage { MS_DIGITS = 0, MS_EXPAND, MS_LIFT, MS_REST, MS_COUNT };
 cudaError_t launch_mrr_multi(MultiStage stage, const EvalArgs &a, const JobTable &t, u32 units, cudaStream_t s);
 
 enum EvalKernel {
-    EK_KS_DIGITS = 0,
+    EK_KS_DIGITS = 0,   // by the source: pair (also job tables), three components, rotation
+    EK_KS_DIGITS_THREE,
+    EK_KS_DIGITS_ROTATE,
     EK_KS_MODUP,
     EK_KS_EXPAND,
     EK_KS_MODDOWN,
