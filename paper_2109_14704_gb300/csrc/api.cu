@@ -1463,7 +1463,7 @@ static he_status crt_compose(const he_encoder *enc, double *out, const uint64_t 
                              cudaStream_t s)
 {
     const u64 total = (u64)count * enc->ctx->N;
-    HE_CUDA(he::launch_crt_compose(out, coeffs, enc->d_crt + enc->crt_off[level], enc->crt_nw[level],
+    HE_CUDA(he::launch_crt_compose(out, coeffs, enc->d_crt + enc->crt_off[level], enc->d_primes, enc->crt_nw[level],
                                    (u32)enc->ctx->log_n, level + 1, total, stream_grid(total, 128), s));
     return HE_OK;
 }
@@ -1495,8 +1495,9 @@ extern "C" he_status he_decode(const he_encoder *enc, double *slots_out, const u
     u64 *coef = (u64 *)scratch;                            // [count][level + 1][N]
     double *m = (double *)(coef + words);                  // [count][N]
     double2 *u = (double2 *)(m + (size_t)count * ctx->N);  // [count][N / 2]
-    HE_CUDA(cudaMemcpyAsync(coef, pt, words * 8, cudaMemcpyDeviceToDevice, s));
-    if (he_status r = ntt_launch(uniform_launch(coef, level + 1, count, ctx->tables), ctx->log_n, true, s)) return r;
+    he::NttLaunch L = uniform_launch(coef, level + 1, count, ctx->tables);
+    L.src = pt;
+    if (he_status r = ntt_launch(L, ctx->log_n, true, s)) return r;
     if (he_status r = crt_compose(enc, m, coef, count, level, s)) return r;
     he::FftArgs a = fft_args(enc, count, level + 1, 1.0 / scale);
     a.m_in = m;

@@ -42,8 +42,8 @@ __device__ __forceinline__ void tma_store_rows(const u64 (&x)[16], u32 wbase, co
     __syncwarp();
 }
 
-// Forward or inverse transform of one limb stored at `data` (in place). The
-// forward transform's last round and the inverse transform's first round
+// Forward or inverse transform of one limb stored at `data` (in place; the
+// inverse reads its input at `src`, which may be another buffer). The forward transform's last round and the inverse transform's first round
 // give each thread runs of consecutive words, which move as 32-byte quarters
 // (streaming cache hints: every word is read and written once per launch);
 // the cross-CTA columns move as single coalesced words. Stores are skipped
@@ -53,8 +53,8 @@ __device__ __forceinline__ void tma_store_rows(const u64 (&x)[16], u32 wbase, co
 // shared memory are 1024-byte aligned (the swizzle's period).
 template <class Sh, bool INV>
 __device__ __forceinline__ void ntt_limb(u64 *smem, u32 m, u32 rbase, u64 *data, const ulonglong2 *tw,
-                                         const PrimeConst &pc, bool valid = true, const CUtensorMap *tm = nullptr,
-                                         u32 row0 = 0)
+                                         const PrimeConst &pc, const u64 *src, bool valid = true,
+                                         const CUtensorMap *tm = nullptr, u32 row0 = 0)
 {
     u64 x[Sh::E];
     const u32 tid = threadIdx.x;
@@ -77,7 +77,7 @@ __device__ __forceinline__ void ntt_limb(u64 *smem, u32 m, u32 rbase, u64 *data,
     } else {
 #pragma unroll
         for (int e = 0; e < Sh::E; e += 4)
-            ld4_cs(data + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+            ld4_cs(src + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
         auto nold = [&](u32) -> u64 { return 0; };
         auto st = [&](int P, u64 v) {
             if (valid) __stcs(reinterpret_cast<unsigned long long *>(data + P), (unsigned long long)v);
@@ -111,7 +111,7 @@ template <class Sh>
 __device__ __forceinline__ void prefetch_limb_block(const NttLaunch &a, u32 item, u32 m)
 {
     if (threadIdx.x != 0 || item >= a.items) return;
-    const u64 *p = a.jobs ? a.jobs[item].data : a.base + (size_t)item * Sh::N;
+    const u64 *p = a.jobs ? a.jobs[item].data : (a.src ? a.src : a.base) + (size_t)item * Sh::N;
     asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p + (size_t)m * Sh::B), "r"(Sh::B * 8u)
                  : "memory");
 }
@@ -134,9 +134,10 @@ k_ntt(const __grid_constant__ NttLaunch a)   // grid constant: tmap is addressed
     resolve_item<Sh, INV>(a, item, data, tw, pcp);
     const PrimeConst pc = *pcp;
     if (!INV && a.tma_store)
-        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc, true, &a.tmap, (u32)(((size_t)item * Sh::N + m * Sh::B) >> 4));
+        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc, data, true, &a.tmap,
+                          (u32)(((size_t)item * Sh::N + m * Sh::B) >> 4));
     else
-        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc);
+        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc, a.src ? a.src + (size_t)item * Sh::N : data);
 }
 
 // Persistent form: a fixed grid of clusters walks the limbs (job list or
@@ -159,7 +160,7 @@ k_ntt_persistent(NttLaunch a)
         const PrimeConst *pcp;
         resolve_item<Sh, INV>(a, item, data, tw, pcp);
         const PrimeConst pc = *pcp;
-        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc);
+        ntt_limb<Sh, INV>(smem, m, 0, data, tw, pc, a.src ? a.src + (size_t)item * Sh::N : data);
     }
 }
 
@@ -180,14 +181,14 @@ __device__ __noinline__ void mixed_unit(u64 *smem, u32 rank, const MixedUnit &un
         // the whole cluster transforms the unit's one limb
         const LimbJob j = jobs[un.first_job];
         const PrimeConst pc = *j.pc;
-        ntt_limb<Sh, INV>(smem, rank, 0, j.data, INV ? j.tw_inv : j.tw_fwd, pc);
+        ntt_limb<Sh, INV>(smem, rank, 0, j.data, INV ? j.tw_inv : j.tw_fwd, pc, j.data);
     } else if constexpr (Sh::LOG_C == 0) {
         // one CTA per limb and no cluster barrier inside the transform: a
         // CTA without a limb has nothing to do
         if (rank >= un.n_jobs) return;
         const LimbJob j = jobs[un.first_job + rank];
         const PrimeConst pc = *j.pc;
-        ntt_limb<Sh, INV>(smem, 0, 0, j.data, INV ? j.tw_inv : j.tw_fwd, pc);
+        ntt_limb<Sh, INV>(smem, 0, 0, j.data, INV ? j.tw_inv : j.tw_fwd, pc, j.data);
     } else {
         const u32 sub = rank >> Sh::LOG_C;
         const u32 m = rank & (Sh::C - 1);
@@ -195,7 +196,7 @@ __device__ __noinline__ void mixed_unit(u64 *smem, u32 rank, const MixedUnit &un
         const bool valid = sub < un.n_jobs;
         const LimbJob j = jobs[un.first_job + (valid ? sub : 0u)];
         const PrimeConst pc = *j.pc;
-        ntt_limb<Sh, INV>(smem, m, rbase, j.data, INV ? j.tw_inv : j.tw_fwd, pc, valid);
+        ntt_limb<Sh, INV>(smem, m, rbase, j.data, INV ? j.tw_inv : j.tw_fwd, pc, j.data, valid);
     }
 }
 

@@ -25,8 +25,11 @@ struct LimbJob {
 // tma_store: the forward transform writes its output with bulk tensor
 // stores through tmap, the batch viewed as rows of 16 words (128 bytes),
 // boxes of 32 rows, 128-byte swizzle (uniform batches, 16 words a thread).
+// src: the inverse transform reads its input there instead (same layout,
+// null: in place).
 struct NttLaunch {
     u64 *base;
+    const u64 *src;
     u32 limbs;
     u32 first_prime;
     u32 items;
@@ -218,7 +221,7 @@ cudaError_t launch_encode_fft(const FftArgs &a, cudaStream_t s);
 cudaError_t launch_decode_fft(const FftArgs &a, cudaStream_t s);
 // Words of the CRT kernel's multi-word integers for `need` words (0: too many).
 u32 crt_words(u32 need);
-cudaError_t launch_crt_compose(double *out, const u64 *coef, const u64 *tab, u32 nw, u32 log_N, u32 limbs, u64 total,
-                               u32 blocks, cudaStream_t s);
+cudaError_t launch_crt_compose(double *out, const u64 *coef, const u64 *tab, const u64 *primes, u32 nw, u32 log_N,
+                               u32 limbs, u64 total, u32 blocks, cudaStream_t s);
 
 }  // namespace he
