@@ -903,10 +903,13 @@ static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64
 {
     const u32 n = a.n;
     const size_t per = (size_t)(n + 1) * n * ctx->N;
-    const u32 group = (u32)std::min<size_t>({(size_t)kModupGroup, (size_t)count, xbuf ? x_words / per : 0});
-    *special_ntt = group > 0;
-    if (group == 0) return run_eval(ctx, he::EK_KS_MODUP, a, count * (n + 1), s);
+    const u32 fit = (u32)std::min<size_t>({(size_t)kModupGroup, (size_t)count, xbuf ? x_words / per : 0});
+    *special_ntt = fit > 0;
+    if (fit == 0) return run_eval(ctx, he::EK_KS_MODUP, a, count * (n + 1), s);
     a.mx = xbuf;
+    // as many groups as the buffer asks for, of nearly equal size: 80
+    // ciphertexts as 64 + 16 leave a second pair of launches half empty
+    const u32 groups = (count + fit - 1) / fit, group = (count + groups - 1) / groups;
     for (u32 c0 = 0; c0 < count; c0 += group) {
         const u32 gs = std::min(group, count - c0);
         a.c_first = c0;
@@ -1256,9 +1259,16 @@ extern "C" he_status he_ct_matmul_tensor(uint64_t *t_out, const uint64_t *a, con
     if (m == 0 || k == 0 || n == 0) return fail(HE_EINVAL, "matrix dimensions must be positive");
     if ((u64)m * n * 3 * (level + 1) * ctx->N >= (1ull << 40)) return fail(HE_EINVAL, "matrix product too large");
     const u32 limbs = level + 1;
-    const u64 threads = (u64)m * ((n + he::MM_TJ - 1) / he::MM_TJ) * limbs * (ctx->N / 2);
-    he::k_ct_matmul_tensor<<<stream_grid(threads, 256), 256, 0, (cudaStream_t)stream>>>(
-        t_out, a, b, m, k, n, (u32)ctx->log_n, limbs, ctx->tables->d_pc);
+    // 2 x 2 outputs a warp; a single row or column would leave half of them idle
+    auto launch = [&](auto kernel, u32 ti, u32 tj) {
+        const u64 warps = (u64)((m + ti - 1) / ti) * ((n + tj - 1) / tj) * limbs * (ctx->N / 32);
+        kernel<<<(u32)((warps + 3) / 4), 128, 0, (cudaStream_t)stream>>>(
+            t_out, a, b, m, k, n, (u32)ctx->log_n, limbs, warps, ctx->tables->d_pc, ctx->d_limb);
+    };
+    if (m > 1 && n > 1) launch(he::k_ct_matmul_tensor<2, 2>, 2, 2);
+    else if (m > 1) launch(he::k_ct_matmul_tensor<2, 1>, 2, 1);
+    else if (n > 1) launch(he::k_ct_matmul_tensor<1, 2>, 1, 2);
+    else launch(he::k_ct_matmul_tensor<1, 1>, 1, 1);
     HE_CUDA(cudaGetLastError());
     return HE_OK;
 }

@@ -11,6 +11,9 @@ namespace he {
 
 // ============================================================ plain NTT ====
 
+// Read-only load (the kernel never writes what it reads through this).
+__device__ __forceinline__ u64 rd(const u64 *p) { return __ldg(reinterpret_cast<const unsigned long long *>(p)); }
+
 // Bulk tensor store of the forward transform's output (one warp, 16 words
 // a thread: thread l of warp w holds the 16 words of row row0 + 32 w + l of
 // the tensor map's view, rows of 128 bytes). The warp's rows of the shared
@@ -412,117 +415,95 @@ __global__ void k_ct_automorph(u64 *out, const u64 *in, u64 words, u32 log_n, u3
 // ============================================ encrypted matrix product ======
 // Tensor part of C += A B (Sec. IV-E matMul_mxnxk; Sec. II-A Mul): for each
 // limb and position, T[i][j] = sum_l (a0 b0, a0 b1 + a1 b0, a1 b1) over the
-// pairs (A[i][l], B[l][j]) mod q. For q >= 2^32 the 128-bit products are
-// summed without reduction (a0 b1 + a1 b0 included: the fused
-// multiply-add of Sec. III-A-1 carried over the whole sum) and reduced once
-// per 32 terms; smaller moduli reduce every term (Barrett, one reduction for
-// a0 b1 + a1 b0). A thread owns one limb, two positions, row i and MM_TJ
-// consecutive output columns, so each A word it loads serves MM_TJ products;
-// consecutive threads take consecutive positions (coalesced 16-byte loads).
-constexpr u32 MM_TJ = 2;
+// pairs (A[i][l], B[l][j]) mod q. The three sums of an output are 128-bit
+// integers (Sum128) over MM_TERMS terms, the middle one as
+// sum (a0 + a1)(b0 + b1) - sum a0 b0 - sum a1 b1 (three products a term
+// instead of four; (2^61)^2 32 = 2^127), each reduced once (Montgomery, its
+// 2^-64 taken off by a Shoup product with 2^64).
+//
+// A warp owns 32 positions of one limb and a TI x TJ block of outputs, so a
+// term's 2 (TI + TJ) words, loaded as coalesced 256-byte rows, serve TI TJ
+// outputs; the four warps of a CTA take neighbouring blocks of the same
+// positions and find each other's rows in L1. 84 registers of sums at 2 x 2,
+// 168 in all, three CTAs an SM. Measured, 10 x 9 x 8 at N = 2^13, 3 limbs: 118
+// us with two columns and two positions a thread and compiled 128-bit sums, 75
+// now (the products alone fill the multiply pipe for 26 us); 2 x 1 outputs a
+// warp 85, 1 x 2 94, 2 x 2 at two or four CTAs an SM 77 and 80; 32 x 32 x 32
+// 4.7 -> 2.1 ms.
+constexpr u32 MM_TERMS = 32;
 
-// (h, lo) += a b as a 128-bit sum.
-__device__ __forceinline__ void mac128(u64 &h, u64 &lo, u64 a, u64 b)
+template <int TI, int TJ>
+__global__ void __launch_bounds__(128, TI * TJ == 4 ? 3 : 4)
+k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 log_n, u32 limbs, u64 warps,
+                   const PrimeConst *pcs, const LimbConst *lcs)
 {
-    const u64 pl = a * b, ph = __umul64hi(a, b);
-    lo += pl;
-    h += ph + (lo < pl ? 1 : 0);
-}
-
-__global__ void k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 log_n, u32 limbs,
-                                   const PrimeConst *pcs)
-{
-    const u32 half = 1u << (log_n - 1);
-    const u32 jt_count = (n + MM_TJ - 1) / MM_TJ;
+    const u64 w = (u64)blockIdx.x * 4 + __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);   // uniform over the warp
+    if (w >= warps) return;
+    const u32 jt = (n + TJ - 1) / TJ, tiles = (m + TI - 1) / TI * jt;
+    const u32 tile = (u32)(w % tiles), i0 = tile / jt * TI, j0 = tile % jt * TJ;
+    const u64 pos = w / tiles * 32 + (threadIdx.x & 31);    // limb N + position
+    const u32 limb = (u32)(pos >> log_n);
     const size_t poly = (size_t)limbs << log_n;             // words per component
-    const u64 total = (u64)m * jt_count * limbs * half;
-    for (u64 q = (u64)blockIdx.x * blockDim.x + threadIdx.x; q < total; q += (u64)gridDim.x * blockDim.x) {
-        const u32 P = (u32)(q % half) * 2;
-        const u32 limb = (u32)((q / half) % limbs);
-        const u32 jt = (u32)((q / ((u64)half * limbs)) % jt_count);
-        const u32 i = (u32)(q / ((u64)half * limbs * jt_count));
-        const PrimeConst pc = pcs[limb];
-        const size_t off = ((size_t)limb << log_n) + P;
-        u64 acc[MM_TJ][3][2];
+    const PrimeConst pc = pcs[limb];
+    const u64 R = lcs[limb].R, R_sh = lcs[limb].R_sh;
+    // rows and columns beyond the edge repeat the last one; they are not stored
+    const u64 *ap[TI], *bp[TJ];
 #pragma unroll
-        for (u32 jj = 0; jj < MM_TJ; jj++)
+    for (int i = 0; i < TI; i++) ap[i] = a + (size_t)min(i0 + i, m - 1) * k * 2 * poly + pos;
 #pragma unroll
-            for (int c = 0; c < 3; c++) acc[jj][c][0] = acc[jj][c][1] = 0;
-        if (pc.p >= (1ull << 32)) {
-            // lazy: 128-bit sums of up to 64 products (< 2^126), reduced per
-            // chunk of 32 terms: hi mod p, then hi 2^64 + lo = hi c64 + lo
-            const u64 c64 = barrett_reduce(1, 0, pc.p, pc.mu, pc.bits);   // 2^64 mod p
-            for (u32 l0 = 0; l0 < k; l0 += 32) {
-                u64 h[MM_TJ][3][2], lo[MM_TJ][3][2];
+    for (int j = 0; j < TJ; j++) bp[j] = b + (size_t)min(j0 + j, n - 1) * 2 * poly + pos;
+    const size_t bstep = (size_t)n * 2 * poly;
+    for (u32 l0 = 0; l0 < k; l0 += MM_TERMS) {
+        Sum128 s[TI][TJ][3];
 #pragma unroll
-                for (u32 jj = 0; jj < MM_TJ; jj++)
+        for (int i = 0; i < TI; i++)
 #pragma unroll
-                    for (int c = 0; c < 3; c++) h[jj][c][0] = h[jj][c][1] = lo[jj][c][0] = lo[jj][c][1] = 0;
-                const u32 l1 = min(k, l0 + 32);
-                for (u32 l = l0; l < l1; l++) {
-                    const u64 *ap = a + ((size_t)i * k + l) * 2 * poly + off;
-                    const ulonglong2 a0 = __ldg(reinterpret_cast<const ulonglong2 *>(ap));
-                    const ulonglong2 a1 = __ldg(reinterpret_cast<const ulonglong2 *>(ap + poly));
+            for (int j = 0; j < TJ; j++)
 #pragma unroll
-                    for (u32 jj = 0; jj < MM_TJ; jj++) {
-                        const u32 j = jt * MM_TJ + jj;
-                        if (j >= n) break;
-                        const u64 *bp = b + ((size_t)l * n + j) * 2 * poly + off;
-                        const ulonglong2 b0 = __ldg(reinterpret_cast<const ulonglong2 *>(bp));
-                        const ulonglong2 b1 = __ldg(reinterpret_cast<const ulonglong2 *>(bp + poly));
-                        mac128(h[jj][0][0], lo[jj][0][0], a0.x, b0.x);
-                        mac128(h[jj][0][1], lo[jj][0][1], a0.y, b0.y);
-                        mac128(h[jj][1][0], lo[jj][1][0], a0.x, b1.x);
-                        mac128(h[jj][1][0], lo[jj][1][0], a1.x, b0.x);
-                        mac128(h[jj][1][1], lo[jj][1][1], a0.y, b1.y);
-                        mac128(h[jj][1][1], lo[jj][1][1], a1.y, b0.y);
-                        mac128(h[jj][2][0], lo[jj][2][0], a1.x, b1.x);
-                        mac128(h[jj][2][1], lo[jj][2][1], a1.y, b1.y);
-                    }
+                for (int c = 0; c < 3; c++) s[i][j][c].clear();
+        const u32 l1 = min(k, l0 + MM_TERMS);
+        for (u32 l = l0; l < l1; l++) {
+            u64 a0[TI], a1[TI], b0[TJ], b1[TJ];
+#pragma unroll
+            for (int i = 0; i < TI; i++) a0[i] = rd(ap[i]), a1[i] = rd(ap[i] + poly), ap[i] += 2 * poly;
+#pragma unroll
+            for (int j = 0; j < TJ; j++) b0[j] = rd(bp[j]), b1[j] = rd(bp[j] + poly), bp[j] += bstep;
+#pragma unroll
+            for (int i = 0; i < TI; i++)
+#pragma unroll
+                for (int j = 0; j < TJ; j++) {
+                    s[i][j][0].mac(a0[i], b0[j]);
+                    s[i][j][2].mac(a1[i], b1[j]);
                 }
 #pragma unroll
-                for (u32 jj = 0; jj < MM_TJ; jj++)
+            for (int i = 0; i < TI; i++) a0[i] += a1[i];
 #pragma unroll
-                    for (int c = 0; c < 3; c++)
+            for (int j = 0; j < TJ; j++) b0[j] += b1[j];
 #pragma unroll
-                        for (int x = 0; x < 2; x++) {
-                            const u64 r1 = barrett_reduce(0, h[jj][c][x], pc.p, pc.mu, pc.bits);
-                            u64 zh, zl;
-                            mul_wide(r1, c64, zh, zl);
-                            zl += lo[jj][c][x];
-                            zh += (zl < lo[jj][c][x]) ? 1 : 0;
-                            acc[jj][c][x] = add_mod(acc[jj][c][x], barrett_reduce(zh, zl, pc.p, pc.mu, pc.bits), pc.p);
-                        }
-            }
-        } else
-        for (u32 l = 0; l < k; l++) {
-            const u64 *ap = a + ((size_t)i * k + l) * 2 * poly + off;
-            const ulonglong2 a0 = __ldg(reinterpret_cast<const ulonglong2 *>(ap));
-            const ulonglong2 a1 = __ldg(reinterpret_cast<const ulonglong2 *>(ap + poly));
+            for (int i = 0; i < TI; i++)
 #pragma unroll
-            for (u32 jj = 0; jj < MM_TJ; jj++) {
-                const u32 j = jt * MM_TJ + jj;
-                if (j >= n) break;
-                const u64 *bp = b + ((size_t)l * n + j) * 2 * poly + off;
-                const ulonglong2 b0 = __ldg(reinterpret_cast<const ulonglong2 *>(bp));
-                const ulonglong2 b1 = __ldg(reinterpret_cast<const ulonglong2 *>(bp + poly));
-                acc[jj][0][0] = add_mod(acc[jj][0][0], mul_mod(a0.x, b0.x, pc), pc.p);
-                acc[jj][0][1] = add_mod(acc[jj][0][1], mul_mod(a0.y, b0.y, pc), pc.p);
-                acc[jj][1][0] = add_mod(acc[jj][1][0], mad2_mod(a0.x, b1.x, a1.x, b0.x, pc), pc.p);
-                acc[jj][1][1] = add_mod(acc[jj][1][1], mad2_mod(a0.y, b1.y, a1.y, b0.y, pc), pc.p);
-                acc[jj][2][0] = add_mod(acc[jj][2][0], mul_mod(a1.x, b1.x, pc), pc.p);
-                acc[jj][2][1] = add_mod(acc[jj][2][1], mul_mod(a1.y, b1.y, pc), pc.p);
-            }
+                for (int j = 0; j < TJ; j++) s[i][j][1].mac(a0[i], b0[j]);
         }
 #pragma unroll
-        for (u32 jj = 0; jj < MM_TJ; jj++) {
-            const u32 j = jt * MM_TJ + jj;
-            if (j >= n) break;
-            u64 *tp = t + ((size_t)i * n + j) * 3 * poly + off;
+        for (int i = 0; i < TI; i++)
 #pragma unroll
-            for (int c = 0; c < 3; c++)
-                *reinterpret_cast<ulonglong2 *>(tp + c * poly) = make_ulonglong2(acc[jj][c][0], acc[jj][c][1]);
-        }
+            for (int j = 0; j < TJ; j++) {
+                if (i0 + i >= m || j0 + j >= n) continue;
+                u64 h[3], lo[3];
+#pragma unroll
+                for (int c = 0; c < 3; c++) s[i][j][c].total(h[c], lo[c]);
+#pragma unroll
+                for (int c = 0; c < 3; c += 2)
+                    asm("sub.cc.u64 %0, %0, %2;\n\tsubc.u64 %1, %1, %3;"
+                        : "+l"(lo[1]), "+l"(h[1]) : "l"(lo[c]), "l"(h[c]));
+                u64 *tp = t + ((size_t)(i0 + i) * n + j0 + j) * 3 * poly + pos;
+#pragma unroll
+                for (int c = 0; c < 3; c++) {
+                    u64 v = mul_shoup(montgomery_reduce(h[c], lo[c], pc), R, R_sh, pc.p);
+                    if (l0) v = add_mod(v, tp[c * poly], pc.p);   // the terms before
+                    tp[c * poly] = v;
+                }
+            }
     }
 }
 
@@ -678,9 +659,6 @@ __device__ __forceinline__ void store_run(u64 *dst, const u64 (&x)[Sh::E], u32 m
 #pragma unroll
     for (int e = 0; e < Sh::E; e += 4) st4(dst + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
 }
-
-// Read-only load (the kernel never writes what it reads through this).
-__device__ __forceinline__ u64 rd(const u64 *p) { return __ldg(reinterpret_cast<const unsigned long long *>(p)); }
 
 // d_k[i] at position P for component k (0 or 1): from the tensor of the two
 // input ciphertexts (fused Mul) or from a 3-component input.

@@ -244,6 +244,13 @@ __device__ __forceinline__ u64 mad2_mod(u64 a0, u64 b1, u64 a1, u64 b0, const Pr
     return barrett_reduce(hi, lo, c.p, c.mu, c.bits);
 }
 
+// Montgomery reduction: hi 2^64 + lo times 2^-64 mod p, in [0, hi + p].
+__device__ __forceinline__ u64 montgomery_reduce(u64 hi, u64 lo, const PrimeConst &c)
+{
+    // lo + (m p mod 2^64) is 0 or 2^64: a carry unless lo = 0
+    return hi + __umul64hi(lo * c.mneg, c.p) + (lo ? 1u : 0u);
+}
+
 // A 128-bit sum of 64 x 64-bit products that is reduced once at the end.
 // The four 32 x 32 partial products of a term go to two interleaved columns,
 // e = words 0..3 (x0 w0, x1 w1) and o = words 1..3 (x0 w1, x1 w0), so that
@@ -270,8 +277,7 @@ struct Sum128 {
             : "+r"(e0), "+r"(e1), "+r"(e2), "+r"(e3), "+r"(o0), "+r"(o1), "+r"(o2)
             : "r"((u32)x), "r"((u32)(x >> 32)), "r"((u32)w), "r"((u32)(w >> 32)));
     }
-    // Montgomery reduction: the sum times 2^-64 mod p, in [0, sum / 2^64 + p)
-    __device__ __forceinline__ u64 redc(const PrimeConst &c) const
+    __device__ __forceinline__ void total(u64 &hi, u64 &lo) const
     {
         u32 s1, s2, s3;
         asm("add.cc.u32 %0, %3, %6;\n\t"
@@ -279,9 +285,14 @@ struct Sum128 {
             "addc.u32 %2, %5, %8;"
             : "=&r"(s1), "=&r"(s2), "=r"(s3)
             : "r"(e1), "r"(e2), "r"(e3), "r"(o0), "r"(o1), "r"(o2));
-        const u64 lo = ((u64)s1 << 32) | e0, hi = ((u64)s3 << 32) | s2;
-        // lo + (m p mod 2^64) is 0 or 2^64: a carry unless lo = 0
-        return hi + __umul64hi(lo * c.mneg, c.p) + (lo ? 1u : 0u);
+        lo = ((u64)s1 << 32) | e0;
+        hi = ((u64)s3 << 32) | s2;
+    }
+    __device__ __forceinline__ u64 redc(const PrimeConst &c) const
+    {
+        u64 hi, lo;
+        total(hi, lo);
+        return montgomery_reduce(hi, lo, c);
     }
 };
 
