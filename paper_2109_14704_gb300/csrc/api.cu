@@ -401,6 +401,43 @@ extern "C" he_status he_ntt_set_shape(uint32_t N, uint32_t direction, uint32_t l
     return HE_OK;
 }
 
+static int g_num_sms = 0;
+
+static int num_sms()
+{
+    if (!g_num_sms) {
+        int dev = 0;
+        cudaGetDevice(&dev);
+        if (cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) g_num_sms = 152;
+    }
+    return g_num_sms;
+}
+
+// Batches of at most this many words take the radix-8 shapes: 8 words a thread
+// put twice the threads on the batch and halve each one's chain of butterflies,
+// which is what a launch costs that does not fill the GPU (512 threads an SM);
+// above it the 16-word shapes' fewer exchanges win. Measured, 60-bit prime,
+// forward, 16 / 8 words a thread: one limb of 2^12 8.5 / 7.0 us, of 2^15 11.3 /
+// 9.4; 2^19 words in all 8.9 / 7.2 (2^12), 14.8 / 14.5 (2^15); 2^20 words 11.6 /
+// 11.7 and 16.7 / 15.5; 2^21 words 19.9 / 20.9 and 25.6 / 32.2.
+static u64 small_batch_words() { return (u64)num_sms() * 4096; }
+
+// Shape of a batch of `items` limbs when none is set for the degree.
+//   2^10 .. 2^15, small batch: one block of 8-word threads where the degree fits
+//     it, 2^12-word blocks above; 2^13 in four 2^11-word blocks of 16-word
+//     threads while those leave SMs idle (inverse 8.1 us against 8.7).
+//   2^16: 2^12-word blocks in clusters of 16 at every size (one limb 12.2 us
+//     against 17.3 with 2^13-word blocks, 128 limbs 101 against 117).
+static void auto_shape(int log_n, u32 items, int *lb, int *le)
+{
+    if (log_n == 16) {
+        *lb = 12, *le = 4;
+    } else if (((u64)items << log_n) <= small_batch_words()) {
+        if (log_n == 13 && items * 4 <= (u32)num_sms()) *lb = 11, *le = 4;
+        else *lb = std::min(log_n, 12), *le = 3;
+    }
+}
+
 // One launch of a batch of limb transforms in the shape set for the degree.
 // cuTensorMapEncodeTiled, fetched through the runtime's driver entry points
 // (the library does not link the driver library); null if unavailable.
@@ -447,7 +484,9 @@ static bool batch_tmap(he::NttLaunch &a, u32 N)
 static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaStream_t stream)
 {
     const he::DegreeOps *ops = he::degree_ops(log_n);
-    const int lb = g_shape_b[inv][log_n].load(), le = g_shape_e[inv][log_n].load();
+    int lb = g_shape_b[inv][log_n].load(), le = g_shape_e[inv][log_n].load();
+    const bool persistent = g_shape_persistent[inv][log_n].load() != 0;
+    if (!lb && !le && !persistent) auto_shape(log_n, a0.items, &lb, &le);
     he::NttLaunch a = a0;
     const u32 resident = (u32)std::max(ops->max_clusters(lb, le, inv), 1);
 #ifndef HE_NO_L2_PREFETCH
@@ -455,10 +494,14 @@ static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaSt
 #else
     a.prefetch = 0;
 #endif
-    if (g_shape_persistent[inv][log_n].load()) {
+    if (persistent) {
         HE_CUDA(ops->ntt_persistent(a, lb, le, inv, std::min<u32>(a.items, resident), stream));
     } else {
-        a.tma_store = (!inv && le == 4 && batch_tmap(a, 1u << log_n)) ? 1u : 0u;
+        // le = 0: the degree's default, 16 words a thread; from 32 MB on, where
+        // the 2 % they give (2477 -> 2425 us for 8192 limbs of 2^15) is more than
+        // the host's time to encode the tensor map
+        const bool tma = !inv && (le == 4 || (le == 0 && ((u64)a.items << log_n) >= (1u << 22)));
+        a.tma_store = (tma && batch_tmap(a, 1u << log_n)) ? 1u : 0u;
         HE_CUDA(ops->ntt(a, lb, le, inv, stream));
     }
     return HE_OK;
@@ -521,18 +564,6 @@ extern "C" he_status he_ntt_inv_naive(uint64_t *poly, uint32_t N, uint32_t limbs
     return naive_common(poly, N, limbs, count, moduli_host, tw, stream, true);
 }
 
-static int g_num_sms = 0;
-
-static int num_sms()
-{
-    if (!g_num_sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        if (cudaDeviceGetAttribute(&g_num_sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess) g_num_sms = 152;
-    }
-    return g_num_sms;
-}
-
 static u32 stream_grid(u64 work_items, u32 threads)
 {
     const u64 want = (work_items + threads - 1) / threads;
@@ -582,8 +613,9 @@ extern "C" he_status he_negacyclic_mul(uint64_t *c, const uint64_t *a, const uin
     L.tw_fwd = tw->d_fwd;
     L.tw_inv = tw->d_inv;
     L.pc = tw->d_pc;
-    HE_CUDA(he::degree_ops(log_n)->negacyclic(L, g_shape_b[0][log_n].load(), g_shape_e[0][log_n].load(),
-                                              (cudaStream_t)stream));
+    int lb = g_shape_b[0][log_n].load(), le = g_shape_e[0][log_n].load();
+    if (!lb && !le) auto_shape(log_n, (u32)items, &lb, &le);
+    HE_CUDA(he::degree_ops(log_n)->negacyclic(L, lb, le, (cudaStream_t)stream));
     return HE_OK;
 }
 
@@ -600,7 +632,7 @@ struct he_context {
     he::DropConst *d_drop = nullptr;
     he::PrimeConst *d_pc_lift = nullptr;
     u64 R_special = 0;                 // 2^64 mod P
-    std::atomic<int> eval_log_e{4};    // words per thread of the evaluation kernels
+    std::atomic<int> eval_log_e{0};    // log2 words per thread of the evaluation kernels (0: by the stage's size)
 };
 
 struct he_relin_key {
@@ -693,7 +725,7 @@ extern "C" he_status he_context_set_eval_shape(he_context *ctx, uint32_t log_thr
     if (!ctx) return fail(HE_EINVAL, "context is NULL");
     if (log_thread_words != 0 && log_thread_words != 3 && log_thread_words != 4)
         return fail(HE_EUNSUPPORTED, "evaluation kernels are built with 2^3 or 2^4 words per thread");
-    ctx->eval_log_e.store(log_thread_words ? (int)log_thread_words : 4);
+    ctx->eval_log_e.store((int)log_thread_words);
     return HE_OK;
 }
 
@@ -839,7 +871,12 @@ static he_status run_eval(const he_context *ctx, he::EvalKernel k, const he::Eva
                           cudaStream_t s, const he::JobTable *jobs = nullptr)
 {
     if (!items) return HE_OK;
-    HE_CUDA(he::degree_ops(ctx->log_n)->eval(k, a, items, ctx->eval_log_e.load(), jobs, s));
+    // unset: 8 words a thread up to twice the transforms' limit (the stages load
+    // and finish more per word): one product at 2^14, 7 + 1 primes 69 -> 57 us,
+    // four 98 -> 97, from eight on the same within 1 %
+    int log_e = ctx->eval_log_e.load();
+    if (!log_e) log_e = ((u64)items << ctx->log_n) <= 2 * small_batch_words() ? 3 : 4;
+    HE_CUDA(he::degree_ops(ctx->log_n)->eval(k, a, items, log_e, jobs, s));
     return HE_OK;
 }
 
