@@ -50,6 +50,7 @@ __device__ __forceinline__ double2 c_conj_if(double2 a, bool c) { return c ? mak
 template <int MODE, int PASS>
 __global__ void __launch_bounds__(kFftThreads) k_fft_pass(FftArgs a)
 {
+    stream_order();
     extern __shared__ double2 sm[];
     const u32 n = 1u << a.log_n;
     const u32 log_L = PASS == 0 ? a.log_n1 : a.log_n - a.log_n1;
@@ -284,6 +285,7 @@ template <int NW>
 __global__ void __launch_bounds__(128) k_crt_compose(double *out, const u64 *coef, const u64 *tab, const u64 *primes,
                                                      u32 log_N, u32 limbs, u64 total)
 {
+    stream_order();
     const u64 *Q = tab, *Qh = tab + NW, *Qhat = tab + 2 * NW, *pr = tab + (2 + limbs) * NW;
     const double inv_qtop = __longlong_as_double((long long)pr[3 * limbs]);
     const u64 N = 1ull << log_N;
@@ -350,9 +352,9 @@ template <int MODE>
 static cudaError_t fft_two_pass(const FftArgs &a, cudaStream_t s)
 {
     const u32 lA = a.log_n1, lB = a.log_n - a.log_n1;
-    k_fft_pass<MODE, 0><<<fft_blocks(a, lA), kFftThreads, fft_smem(lA), s>>>(a);
-    k_fft_pass<MODE, 1><<<fft_blocks(a, lB), kFftThreads, fft_smem(lB), s>>>(a);
-    return cudaGetLastError();
+    if (cudaError_t e = launch_k(k_fft_pass<MODE, 0>, fft_blocks(a, lA), kFftThreads, (u32)fft_smem(lA), 1, s, a)) return e;
+    if (cudaError_t e = launch_k(k_fft_pass<MODE, 1>, fft_blocks(a, lB), kFftThreads, (u32)fft_smem(lB), 1, s, a)) return e;
+    return cudaSuccess;
 }
 
 cudaError_t launch_encode_fft(const FftArgs &a, cudaStream_t s) { return fft_two_pass<0>(a, s); }
@@ -370,8 +372,7 @@ cudaError_t launch_crt_compose(double *out, const u64 *coef, const u64 *tab, con
     switch (nw) {
 #define HE_CRT_CASE(w)                                                                   \
     case (w):                                                                            \
-        k_crt_compose<(w)><<<blocks, 128, 0, s>>>(out, coef, tab, primes, log_N, limbs, total); \
-        return cudaGetLastError();
+        return launch_k(k_crt_compose<(w)>, blocks, 128, 0, 1, s, out, coef, tab, primes, log_N, limbs, total);
         HE_CRT_NW(HE_CRT_CASE)
 #undef HE_CRT_CASE
     default:

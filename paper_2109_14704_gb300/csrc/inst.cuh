@@ -9,28 +9,6 @@
 
 namespace he {
 
-template <class K, class... Args>
-static cudaError_t launch_k(K kernel, u32 grid, u32 block, u32 smem, u32 cluster, cudaStream_t s,
-                            Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid, 1, 1);
-    cfg.blockDim = dim3(block, 1, 1);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    cfg.numAttrs = 0;
-    if (cluster > 1) {
-        attr[0].id = cudaLaunchAttributeClusterDimension;
-        attr[0].val.clusterDim.x = cluster;
-        attr[0].val.clusterDim.y = 1;
-        attr[0].val.clusterDim.z = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-    }
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
-}
-
 // Raise the dynamic shared-memory limit of a kernel once per process, and
 // allow its launch in clusters of more than 8 CTAs (the non-portable size,
 // up to 16 on this GPU) where the shape needs it.

@@ -11,8 +11,9 @@ namespace he {
 
 // ============================================================ plain NTT ====
 
-// Read-only load (the kernel never writes what it reads through this).
-__device__ __forceinline__ u64 rd(const u64 *p) { return __ldg(reinterpret_cast<const unsigned long long *>(p)); }
+// Load of a word the kernel does not write (a kernel ahead in the stream may
+// have: see stream_order).
+__device__ __forceinline__ u64 rd(const u64 *p) { return *p; }
 
 // Bulk tensor store of the forward transform's output (one warp, 16 words
 // a thread: thread l of warp w holds the 16 words of row row0 + 32 w + l of
@@ -126,6 +127,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool INV, int OCC = 0>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E, OCC>::MIN_CTAS)
 k_ntt(const __grid_constant__ NttLaunch a)   // grid constant: tmap is addressed in place
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(1024) u64 smem[];
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -149,6 +151,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool INV, int OCC = 0>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E, OCC>::MIN_CTAS)
 k_ntt_persistent(NttLaunch a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -206,6 +209,7 @@ __device__ __noinline__ void mixed_unit(u64 *smem, u32 rank, const MixedUnit &un
 template <bool INV>
 __global__ void __launch_bounds__(256, 4) k_ntt_mixed(const MixedUnit *units, u32 n_units, const LimbJob *jobs)
 {
+    stream_order();
     extern __shared__ __align__(16) u64 smem[];
     const u32 rank = cluster_ctarank();
     const u32 clusters = gridDim.x >> 3;
@@ -236,6 +240,7 @@ template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::NEGA_MIN_CTAS)
 k_negacyclic(NegaLaunch a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     u64 *park = smem + Sh::B;                    // [E][T]
@@ -294,6 +299,7 @@ __device__ __forceinline__ u32 automorph_index(u32 i, u32 log_n, u32 g)
 
 __global__ void k_ntt_naive_stage(NttLaunch a, u32 log_n, u32 S, bool inv)
 {
+    stream_order();
     const u32 N = 1u << log_n;
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     const size_t total = (size_t)a.items * (N / 2);
@@ -322,6 +328,7 @@ __global__ void k_ntt_naive_stage(NttLaunch a, u32 log_n, u32 S, bool inv)
 
 __global__ void k_ntt_naive_final(NttLaunch a, u32 log_n)
 {
+    stream_order();
     const u32 N = 1u << log_n;
     const size_t gid = (size_t)blockIdx.x * blockDim.x + threadIdx.x;
     if (gid >= (size_t)a.items * N) return;
@@ -337,6 +344,7 @@ __global__ void k_ntt_naive_final(NttLaunch a, u32 log_n)
 __global__ void k_dyadic(u64 *out, const u64 *a, const u64 *b, u32 log_n, u32 items, u32 limbs,
                          u32 first_prime, const PrimeConst *pcs)
 {
+    stream_order();
     const size_t total2 = ((size_t)items << log_n) >> 1;
     for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < total2;
          g += (size_t)gridDim.x * blockDim.x) {
@@ -358,6 +366,7 @@ __global__ void k_dyadic(u64 *out, const u64 *a, const u64 *b, u32 log_n, u32 it
 __global__ void k_tensor(u64 *out3, const u64 *ct_a, const u64 *ct_b, u32 log_n, u32 n, u32 count,
                          const PrimeConst *pcs)
 {
+    stream_order();
     const size_t per = (size_t)n << log_n;           // words per component
     const size_t total2 = (size_t)count * per / 2;
     for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < total2;
@@ -391,6 +400,7 @@ __global__ void k_tensor(u64 *out3, const u64 *ct_a, const u64 *ct_b, u32 log_n,
 // limbs of 2^log_n words (any number of components), two words per thread.
 __global__ void k_ct_add(u64 *out, const u64 *a, const u64 *b, u64 words, u32 log_n, u32 n, const PrimeConst *pcs)
 {
+    stream_order();
     for (u64 g = (u64)blockIdx.x * blockDim.x + threadIdx.x; 2 * g < words; g += (u64)gridDim.x * blockDim.x) {
         const u64 e = 2 * g;
         const PrimeConst pc = pcs[(u32)((e >> log_n) % n)];
@@ -405,10 +415,11 @@ __global__ void k_ct_add(u64 *out, const u64 *a, const u64 *b, u64 words, u32 lo
 // the same for every limb (automorph_index).
 __global__ void k_ct_automorph(u64 *out, const u64 *in, u64 words, u32 log_n, u32 g)
 {
+    stream_order();
     const u32 N = 1u << log_n;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u32 i = (u32)e & (N - 1);
-        out[e] = __ldg(reinterpret_cast<const unsigned long long *>(in + (e - i) + automorph_index(i, log_n, g)));
+        out[e] = rd(in + (e - i) + automorph_index(i, log_n, g));
     }
 }
 
@@ -437,6 +448,7 @@ __global__ void __launch_bounds__(128, TI * TJ == 4 ? 3 : 4)
 k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 log_n, u32 limbs, u64 warps,
                    const PrimeConst *pcs, const LimbConst *lcs)
 {
+    stream_order();
     const u64 w = (u64)blockIdx.x * 4 + __shfl_sync(0xffffffffu, threadIdx.x >> 5, 0);   // uniform over the warp
     if (w >= warps) return;
     const u32 jt = (n + TJ - 1) / TJ, tiles = (m + TI - 1) / TI * jt;
@@ -515,6 +527,7 @@ k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 
 __global__ void k_enc_noise(u64 *out, const int8_t *v, const int8_t *e0, const int8_t *e1, u32 log_n, u32 n,
                             u32 count, const PrimeConst *pcs)
 {
+    stream_order();
     const u64 N = 1ull << log_n, words = (u64)count * 3 * n * N;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u64 i = e & (N - 1), row = e >> log_n;
@@ -556,6 +569,7 @@ __device__ __forceinline__ int enc_draw(u64 seed, u32 w, u64 c, u64 i, u32 log_n
 // The draws themselves, as signed 8-bit values [count][N] each.
 __global__ void k_enc_draws(int8_t *v, int8_t *e0, int8_t *e1, u64 seed, u32 log_n, u32 count)
 {
+    stream_order();
     const u64 N = 1ull << log_n, total = (u64)count * N;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (u64)gridDim.x * blockDim.x) {
         const u64 c = e >> log_n, i = e & (N - 1);
@@ -568,6 +582,7 @@ __global__ void k_enc_draws(int8_t *v, int8_t *e0, int8_t *e1, u64 seed, u32 log
 // As k_enc_noise, with the draws generated in place from the seed.
 __global__ void k_enc_noise_seeded(u64 *out, u64 seed, u32 log_n, u32 n, u32 count, const PrimeConst *pcs)
 {
+    stream_order();
     const u64 N = 1ull << log_n, words = (u64)count * 3 * n * N;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u64 i = e & (N - 1), row = e >> log_n;
@@ -585,6 +600,7 @@ __global__ void k_enc_noise_seeded(u64 *out, u64 seed, u32 log_n, u32 n, u32 cou
 __global__ void k_enc_combine(u64 *ct, const u64 *noise, const u64 *pt, const u64 *pk, u32 log_n, u32 n, u32 count,
                               u32 pk_limbs, const PrimeConst *pcs)
 {
+    stream_order();
     const u64 N = 1ull << log_n, per = (u64)n * N, total = (u64)count * per;
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (u64)gridDim.x * blockDim.x) {
         const u64 c = e / per, off = e - c * per;
@@ -715,7 +731,7 @@ struct DSource {
     __device__ __forceinline__ ulonglong2 pair(const u64 *row, u32 log_n, u32 P) const
     {
         const u32 src = galois ? automorph_index(P, log_n, galois) : P;
-        const ulonglong2 v = __ldg(reinterpret_cast<const ulonglong2 *>(row + (src & ~1u)));
+        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(row + (src & ~1u));
         return (src & 1u) ? make_ulonglong2(v.y, v.x) : v;
     }
 };
@@ -766,7 +782,7 @@ __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 
                 const u32 P = (u32)last_pos<Sh>(m, tid, e);
                 const u32 src = automorph_index(P, Sh::LOG_N, ds.galois);
                 u64 v[4];
-                ld4_nc(d + (src & ~3u), v[0], v[1], v[2], v[3]);
+                ld4(d + (src & ~3u), v[0], v[1], v[2], v[3]);
 #pragma unroll
                 for (u32 i = 0; i < 4; i++) {
                     const u32 o = (i ? automorph_index(P + i, Sh::LOG_N, ds.galois) : src) & 3u;
@@ -776,7 +792,7 @@ __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 
         } else {
 #pragma unroll
             for (int e = 0; e < Sh::E; e += 4)
-                ld4_nc(d + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
+                ld4(d + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
         }
     } else {
         const size_t off = ds.per + (size_t)j * Sh::N;
@@ -784,8 +800,8 @@ __device__ __forceinline__ void ks_digits_body(const EvalArgs &a, u32 item, u32 
         for (int e = 0; e < Sh::E; e += 4) {
             const int P = last_pos<Sh>(m, tid, e);
             u64 b[4];
-            ld4_nc(ds.ct_a + off + P, x[e], x[e + 1], x[e + 2], x[e + 3]);
-            ld4_nc(ds.ct_b + off + P, b[0], b[1], b[2], b[3]);
+            ld4(ds.ct_a + off + P, x[e], x[e + 1], x[e + 2], x[e + 3]);
+            ld4(ds.ct_b + off + P, b[0], b[1], b[2], b[3]);
 #pragma unroll
             for (int i = 0; i < 4; i++) x[e + i] = mul_mont(x[e + i], b[i], pc);
         }
@@ -801,6 +817,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_ks_digits(EvalArgs a0, JobsArg<JOBS> tab)
 {
+    stream_order();
     EvalArgs a = a0;
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -814,6 +831,7 @@ template <int LOG_B, int LOG_C, int LOG_E, int KIND>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_ks_digits_of(EvalArgs a)
 {
+    stream_order();
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
     ks_digits_body<NttShape<LOG_B, LOG_C, LOG_E>, KIND>(a, blockIdx.x >> LOG_C, m, 0, true);
 }
@@ -822,6 +840,7 @@ template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::EVAL_MIN_CTAS)
 k_ks_modup(EvalArgs a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     u64 *acc = smem + Sh::B;                   // [2][E][T], own positions only
@@ -846,11 +865,11 @@ k_ks_modup(EvalArgs a)
             // The transform takes any input below 8t + 2^32 congruent to the
             // digit: when q_j <= 8t the digit c2_j < q_j goes in as it is.
             if (a.ctx.pc[j].p <= (pc.four_p << 1)) {
-                auto ld = [&](u32 P) -> u64 { return __ldg(reinterpret_cast<const unsigned long long *>(src + P)); };
+                auto ld = [&](u32 P) -> u64 { return rd(src + P); };
                 ntt_fwd_block<Sh, false>(smem, m, 0, twf, pc, ld, st, x);
             } else {
                 auto ld = [&](u32 P) -> u64 {
-                    return reduce_word(__ldg(reinterpret_cast<const unsigned long long *>(src + P)), pc);
+                    return reduce_word(rd(src + P), pc);
                 };
                 ntt_fwd_block<Sh, false>(smem, m, 0, twf, pc, ld, st, x);
             }
@@ -941,6 +960,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_ks_expand(EvalArgs a0, JobsArg<JOBS> tab)
 {
+    stream_order();
     EvalArgs a = a0;
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -970,6 +990,11 @@ k_ks_expand(EvalArgs a0, JobsArg<JOBS> tab)
 struct MacVec {
     u64 v[2];
     __device__ __forceinline__ static MacVec load(const u64 *p)
+    {
+        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+        return {{t.x, t.y}};
+    }
+    __device__ __forceinline__ static MacVec key(const u64 *p)   // read-only path: key words
     {
         const ulonglong2 t = __ldg(reinterpret_cast<const ulonglong2 *>(p));
         return {{t.x, t.y}};
@@ -1085,17 +1110,17 @@ __device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 t
     const u64 *mx = a.mx + ((size_t)g * (n + 1) + t) * n * N + P;        // mx [g][target][j][N]
     const u64 *kt = key + (t < n ? t : 0) * key_j;
     MacSums acc;
-    acc.begin(ds, t, n, log_n, P, pc, Vec::load(kt), Vec::load(kt + key_k), a.ctx.limb);
+    acc.begin(ds, t, n, log_n, P, pc, Vec::key(kt), Vec::key(kt + key_k), a.ctx.limb);
     // the digits j != t: n of them on the special prime, n - 1 otherwise
     const u32 terms = t < n ? n - 1 : n;
     u32 j = t == 0 ? 1u : 0u;
     Vec v, w0, w1;
-    if (terms) v = Vec::load(mx + (size_t)j * N), w0 = Vec::load(key + j * key_j), w1 = Vec::load(key + j * key_j + key_k);
+    if (terms) v = Vec::load(mx + (size_t)j * N), w0 = Vec::key(key + j * key_j), w1 = Vec::key(key + j * key_j + key_k);
     for (u32 i = 0; i < terms; i++) {
         const Vec x = v, k0 = w0, k1 = w1;
         if (i + 1 < terms) {
             j += j + 1 == t ? 2u : 1u;
-            v = Vec::load(mx + (size_t)j * N), w0 = Vec::load(key + j * key_j), w1 = Vec::load(key + j * key_j + key_k);
+            v = Vec::load(mx + (size_t)j * N), w0 = Vec::key(key + j * key_j), w1 = Vec::key(key + j * key_j + key_k);
         }
         acc.digit(x, k0, k1, pc);
     }
@@ -1108,6 +1133,7 @@ __device__ __forceinline__ void ks_mac_tile(const EvalArgs &a, u32 groups, u32 t
 template <bool JOBS, int KIND>
 __global__ void __launch_bounds__(MAC_BLOCK / 2, 4) k_ks_mac(EvalArgs a0, u32 groups, u32 total, JobsArg<JOBS> tab)
 {
+    stream_order();
     for (u32 q = blockIdx.x; q < total; q += gridDim.x) {
         if constexpr (JOBS) {
             EvalArgs a = a0;
@@ -1135,6 +1161,7 @@ constexpr u32 MAC_TILE = 64, MAC_CHUNK = 32;
 template <int KIND>
 __global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
 {
+    stream_order();
     using Vec = MacVec;
     extern __shared__ __align__(16) u64 key_tile[];   // [2 n][MAC_TILE]
     const u32 n = a.n, N = a.ctx.N, nd1 = a.ctx.n_data + 1;
@@ -1146,7 +1173,7 @@ __global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
     const u32 P0 = tile * MAC_TILE;
     for (u32 i = 2 * threadIdx.x; i < n * 2 * MAC_TILE; i += 2 * blockDim.x) {
         const u32 row = i / MAC_TILE, col = i % MAC_TILE;   // row 2 j + k: evk [j][k][target][N]
-        MacVec::load(a.evk_mac + ((size_t)row * nd1 + tp) * N + P0 + col).store(key_tile + i);
+        MacVec::key(a.evk_mac + ((size_t)row * nd1 + tp) * N + P0 + col).store(key_tile + i);
     }
     __syncthreads();
     const u32 lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1197,6 +1224,7 @@ __device__ __forceinline__ u64 shoup_step(u64 &r, const PrimeConst &c)
 __global__ void k_key_prepare(ulonglong2 *evk, u64 *evk_mac, const u64 *raw, u64 words, u32 log_n, u32 nd,
                               const PrimeConst *pcs, const LimbConst *limb, u64 R_special)
 {
+    stream_order();
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u32 t = (u32)((e >> log_n) % (nd + 1));
         const PrimeConst pc = pcs[t];
@@ -1223,6 +1251,7 @@ template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_ks_moddown(EvalArgs a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     const u32 tid = threadIdx.x;
@@ -1253,6 +1282,7 @@ template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_rs_lift(EvalArgs a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -1273,6 +1303,7 @@ template <int LOG_B, int LOG_C, int LOG_E>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_rs(EvalArgs a)
 {
+    stream_order();
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     extern __shared__ __align__(16) u64 smem[];
     const u32 tid = threadIdx.x;
@@ -1400,6 +1431,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_mrr_lift(EvalArgs a0, JobsArg<JOBS> tab)
 {
+    stream_order();
     EvalArgs a = a0;
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
@@ -1412,6 +1444,7 @@ template <int LOG_B, int LOG_C, int LOG_E, bool JOBS = false>
 __global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
 k_mrr_rest(EvalArgs a0, JobsArg<JOBS> tab)
 {
+    stream_order();
     EvalArgs a = a0;
     using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
     const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;

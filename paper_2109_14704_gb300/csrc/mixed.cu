@@ -19,33 +19,15 @@ static cudaError_t mixed_prepare()
     return e;
 }
 
-static cudaLaunchConfig_t mixed_cfg(u32 clusters, cudaStream_t s, cudaLaunchAttribute *attr)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(clusters * 8, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = kMixedSmem;
-    cfg.stream = s;
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 8;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cfg;
-}
-
 cudaError_t launch_ntt_mixed(const MixedUnit *units, u32 n_units, const LimbJob *jobs, bool inverse, u32 clusters,
                              cudaStream_t s)
 {
-    cudaLaunchAttribute attr[1];
-    cudaLaunchConfig_t cfg = mixed_cfg(clusters, s, attr);
     if (inverse) {
         if (cudaError_t e = mixed_prepare<true>()) return e;
-        return cudaLaunchKernelEx(&cfg, k_ntt_mixed<true>, units, n_units, jobs);
+        return launch_k(k_ntt_mixed<true>, clusters * 8, 256, kMixedSmem, 8, s, units, n_units, jobs);
     }
     if (cudaError_t e = mixed_prepare<false>()) return e;
-    return cudaLaunchKernelEx(&cfg, k_ntt_mixed<false>, units, n_units, jobs);
+    return launch_k(k_ntt_mixed<false>, clusters * 8, 256, kMixedSmem, 8, s, units, n_units, jobs);
 }
 
 }  // namespace he

@@ -72,6 +72,7 @@ __device__ __noinline__ void multi_item(const EvalArgs &a, u32 item, u32 m, u32 
 template <MultiStage S>
 __global__ void __launch_bounds__(256, 4) k_mrr_multi(EvalArgs a0, JobTable t)
 {
+    stream_order();
     EvalArgs a = a0;
     const u32 rank = cluster_ctarank();
     const u32 unit = bind_job(a, t, multi_slot(S), blockIdx.x >> 3);
@@ -99,19 +100,7 @@ static cudaError_t launch_stage(const EvalArgs &a, const JobTable &t, u32 units,
         e = cudaFuncSetAttribute(k_mrr_multi<S>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kMultiSmem);
     });
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(units * 8, 1, 1);
-    cfg.blockDim = dim3(256, 1, 1);
-    cfg.dynamicSmemBytes = kMultiSmem;
-    cfg.stream = s;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeClusterDimension;
-    attr[0].val.clusterDim.x = 8;
-    attr[0].val.clusterDim.y = 1;
-    attr[0].val.clusterDim.z = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_mrr_multi<S>, a, t);
+    return launch_k(k_mrr_multi<S>, units * 8, 256, kMultiSmem, 8, s, a, t);
 }
 
 cudaError_t launch_mrr_multi(MultiStage stage, const EvalArgs &a, const JobTable &t, u32 units, cudaStream_t s)
