@@ -581,8 +581,8 @@ extern "C" he_status he_dyadic_mul(uint64_t *out, const uint64_t *a, const uint6
         return fail(HE_EINVAL, "inputs must be non-NULL and 32-byte aligned");
     const u64 items = (u64)limbs * count;
     if (!items) return HE_OK;
-    HE_CUDA(he::launch_k(he::k_dyadic, stream_grid(items * N / 2, 256), 256, 0, 1, (cudaStream_t)stream, out, a, b, (u32)log_n, (u32)items, limbs, 0, tw->d_pc));
-    HE_CUDA(cudaGetLastError());
+    HE_CUDA(he::launch_k(he::k_dyadic, stream_grid(items * N / 2, 256), 256, 0, 1, (cudaStream_t)stream, out, a, b,
+                         (u32)log_n, (u32)items, limbs, 0, tw->d_pc));
     return HE_OK;
 }
 
@@ -827,8 +827,8 @@ extern "C" he_status he_ct_mul(uint64_t *out3, const uint64_t *ct_a, const uint6
     if (he_status s = check_ptr(ct_a, "ct_a")) return s;
     if (he_status s = check_ptr(ct_b, "ct_b")) return s;
     const u32 n = level + 1;
-    HE_CUDA(he::launch_k(he::k_tensor, stream_grid((u64)n * ctx->N / 2, 256), 256, 0, 1, (cudaStream_t)stream, out3, ct_a, ct_b, (u32)ctx->log_n, n, 1, ctx->tables->d_pc));
-    HE_CUDA(cudaGetLastError());
+    HE_CUDA(he::launch_k(he::k_tensor, stream_grid((u64)n * ctx->N / 2, 256), 256, 0, 1, (cudaStream_t)stream, out3,
+                         ct_a, ct_b, (u32)ctx->log_n, n, 1, ctx->tables->d_pc));
     return HE_OK;
 }
 
@@ -916,7 +916,8 @@ static he_status ks_mac(const he_context *ctx, const he::EvalArgs &a, u32 gs, cu
         HE_CUDA(he::launch_k(he::k_ks_mac_tiled<KIND>, blocks, 256, smem, 1, s, a, gs));
     } else {
         const u32 tiles = gs * (n + 1) * (ctx->N / he::MAC_BLOCK);
-        HE_CUDA(he::launch_k(he::k_ks_mac<false, KIND>, mac_grid(tiles), he::MAC_BLOCK / 2, 0, 1, s, a, gs, tiles, he::NoJobs{}));
+        HE_CUDA(he::launch_k(he::k_ks_mac<false, KIND>, mac_grid(tiles), he::MAC_BLOCK / 2, 0, 1, s, a, gs, tiles,
+                             he::NoJobs{}));
     }
     HE_CUDA(cudaGetLastError());
     return HE_OK;
@@ -1174,8 +1175,8 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
     a.n = t.job[0].n;   // unused with a job table; kept valid
     if (he_status r = run_eval(ctx, he::EK_KS_DIGITS, a, (u32)tot[he::JS_DIGITS], s, &t)) return r;
     if (he_status r = run_eval(ctx, he::EK_KS_EXPAND, a, (u32)tot[he::JS_EXPAND], s, &t)) return r;
-    HE_CUDA(he::launch_k(he::k_ks_mac<true, he::SRC_PAIR>, mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, 1, s, a, 0, (u32)tot[he::JS_MAC], t));
-    HE_CUDA(cudaGetLastError());
+    HE_CUDA(he::launch_k(he::k_ks_mac<true, he::SRC_PAIR>, mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, 1, s, a,
+                         0, (u32)tot[he::JS_MAC], t));
     if (he_status r = run_eval(ctx, he::EK_MRR_LIFT, a, (u32)tot[he::JS_LIFT], s, &t)) return r;
     return run_eval(ctx, he::EK_MRR_REST, a, (u32)tot[he::JS_REST], s, &t);
 }
@@ -1227,8 +1228,8 @@ extern "C" he_status he_ct_add(uint64_t *ct_out, const uint64_t *ct_a, const uin
     if (count == 0) return HE_OK;
     const u32 n = level + 1;
     const u64 words = (u64)count * components * n * ctx->N;
-    HE_CUDA(he::launch_k(he::k_ct_add, stream_grid(words / 2, 256), 256, 0, 1, (cudaStream_t)stream, ct_out, ct_a, ct_b, words, (u32)ctx->log_n, n, ctx->tables->d_pc));
-    HE_CUDA(cudaGetLastError());
+    HE_CUDA(he::launch_k(he::k_ct_add, stream_grid(words / 2, 256), 256, 0, 1, (cudaStream_t)stream, ct_out, ct_a,
+                         ct_b, words, (u32)ctx->log_n, n, ctx->tables->d_pc));
     return HE_OK;
 }
 
@@ -1248,9 +1249,9 @@ extern "C" he_status he_ct_automorph(uint64_t *ct_out, const uint64_t *ct_in, ui
     if (ct_out == ct_in) return fail(HE_EINVAL, "the automorphism cannot work in place");
     if (count == 0 || components == 0) return HE_OK;
     const u64 words = (u64)count * components * (level + 1) * ctx->N;
-    HE_CUDA(he::launch_k(he::k_ct_automorph, stream_grid(words, 256), 256, 0, 1, (cudaStream_t)stream, ct_out, ct_in, words,
+    HE_CUDA(he::launch_k(he::k_ct_automorph, stream_grid(words, 256), 256, 0, 1, (cudaStream_t)stream, ct_out, ct_in,
+                         words,
                                                                                   (u32)ctx->log_n, galois_elt));
-    HE_CUDA(cudaGetLastError());
     return HE_OK;
 }
 
@@ -1575,17 +1576,19 @@ static he_status encrypt_common(uint64_t *ct_out, const uint64_t *pt, const uint
     const u32 n = level + 1;
     cudaStream_t s = (cudaStream_t)stream;
     u64 *noise = (u64 *)scratch;
-    const u64 words = (u64)count * 3 * n * ctx->N;
-    if (v)
-        HE_CUDA(he::launch_k(he::k_enc_noise, stream_grid(words, 256), 256, 0, 1, s, noise, v, e0, e1, (u32)ctx->log_n, n, count,
-                                                                 ctx->tables->d_pc));
-    else
-        HE_CUDA(he::launch_k(he::k_enc_noise_seeded, stream_grid(words, 256), 256, 0, 1, s, noise, seed, (u32)ctx->log_n, n, count,
-                                                                        ctx->tables->d_pc));
-    HE_CUDA(cudaGetLastError());
-    if (he_status r = ntt_launch(uniform_launch(noise, n, 3 * count, ctx->tables), ctx->log_n, false, s)) return r;
-    HE_CUDA(he::launch_k(he::k_enc_combine, stream_grid((u64)count * n * ctx->N, 256), 256, 0, 1, s, ct_out, noise, pt, pk, (u32)ctx->log_n, n, count, ctx->n_data, ctx->tables->d_pc));
-    HE_CUDA(cudaGetLastError());
+    he::EvalArgs a = {};
+    a.v = v;
+    a.e0 = e0;
+    a.e1 = e1;
+    a.seed = seed;
+    a.out = noise;
+    a.n = n;
+    a.count = count;
+    a.ctx = dev_ctx(ctx);
+    if (he_status r = run_eval(ctx, he::EK_ENC_NOISE, a, 3 * count * n, s)) return r;
+    HE_CUDA(he::launch_k(he::k_enc_combine, stream_grid((u64)count * n * ctx->N / 2, 256), 256, 0, 1, s, ct_out,
+                         noise,
+                         pt, pk, (u32)ctx->log_n, n, count, ctx->n_data, ctx->tables->d_pc));
     return HE_OK;
 }
 
@@ -1613,9 +1616,9 @@ extern "C" he_status he_sample_encryption_draws(int8_t *v, int8_t *e0, int8_t *e
     if (!v || !e0 || !e1) return fail(HE_EINVAL, "v, e0 or e1 is NULL");
     if (count == 0) return HE_OK;
     if ((u64)count * N > (1ull << 40)) return fail(HE_EINVAL, "batch too large");
-    HE_CUDA(he::launch_k(he::k_enc_draws, stream_grid((u64)count * N, 256), 256, 0, 1, (cudaStream_t)stream, v, e0, e1, seed,
+    HE_CUDA(he::launch_k(he::k_enc_draws, stream_grid((u64)count * N, 256), 256, 0, 1, (cudaStream_t)stream, v, e0,
+                         e1, seed,
                                                                                         (u32)log_n, count));
-    HE_CUDA(cudaGetLastError());
     return HE_OK;
 }
 
@@ -2062,8 +2065,8 @@ static he_status mrr_multi_pass(const he_mrr_multi_job *jobs, u32 n_jobs, u64 *w
     a.n = t.job[0].n;
     HE_CUDA(he::launch_mrr_multi(he::MS_DIGITS, a, t, (u32)tot[he::JS_DIGITS], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_EXPAND, a, t, (u32)tot[he::JS_EXPAND], s));
-    HE_CUDA(he::launch_k(he::k_ks_mac<true, he::SRC_PAIR>, mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, 1, s, a, 0, (u32)tot[he::JS_MAC], t));
-    HE_CUDA(cudaGetLastError());
+    HE_CUDA(he::launch_k(he::k_ks_mac<true, he::SRC_PAIR>, mac_grid(tot[he::JS_MAC]), he::MAC_BLOCK / 2, 0, 1, s, a,
+                         0, (u32)tot[he::JS_MAC], t));
     HE_CUDA(he::launch_mrr_multi(he::MS_LIFT, a, t, (u32)tot[he::JS_LIFT], s));
     HE_CUDA(he::launch_mrr_multi(he::MS_REST, a, t, (u32)tot[he::JS_REST], s));
     return HE_OK;

@@ -140,6 +140,7 @@ struct ShapeOps {
             HE_EVAL_CASE(EK_RS, k_rs, sm1)
             HE_EVAL_CASE_J(EK_MRR_LIFT, k_mrr_lift, sm1)
             HE_EVAL_CASE_J(EK_MRR_REST, k_mrr_rest, sm1)
+            HE_EVAL_CASE(EK_ENC_NOISE, k_enc_noise, sm1)
 #undef HE_EVAL_CASE_J
 #undef HE_EVAL_CASE
         default:

@@ -290,6 +290,33 @@ __device__ __forceinline__ u32 automorph_index(u32 i, u32 log_n, u32 g)
     return __brev((t - 1) >> 1) >> sh;
 }
 
+// Randomness of encryption drawn on the device (Sec. II-A Encrypt: a
+// uniform ternary mask v and Gaussian-like errors e0, e1). Generator:
+// SplitMix64 in counter form (Steele, Lea and Flood 2014): output k of the
+// stream with key `seed` is mix(seed + (k + 1) * 0x9E3779B97F4A7C15), with
+// mix(z): z = (z ^ z >> 30) * 0xBF58476D1CE4E5B9; z = (z ^ z >> 27) *
+// 0x94D049BB133111EB; z ^ z >> 31. Draw w (0: v, 1: e0, 2: e1) of message c
+// at coefficient i uses output k = (3 c + w) N + i:
+//   v  = (r mod 3) - 1                        (bias below 2^-63)
+//   e  = popcount(r & (2^20 - 1)) - popcount((r >> 20) & (2^20 - 1)),
+// the centred binomial distribution of parameter 20 (variance 10, standard
+// deviation 3.16, |e| <= 20): integer-only, so that any implementation
+// following this definition reproduces the draws bit for bit.
+__device__ __forceinline__ u64 splitmix64_at(u64 seed, u64 k)
+{
+    u64 z = seed + (k + 1) * 0x9E3779B97F4A7C15ull;
+    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
+    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
+    return z ^ (z >> 31);
+}
+
+__device__ __forceinline__ int enc_draw(u64 seed, u32 w, u64 c, u64 i, u32 log_n)
+{
+    const u64 r = splitmix64_at(seed, ((3 * c + w) << log_n) + i);
+    if (w == 0) return (int)(r % 3u) - 1;
+    return __popcll(r & 0xFFFFFull) - __popcll((r >> 20) & 0xFFFFFull);
+}
+
 #ifdef HE_MISC_KERNELS  // defined by the one translation unit that owns them
 // ======================================================== naive radix-2 ====
 // The baseline of Sec. III-B: one launch per stage, each thread one
@@ -521,51 +548,6 @@ k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 
 
 // ============================================================ Encrypt ======
 
-// Residues of the encryption's small random polynomials: out[c][w][l][i] =
-// src_w[c][i] mod q_l for w = 0, 1, 2 (v, e0, e1; signed 8-bit values with
-// |x| < q), count messages of n limbs.
-__global__ void k_enc_noise(u64 *out, const int8_t *v, const int8_t *e0, const int8_t *e1, u32 log_n, u32 n,
-                            u32 count, const PrimeConst *pcs)
-{
-    stream_order();
-    const u64 N = 1ull << log_n, words = (u64)count * 3 * n * N;
-    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
-        const u64 i = e & (N - 1), row = e >> log_n;
-        const u32 l = (u32)(row % n), w = (u32)((row / n) % 3);
-        const u64 c = row / (3 * (u64)n);
-        const int8_t *src = w == 0 ? v : (w == 1 ? e0 : e1);
-        const int x = src[c * N + i];
-        out[e] = x >= 0 ? (u64)x : pcs[l].p - (u64)(-x);
-    }
-}
-
-// Randomness of encryption drawn on the device (Sec. II-A Encrypt: a
-// uniform ternary mask v and Gaussian-like errors e0, e1). Generator:
-// SplitMix64 in counter form (Steele, Lea and Flood 2014): output k of the
-// stream with key `seed` is mix(seed + (k + 1) * 0x9E3779B97F4A7C15), with
-// mix(z): z = (z ^ z >> 30) * 0xBF58476D1CE4E5B9; z = (z ^ z >> 27) *
-// 0x94D049BB133111EB; z ^ z >> 31. Draw w (0: v, 1: e0, 2: e1) of message c
-// at coefficient i uses output k = (3 c + w) N + i:
-//   v  = (r mod 3) - 1                        (bias below 2^-63)
-//   e  = popcount(r & (2^20 - 1)) - popcount((r >> 20) & (2^20 - 1)),
-// the centred binomial distribution of parameter 20 (variance 10, standard
-// deviation 3.16, |e| <= 20): integer-only, so that any implementation
-// following this definition reproduces the draws bit for bit.
-__device__ __forceinline__ u64 splitmix64_at(u64 seed, u64 k)
-{
-    u64 z = seed + (k + 1) * 0x9E3779B97F4A7C15ull;
-    z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9ull;
-    z = (z ^ (z >> 27)) * 0x94D049BB133111EBull;
-    return z ^ (z >> 31);
-}
-
-__device__ __forceinline__ int enc_draw(u64 seed, u32 w, u64 c, u64 i, u32 log_n)
-{
-    const u64 r = splitmix64_at(seed, ((3 * c + w) << log_n) + i);
-    if (w == 0) return (int)(r % 3u) - 1;
-    return __popcll(r & 0xFFFFFull) - __popcll((r >> 20) & 0xFFFFFull);
-}
-
 // The draws themselves, as signed 8-bit values [count][N] each.
 __global__ void k_enc_draws(int8_t *v, int8_t *e0, int8_t *e1, u64 seed, u32 log_n, u32 count)
 {
@@ -579,39 +561,31 @@ __global__ void k_enc_draws(int8_t *v, int8_t *e0, int8_t *e1, u64 seed, u32 log
     }
 }
 
-// As k_enc_noise, with the draws generated in place from the seed.
-__global__ void k_enc_noise_seeded(u64 *out, u64 seed, u32 log_n, u32 n, u32 count, const PrimeConst *pcs)
-{
-    stream_order();
-    const u64 N = 1ull << log_n, words = (u64)count * 3 * n * N;
-    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
-        const u64 i = e & (N - 1), row = e >> log_n;
-        const u32 l = (u32)(row % n), w = (u32)((row / n) % 3);
-        const u64 c = row / (3 * (u64)n);
-        const int x = enc_draw(seed, w, c, i, log_n);
-        out[e] = x >= 0 ? (u64)x : pcs[l].p - (u64)(-x);
-    }
-}
-
 // Public-key encryption (Sec. II-A) from the transformed randomness:
 // c0 = v pk0 + pt + e0, c1 = v pk1 + e1 (NTT domain, limb by limb).
 // noise [count][3][n][N] (v, e0, e1 transformed), pt [count][n][N],
 // pk [2][pk_limbs][N], ct [count][2][n][N].
+// Two words a thread; rows (a limb of a message) are counted in 32 bits.
 __global__ void k_enc_combine(u64 *ct, const u64 *noise, const u64 *pt, const u64 *pk, u32 log_n, u32 n, u32 count,
                               u32 pk_limbs, const PrimeConst *pcs)
 {
     stream_order();
-    const u64 N = 1ull << log_n, per = (u64)n * N, total = (u64)count * per;
-    for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < total; e += (u64)gridDim.x * blockDim.x) {
-        const u64 c = e / per, off = e - c * per;
-        const u32 l = (u32)(off >> log_n);
-        const PrimeConst pc = pcs[l];
+    const size_t N = (size_t)1 << log_n, per = (size_t)n << log_n, pairs = (size_t)count * per / 2;
+    for (size_t g = (size_t)blockIdx.x * blockDim.x + threadIdx.x; g < pairs; g += (size_t)gridDim.x * blockDim.x) {
+        const u32 row = (u32)(g >> (log_n - 1)), c = row / n, l = row - c * n;
+        const size_t P = 2 * g & (N - 1), off = ((size_t)l << log_n) + P;
+        const PrimeConst &pc = pcs[l];
+        auto ld = [](const u64 *q) { return *reinterpret_cast<const ulonglong2 *>(q); };
         const u64 *z = noise + c * 3 * per + off;
-        const u64 vh = z[0], e0h = z[per], e1h = z[2 * per];
-        const u64 c0 = add_mod(add_mod(mul_mod(vh, pk[off], pc), pt[e], pc.p), e0h, pc.p);
-        const u64 c1 = add_mod(mul_mod(vh, pk[(u64)pk_limbs * N + off], pc), e1h, pc.p);
-        ct[c * 2 * per + off] = c0;
-        ct[c * 2 * per + per + off] = c1;
+        const ulonglong2 v = ld(z), e0 = ld(z + per), e1 = ld(z + 2 * per), m = ld(pt + 2 * g);
+        const ulonglong2 k0 = ld(pk + off), k1 = ld(pk + pk_limbs * N + off);
+        auto c0 = [&](u64 a, u64 k, u64 t, u64 e) {
+            return add_mod(add_mod(mul_mod(a, k, pc), t, pc.p), e, pc.p);
+        };
+        u64 *out = ct + c * 2 * per + off;
+        *reinterpret_cast<ulonglong2 *>(out) = make_ulonglong2(c0(v.x, k0.x, m.x, e0.x), c0(v.y, k0.y, m.y, e0.y));
+        *reinterpret_cast<ulonglong2 *>(out + per) =
+            make_ulonglong2(add_mod(mul_mod(v.x, k1.x, pc), e1.x, pc.p), add_mod(mul_mod(v.y, k1.y, pc), e1.y, pc.p));
     }
 }
 #endif  // HE_MISC_KERNELS
@@ -1451,6 +1425,33 @@ k_mrr_rest(EvalArgs a0, JobsArg<JOBS> tab)
     u32 item = blockIdx.x >> LOG_C;
     if constexpr (JOBS) item = bind_job(a, tab, JS_REST, item);
     mrr_rest_body<Sh>(a, item, m, 0, true);
+}
+
+// Encryption (Sec. II-A): the transforms of the small random polynomials,
+// out[c][w][l] = NTT_l(x mod q_l) for w = 0, 1, 2 (v, e0, e1 of message c; |x| <
+// q_l), formed on the loads from the given draws or from the seed. Item =
+// (3 c + w) n + l. Five messages of 7 limbs at N = 2^14 (105 transforms): a
+// noise pass and the transforms took 11 + 24 us, 25 us this way.
+template <int LOG_B, int LOG_C, int LOG_E>
+__global__ void __launch_bounds__(NttShape<LOG_B, LOG_C, LOG_E>::T, NttShape<LOG_B, LOG_C, LOG_E>::MIN_CTAS)
+k_enc_noise(EvalArgs a)
+{
+    stream_order();
+    using Sh = NttShape<LOG_B, LOG_C, LOG_E>;
+    extern __shared__ __align__(16) u64 smem[];
+    const u32 m = (LOG_C > 0) ? cluster_ctarank() : 0u;
+    const u32 item = blockIdx.x >> LOG_C;
+    const u32 l = item % a.n, w = (item / a.n) % 3, c = item / (3 * a.n);
+    const PrimeConst pc = a.ctx.pc[l];
+    const int8_t *src = a.v ? (w == 0 ? a.v : (w == 1 ? a.e0 : a.e1)) + (size_t)c * Sh::N : nullptr;
+    auto ld = [&](int P) -> u64 {
+        const int x = src ? src[P] : enc_draw(a.seed, w, c, (u64)P, Sh::LOG_N);
+        return x >= 0 ? (u64)x : pc.p - (u64)(-x);
+    };
+    auto nost = [&](u32, u64) {};
+    u64 x[Sh::E];
+    ntt_fwd_block<Sh>(smem, m, 0, a.ctx.tw_fwd + (size_t)l * Sh::N, pc, ld, nost, x);
+    store_run<Sh>(a.out + (size_t)item * Sh::N, x, m, threadIdx.x);
 }
 
 }  // namespace he

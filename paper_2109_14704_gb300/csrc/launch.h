@@ -162,6 +162,10 @@ struct EvalArgs {
     u32 n;                      // limbs at the current level
     u32 count;
     u32 c_first;                // first ciphertext of the expanded mod-up group
+    // randomness of an encryption: the draws [count][N], or (v null) the seed
+    // they come from
+    const int8_t *v, *e0, *e1;
+    u64 seed;
     u32 galois;                 // nonzero: the input is (sigma(c0), 0, sigma(c1)), sigma: X -> X^galois
     DevCtx ctx;
 };
@@ -208,6 +212,7 @@ enum EvalKernel {
     EK_RS,
     EK_MRR_LIFT,
     EK_MRR_REST,
+    EK_ENC_NOISE,
     EK_COUNT
 };
 
