@@ -222,10 +222,19 @@ def _i8ptr(x, values: int):
     return x.data_ptr()
 
 
+def _current_stream() -> int:
+    """Handle of the current CUDA stream, without building a Stream object
+    where this PyTorch hands it out."""
+    import torch
+    raw = getattr(torch._C, "_cuda_getCurrentRawStream", None)
+    if raw is None:
+        return torch.cuda.current_stream().cuda_stream
+    return raw(torch.cuda.current_device())
+
+
 def _stream(stream):
     if stream is None:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
@@ -267,9 +276,9 @@ class NttTables:
     def __init__(self, N: int, moduli):
         self.N = int(N)
         self.moduli = [int(q) for q in moduli]
-        self._m = _host_u64(self.moduli)
+        self._mp = _hp(_host_u64(self.moduli))
         h = _vp()
-        _check(load().he_ntt_tables_create(self.N, len(self.moduli), _hp(self._m), ctypes.byref(h)))
+        _check(load().he_ntt_tables_create(self.N, len(self.moduli), self._mp, ctypes.byref(h)))
         self.handle = h
 
     def psi(self, index: int) -> int:
@@ -310,18 +319,19 @@ def ntt_set_shape(N: int, log_block: int = 0, log_thread_words: int = 0, persist
 
 
 def _moduli_arg(tables: NttTables, limbs: int, moduli):
-    m = _host_u64(tables.moduli[:limbs] if moduli is None else list(moduli)[:limbs])
-    return m
+    """Pointer to the moduli of a call: the tables' own unless given (it keeps
+    its array alive)."""
+    return tables._mp if moduli is None else _hp(_host_u64(list(moduli)[:limbs]))
 
 
 def ntt_fwd(poly, N, limbs, count, tables: NttTables, moduli=None, stream=None):
     m = _moduli_arg(tables, limbs, moduli)
-    _check(load().he_ntt_fwd(_ptr(poly, N * limbs * count), N, limbs, count, _hp(m), tables.handle, _stream(stream)))
+    _check(load().he_ntt_fwd(_ptr(poly, N * limbs * count), N, limbs, count, m, tables.handle, _stream(stream)))
 
 
 def ntt_inv(poly, N, limbs, count, tables: NttTables, moduli=None, stream=None):
     m = _moduli_arg(tables, limbs, moduli)
-    _check(load().he_ntt_inv(_ptr(poly, N * limbs * count), N, limbs, count, _hp(m), tables.handle, _stream(stream)))
+    _check(load().he_ntt_inv(_ptr(poly, N * limbs * count), N, limbs, count, m, tables.handle, _stream(stream)))
 
 
 NTT_OP_FORWARD, NTT_OP_INVERSE = 1, 2
@@ -354,24 +364,24 @@ def ntt_host(inp, out, N, limbs, count, tables: NttTables, ops, work, moduli=Non
     m = _moduli_arg(tables, limbs, moduli)
     words = N * limbs * count
     nbytes = work.numel() * work.element_size()
-    _check(load().he_ntt_host(_host_ptr(inp, words), _host_ptr(out, words), N, limbs, count, _hp(m),
+    _check(load().he_ntt_host(_host_ptr(inp, words), _host_ptr(out, words), N, limbs, count, m,
                               tables.handle, ops, _ptr(work), nbytes, _stream(stream)))
 
 
 def ntt_fwd_naive(poly, N, limbs, count, tables: NttTables, moduli=None, stream=None):
     m = _moduli_arg(tables, limbs, moduli)
-    _check(load().he_ntt_fwd_naive(_ptr(poly, N * limbs * count), N, limbs, count, _hp(m), tables.handle, _stream(stream)))
+    _check(load().he_ntt_fwd_naive(_ptr(poly, N * limbs * count), N, limbs, count, m, tables.handle, _stream(stream)))
 
 
 def ntt_inv_naive(poly, N, limbs, count, tables: NttTables, moduli=None, stream=None):
     m = _moduli_arg(tables, limbs, moduli)
-    _check(load().he_ntt_inv_naive(_ptr(poly, N * limbs * count), N, limbs, count, _hp(m), tables.handle, _stream(stream)))
+    _check(load().he_ntt_inv_naive(_ptr(poly, N * limbs * count), N, limbs, count, m, tables.handle, _stream(stream)))
 
 
 def dyadic_mul(out, a, b, N, limbs, count, tables: NttTables, moduli=None, stream=None):
     m = _moduli_arg(tables, limbs, moduli)
     w = N * limbs * count
-    _check(load().he_dyadic_mul(_ptr(out, w), _ptr(a, w), _ptr(b, w), N, limbs, count, _hp(m), tables.handle,
+    _check(load().he_dyadic_mul(_ptr(out, w), _ptr(a, w), _ptr(b, w), N, limbs, count, m, tables.handle,
                                 _stream(stream)))
 
 
@@ -380,7 +390,7 @@ def negacyclic_mul(c, a, b, N, limbs, count, tables: NttTables, moduli=None, str
     (coefficient domain in and out)."""
     m = _moduli_arg(tables, limbs, moduli)
     w = N * limbs * count
-    _check(load().he_negacyclic_mul(_ptr(c, w), _ptr(a, w), _ptr(b, w), N, limbs, count, _hp(m), tables.handle,
+    _check(load().he_negacyclic_mul(_ptr(c, w), _ptr(a, w), _ptr(b, w), N, limbs, count, m, tables.handle,
                                     _stream(stream)))
 
 
