@@ -12,8 +12,20 @@ namespace he {
 // ============================================================ plain NTT ====
 
 // Load of a word the kernel does not write (a kernel ahead in the stream may
-// have: see stream_order).
-__device__ __forceinline__ u64 rd(const u64 *p) { return *p; }
+// have: see stream_order); volatile, so that it stays behind the wait.
+__device__ __forceinline__ u64 rd(const u64 *p)
+{
+    u64 v;
+    asm volatile("ld.global.u64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
+
+__device__ __forceinline__ ulonglong2 rd2(const u64 *p)
+{
+    ulonglong2 v;
+    asm volatile("ld.global.v2.u64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
 
 // Bulk tensor store of the forward transform's output (one warp, 16 words
 // a thread: thread l of warp w holds the 16 words of row row0 + 32 w + l of
@@ -504,9 +516,9 @@ k_ct_matmul_tensor(u64 *t, const u64 *a, const u64 *b, u32 m, u32 k, u32 n, u32 
         for (u32 l = l0; l < l1; l++) {
             u64 a0[TI], a1[TI], b0[TJ], b1[TJ];
 #pragma unroll
-            for (int i = 0; i < TI; i++) a0[i] = rd(ap[i]), a1[i] = rd(ap[i] + poly), ap[i] += 2 * poly;
+            for (int i = 0; i < TI; i++) a0[i] = *ap[i], a1[i] = ap[i][poly], ap[i] += 2 * poly;
 #pragma unroll
-            for (int j = 0; j < TJ; j++) b0[j] = rd(bp[j]), b1[j] = rd(bp[j] + poly), bp[j] += bstep;
+            for (int j = 0; j < TJ; j++) b0[j] = *bp[j], b1[j] = bp[j][poly], bp[j] += bstep;
 #pragma unroll
             for (int i = 0; i < TI; i++)
 #pragma unroll
@@ -705,7 +717,7 @@ struct DSource {
     __device__ __forceinline__ ulonglong2 pair(const u64 *row, u32 log_n, u32 P) const
     {
         const u32 src = galois ? automorph_index(P, log_n, galois) : P;
-        const ulonglong2 v = *reinterpret_cast<const ulonglong2 *>(row + (src & ~1u));
+        const ulonglong2 v = rd2(row + (src & ~1u));
         return (src & 1u) ? make_ulonglong2(v.y, v.x) : v;
     }
 };
@@ -965,7 +977,7 @@ struct MacVec {
     u64 v[2];
     __device__ __forceinline__ static MacVec load(const u64 *p)
     {
-        const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(p);
+        const ulonglong2 t = rd2(p);
         return {{t.x, t.y}};
     }
     __device__ __forceinline__ static MacVec key(const u64 *p)   // read-only path: key words
@@ -1364,7 +1376,7 @@ __device__ __forceinline__ void mrr_rest_body(const EvalArgs &a, u32 item, u32 m
     u64 x[Sh::E];
     auto nost = [&](u32, u64) {};
     auto ld = [&](int P) -> u64 { return lift(rd(yP + P), rd(al + P), pc); };
-    ntt_fwd_block<Sh, false>(smem, m, rbase, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, nost, x);
+    ntt_fwd_block<Sh, false, true>(smem, m, rbase, a.ctx.tw_fwd + (size_t)i * Sh::N, pc, ld, nost, x);
     const u64 *accp = a.accq + (((size_t)c * 2 + k) * n + i) * Sh::N;
     u64 *out = a.out + (((size_t)c * 2 + k) * l + i) * Sh::N;
     sub_scale_run<Sh>(x, accp, C, C_sh, pc, m, tid);

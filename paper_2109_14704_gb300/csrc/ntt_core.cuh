@@ -431,14 +431,19 @@ __device__ __forceinline__ void fwd_rounds(u64 (&x)[Sh::E], u64 *s, u32 tid, u32
 // then either scatter into the owning CTAs' shared memory (ranks rbase ..
 // rbase + C - 1 of the cluster) or keep the results for the owners to pull
 // (Sh::FWD_PULL), cluster barrier.
-template <class Sh, class Load>
+// ROLL: columns eight words at a time instead of all unrolled, for callers whose
+// load is long (its code is repeated for every word: with 16 copies of the
+// rest stage's load warps waited for instructions, 173 -> 159 us for 768 limbs
+// of 2^14); with a plain load all columns in flight are 2 % faster.
+template <class Sh, bool ROLL, class Load>
 __device__ __forceinline__ void fwd_cross(u64 *s, u32 tid, u32 m, u32 rbase, const ulonglong2 *tw,
                                           const PrimeConst &pc, Load &load)
 {
     constexpr u32 C = Sh::C;
     constexpr int COLS = Sh::E / (int)C;
     const u32 s_base = smem_u32(s);
-#pragma unroll
+    constexpr int UN = ROLL ? (C < 8 ? 8 / (int)C : 1) : COLS;
+#pragma unroll(UN)
     for (int c = 0; c < COLS; c++) {
         const int j = (int)(m * (Sh::B / C)) + c * (int)Sh::T + (int)tid;
         u64 v[C];
@@ -480,14 +485,14 @@ __device__ __forceinline__ void fwd_cross(u64 *s, u32 tid, u32 m, u32 rbase, con
 // (see last_pos). With CANON = false the final reduction is skipped: x[] and
 // store receive values in [0, 8p + 2^32), below 12p for p >= 2^30, for
 // callers that feed them straight into a Shoup product (any 64-bit input).
-template <class Sh, bool CANON = true, class Load, class Store>
+template <class Sh, bool CANON = true, bool ROLL = false, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_block(u64 *s, u32 m, u32 rbase, const ulonglong2 *tw,
                                               const PrimeConst &pc, Load load, Store store, u64 (&x)[Sh::E])
 {
     const u32 tid = threadIdx.x;
     using R0 = RoundOf<Sh, 0>;
     if constexpr (Sh::LOG_C > 0) {
-        fwd_cross<Sh>(s, tid, m, rbase, tw, pc, load);
+        fwd_cross<Sh, ROLL>(s, tid, m, rbase, tw, pc, load);
         if constexpr (Sh::FWD_PULL) {
             constexpr int LOG_W = Sh::LOG_B - Sh::LOG_C;
             const u32 s_base = smem_u32(s);
@@ -636,7 +641,11 @@ __device__ __forceinline__ void ntt_inv_block(u64 *s, u32 m, u32 rbase, const ul
         constexpr int COLS = Sh::E / (int)C;
         const u32 s_base = smem_u32(s);
         u64 fold = 0;   // every word read from the peers, for the final barrier
-#pragma unroll
+        // columns eight words at a time: unrolled over all 16 words the code costs
+        // more in instruction fetches than it gains (259 limbs of 2^14 45.3 ->
+        // 43.2 us, the uneven batch of 512 polynomials 657 -> 648)
+        constexpr int UN = C < 8 ? 8 / (int)C : 1;
+#pragma unroll(UN)
         for (int c = 0; c < COLS; c++) {
             const int j = (int)(m * (Sh::B / C)) + c * (int)Sh::T + (int)tid;
             const u32 a = s_base + swz<Sh::LOG_E>((u32)j) * 8u;
