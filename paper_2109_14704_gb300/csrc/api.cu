@@ -413,28 +413,37 @@ static int num_sms()
     return g_num_sms;
 }
 
-// Batches of at most this many words take the radix-8 shapes: 8 words a thread
-// put twice the threads on the batch and halve each one's chain of butterflies,
-// which is what a launch costs that does not fill the GPU (512 threads an SM);
-// above it the 16-word shapes' fewer exchanges win. Measured, 60-bit prime,
-// forward, 16 / 8 words a thread: one limb of 2^12 8.5 / 7.0 us, of 2^15 11.3 /
-// 9.4; 2^19 words in all 8.9 / 7.2 (2^12), 14.8 / 14.5 (2^15); 2^20 words 11.6 /
-// 11.7 and 16.7 / 15.5; 2^21 words 19.9 / 20.9 and 25.6 / 32.2.
+// Batches of at most this many words are small: one 512-thread CTA an SM of
+// the 8-word shapes covers them.
 static u64 small_batch_words() { return (u64)num_sms() * 4096; }
 
-// Shape of a batch of `items` limbs when none is set for the degree.
-//   2^10 .. 2^15, small batch: one block of 8-word threads where the degree fits
-//     it, 2^12-word blocks above; 2^13 in four 2^11-word blocks of 16-word
-//     threads while those leave SMs idle (inverse 8.1 us against 8.7).
-//   2^16: 2^12-word blocks in clusters of 16 at every size (one limb 12.2 us
-//     against 17.3 with 2^13-word blocks, 128 limbs 101 against 117).
-static void auto_shape(int log_n, u32 items, int *lb, int *le)
+// Shape of a batch of `items` limbs when none is set for the degree (0, 0: the
+// default, 16 words a thread). Small batches take 8 words a thread, in one CTA
+// up to 2^12 and in 2^12-word blocks above: twice the threads on the batch, and
+// half the chain of butterflies in each, which is what a launch costs that does
+// not fill the GPU. Above the limit the 16-word shapes' fewer exchanges win.
+// Measured against the default, forward / inverse, us:
+//   2^10: 76 limbs 6.4 / 5.8 -> 4.5 / 4.6, 608 7.9 / 7.3 -> 6.5 / 6.2
+//   2^12: 19 limbs 8.4 / 8.5 -> 7.1 / 6.9, 152 8.7 / 8.9 -> 7.1 / 7.2; equal at
+//     256, 5 % slower at 512
+//   2^13: 76 limbs 10.1 / 10.4 -> 9.0 / 8.9; up to 19 limbs four 2^11-word blocks
+//     of 16-word threads, 9.9 / 10.3 -> 8.7 / 8.5
+//   2^14: 33 limbs 10.8 / 10.1 -> 8.9 / 9.0; 2^15: 14 limbs 11.4 / 11.2 -> 9.7 / 9.5.
+//     Clusters of four and eight do not reach every SM: with more than 3/4 of
+//     the words (38 and 16 limbs) a second CTA lands on some, 13.7 / 14.4
+//     against 11.5 / 11.3. The inverse of up to 8 limbs of 2^14 is 2 % faster
+//     in the default.
+//   2^16: 2^12-word blocks in clusters of 16 at every size (one limb 17.3 -> 12.2,
+//     128 limbs 117 / 109 -> 101 / 102).
+static void auto_shape(int log_n, u32 items, bool inv, int *lb, int *le)
 {
+    const u64 words = (u64)items << log_n, small = small_batch_words();
     if (log_n == 16) {
         *lb = 12, *le = 4;
-    } else if (((u64)items << log_n) <= small_batch_words()) {
-        if (log_n == 13 && items * 4 <= (u32)num_sms()) *lb = 11, *le = 4;
-        else *lb = std::min(log_n, 12), *le = 3;
+    } else if (log_n == 13 && items * 8 <= (u32)num_sms()) {
+        *lb = 11, *le = 4;
+    } else if (log_n >= 14 ? words <= small / 4 * 3 && !(log_n == 14 && inv && items <= 8) : words <= small) {
+        *lb = std::min(log_n, 12), *le = 3;
     }
 }
 
@@ -486,7 +495,8 @@ static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaSt
     const he::DegreeOps *ops = he::degree_ops(log_n);
     int lb = g_shape_b[inv][log_n].load(), le = g_shape_e[inv][log_n].load();
     const bool persistent = g_shape_persistent[inv][log_n].load() != 0;
-    if (!lb && !le && !persistent) auto_shape(log_n, a0.items, &lb, &le);
+    const bool set = lb || le || persistent;
+    if (!set) auto_shape(log_n, a0.items, inv, &lb, &le);
     he::NttLaunch a = a0;
     const u32 resident = (u32)std::max(ops->max_clusters(lb, le, inv), 1);
 #ifndef HE_NO_L2_PREFETCH
@@ -497,10 +507,10 @@ static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaSt
     if (persistent) {
         HE_CUDA(ops->ntt_persistent(a, lb, le, inv, std::min<u32>(a.items, resident), stream));
     } else {
-        // le = 0: the degree's default, 16 words a thread; from 32 MB on, where
-        // the 2 % they give (2477 -> 2425 us for 8192 limbs of 2^15) is more than
-        // the host's time to encode the tensor map
-        const bool tma = !inv && (le == 4 || (le == 0 && ((u64)a.items << log_n) >= (1u << 22)));
+        // with no shape set, where the batch is not small: 2477 -> 2425 us for
+        // 8192 limbs of 2^15, 12.3 -> 11.5 for 38 of 2^14; for a smaller one the
+        // host's time to encode the tensor map outweighs the gain
+        const bool tma = !inv && (set ? le == 4 : ((u64)a.items << log_n) > small_batch_words());
         a.tma_store = (tma && batch_tmap(a, 1u << log_n)) ? 1u : 0u;
         HE_CUDA(ops->ntt(a, lb, le, inv, stream));
     }
@@ -613,7 +623,12 @@ extern "C" he_status he_negacyclic_mul(uint64_t *c, const uint64_t *a, const uin
     L.tw_inv = tw->d_inv;
     L.pc = tw->d_pc;
     int lb = g_shape_b[0][log_n].load(), le = g_shape_e[0][log_n].load();
-    if (!lb && !le) auto_shape(log_n, (u32)items, &lb, &le);
+    if (!lb && !le) {
+        // three transforms in a row: at 2^13 the four 2^11-word blocks hold out
+        // longer (27 limbs 20.5 us against 21.9 with one 8-word-thread pair)
+        if (log_n == 13 && items * 4 <= (u64)num_sms()) lb = 11, le = 4;
+        else auto_shape(log_n, (u32)items, false, &lb, &le);
+    }
     HE_CUDA(he::degree_ops(log_n)->negacyclic(L, lb, le, (cudaStream_t)stream));
     return HE_OK;
 }

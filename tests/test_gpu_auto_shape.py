@@ -24,7 +24,8 @@ def test_auto_shape_sides(log_n):
     r = Rng(log_n)
     row = r.uniform_limbs(qs, N)
     want_f, want_i = oracle.ntt_fwd(row, qs)[0], oracle.ntt_inv(row, qs)[0]
-    for count in sorted({1, 2, sms // 4, sms // 4 + 1, limit, limit + 1} - {0}):
+    edges = [1, 8, sms // 8, limit * 3 // 4, limit]
+    for count in sorted({c + d for c in edges for d in (0, 1)} - {0}):
         for f, want in ((he.ntt_fwd, want_f), (he.ntt_inv, want_i)):
             d = dev(row).repeat(count, 1).contiguous()
             f(d, N, 1, count, t)
