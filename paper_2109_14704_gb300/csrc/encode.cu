@@ -277,10 +277,10 @@ __device__ __forceinline__ double mw_to_double(u64 (&v)[NW])
 // message, so below q_0 / 2. If the residue mod q_0, centred, has the given
 // residues mod every other prime, it is the lift (the centred lift is unique),
 // and neither products nor multi-word sums are needed: one reduction a limb
-// instead of 4 NW products and the corrections. Anything else fails in the
-// first four limbs with all but a 2^-30 chance and takes the general path. Bound by
+// instead of 4 NW products and the corrections. Anything else fails at the
+// second limb with all but a 2^-30 chance and takes the general path. Bound by
 // its reads then: 64 messages of 2^15 coefficients at 8 limbs (151 MB), 205 us
-// by the general path, 40 us by this one. primes: (q_i, floor(2^64 / q_i)).
+// by the general path, 44 us by this one. primes: (q_i, floor(2^64 / q_i)).
 template <int NW>
 __global__ void __launch_bounds__(128) k_crt_compose(double *out, const u64 *coef, const u64 *tab, const u64 *primes,
                                                      u32 log_N, u32 limbs, u64 total)
@@ -302,17 +302,20 @@ __global__ void __launch_bounds__(128) k_crt_compose(double *out, const u64 *coe
         const u64 q0 = primes[0];
         const bool neg = r[0] > q0 / 2;
         const u64 mag = neg ? q0 - r[0] : r[0];          // |x|
-        bool small = r[0] < q0;
-        for (u32 i0 = 0;;) {
+        auto agrees = [&](u32 i, u64 word) {
+            const u64 q = primes[2 * i], v = mul_shoup(mag, 1, primes[2 * i + 1], q);
+            return word == (neg && v ? q - v : v);
+        };
+        bool small = r[0] < q0 && (limbs < 2 || agrees(1, r[1]));
+        if (small) {
+            for (u32 i0 = 0;;) {
 #pragma unroll
-            for (u32 i = 0; i < 4; i++) {
-                if (i0 + i == 0 || i0 + i >= limbs) continue;
-                const u64 q = primes[2 * (i0 + i)], v = mul_shoup(mag, 1, primes[2 * (i0 + i) + 1], q);
-                small &= r[i] == (neg && v ? q - v : v);
+                for (u32 i = 0; i < 4; i++)
+                    if (i0 + i >= 2 && i0 + i < limbs) small &= agrees(i0 + i, r[i]);
+                i0 += 4;
+                if (!small || i0 >= limbs) break;
+                load4(i0);
             }
-            i0 += 4;
-            if (!small || i0 >= limbs) break;
-            load4(i0);
         }
         if (small) {
             const double d = __ull2double_rn(mag);

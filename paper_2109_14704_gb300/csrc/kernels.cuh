@@ -632,7 +632,8 @@ __device__ __forceinline__ u64 centred_mod(u64 y, u64 half_m, u64 m_mod_q, const
 
 // a - x + 12p: congruent to a - x mod p and positive for a < 2^63 - 12p and
 // x < 12p (a lazy forward-transform output, see ntt_fwd_block with CANON =
-// false); below 2^64 for a < 2p, so it can go straight into mul_shoup.
+// false); below 2^64 for a < 4p (the stored accumulators), so it can go
+// straight into mul_shoup.
 __device__ __forceinline__ u64 lazy_sub(u64 a, u64 x, u64 twelve_p) { return a + twelve_p - x; }
 
 // Epilogue of a lazy forward transform (ntt_fwd_block with CANON = false):
