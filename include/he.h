@@ -138,8 +138,8 @@ he_status he_ntt_inv_naive(uint64_t *poly, uint32_t N, uint32_t limbs, uint32_t 
 he_status he_ntt_shapes(uint32_t N, uint32_t *shapes_out, uint32_t cap, uint32_t *n_out);
 
 /* Shape used from now on by he_ntt_fwd (direction 1), he_ntt_inv (2) or
- * both (0) at degree N (process wide; all zero restores the built-in
- * default). persistent != 0 launches a fixed grid of as many clusters as fit
+ * both (0) at degree N (process wide; all zero, the initial state, lets each
+ * call choose by the size of its batch). persistent != 0 launches a fixed grid of as many clusters as fit
  * on the GPU, each walking over the limbs, instead of one cluster per limb;
  * ctas_per_sm selects a build of the shape for that register budget (0 =
  * default; he_ntt_shapes lists the builds). The autotuner's choices are
@@ -160,7 +160,8 @@ he_status he_dyadic_mul(uint64_t *out, const uint64_t *a, const uint64_t *b, uin
  * both forward transforms, the pointwise product and the inverse transform
  * with the data on chip (16 bytes read and 8 written per word, against 72
  * for he_ntt_fwd x 2 + he_dyadic_mul + he_ntt_inv). The transform shape is
- * the forward shape set for N (he_ntt_set_shape). c may equal a or b; any
+ * the forward shape set for N (he_ntt_set_shape), or one for the batch's size
+ * where none is set. c may equal a or b; any
  * other overlap is HE_EINVAL. Same layout and checks as he_ntt_fwd. */
 he_status he_negacyclic_mul(uint64_t *c, const uint64_t *a, const uint64_t *b, uint32_t N,
                             uint32_t limbs, uint32_t count, const uint64_t *moduli_host,
@@ -179,8 +180,8 @@ he_status he_context_create(uint32_t N, uint32_t n_data, const uint64_t *data_mo
 he_status he_context_destroy(he_context *ctx);
 
 /* Words per thread of the context's key-switching and rescale kernels:
- * 2^3 (radix-8 register rounds) or 2^4 (radix-16, the default; 0 restores
- * it). The autotuner times both. */
+ * 2^3 (radix-8 register rounds) or 2^4 (radix-16); 0, the initial state, lets
+ * each stage choose by its size. The autotuner times both. */
 he_status he_context_set_eval_shape(he_context *ctx, uint32_t log_thread_words);
 
 /* Upload a relinearization key (the evk of Relin, Sec. II-A; a Galois key
@@ -188,7 +189,8 @@ he_status he_context_set_eval_shape(he_context *ctx, uint32_t log_thread_words);
  * NTT domain: digit j, component k, limbs q_0..q_L then P; it must satisfy
  * evk[j][0] + evk[j][1] s = e_j + [j = i] (P mod q_i) s^2 on limb q_i (and no
  * s^2 term on P), i.e. one RNS digit per data prime and one special prime.
- * The device copy stores each word with its Shoup quotient. Synchronises. */
+ * The device copy stores each word with its Shoup quotient and once more in
+ * the form of the key sums, 24 bytes a word in all. Synchronises. */
 he_status he_relin_key_upload(const he_context *ctx, const uint64_t *evk_host,
                               he_relin_key **out);
 he_status he_relin_key_destroy(he_relin_key *key);
