@@ -886,9 +886,15 @@ static he_status run_eval(const he_context *ctx, he::EvalKernel k, const he::Eva
     if (!items) return HE_OK;
     // unset: 8 words a thread up to twice the transforms' limit (the stages load
     // and finish more per word): one product at 2^14, 7 + 1 primes 69 -> 57 us,
-    // four 98 -> 97, from eight on the same within 1 %
+    // four 98 -> 97, from eight on the same within 1 %. The fused mod-up runs a
+    // transform per digit in each CTA and gains only up to the transforms' own
+    // limit: at 2^14, 7 + 1 primes one product 101 -> 79 us, four 155 -> 123; at
+    // 2^15, 8 + 1 primes two 265 -> 261, but four 297 -> 383 and 32 2018 -> 2381
     int log_e = ctx->eval_log_e.load();
-    if (!log_e) log_e = ((u64)items << ctx->log_n) <= 2 * small_batch_words() ? 3 : 4;
+    if (!log_e) {
+        const u64 limit = (k == he::EK_KS_MODUP ? 1 : 2) * small_batch_words();
+        log_e = ((u64)items << ctx->log_n) <= limit ? 3 : 4;
+    }
     HE_CUDA(he::degree_ops(ctx->log_n)->eval(k, a, items, log_e, jobs, s));
     return HE_OK;
 }

@@ -11,7 +11,7 @@ from paper_2109_14704_gb300.synth import Rng
 torch = pytest.importorskip("torch")
 pytestmark = pytest.mark.gpu
 
-from tests.gpu_util import dev, host  # noqa: E402
+from tests.gpu_util import dev, empty, host  # noqa: E402
 
 
 @pytest.mark.parametrize("log_n", range(10, 17))
@@ -37,3 +37,22 @@ def test_auto_shape_sides(log_n):
         if count == 1:
             want_c = oracle.negacyclic_mul(row, row, qs)[0]
         assert (host(c) == want_c).all(), count
+
+
+@pytest.mark.parametrize("log_n", [12, 15, 16])
+def test_auto_shape_fused_modup(log_n):
+    """The product at minimum scratch, on both sides of the fused mod-up's limit."""
+    N, n = 1 << log_n, 2
+    data, P = he.chain_primes(N, [50] * n, 60)
+    r = Rng(log_n)
+    evk = np.stack([np.stack([r.uniform_limbs(data + [P], N) for _ in range(2)]) for _ in range(n)])
+    ct = np.stack([r.uniform_limbs(data, N) for _ in range(2)])
+    want = oracle.mul_relin_rescale(ct, ct, evk, data, P, n - 1)
+    ctx = he.Context(N, data, P)
+    key = he.RelinKey(ctx, evk)
+    limit = torch.cuda.get_device_properties(0).multi_processor_count * 4096 // N // (n + 1)
+    for count in (limit, limit + 1):
+        a = dev(ct[None]).repeat(count, 1, 1, 1).contiguous()
+        out = empty(count, 2, n - 1, N)
+        he.mul_relin_rescale(out, a, a, count, key, ctx, n - 1, empty(ctx.mrr_scratch_bytes(n - 1, count, 0) // 8))
+        assert (host(out) == want).all(), count
