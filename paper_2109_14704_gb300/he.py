@@ -458,6 +458,10 @@ class Context:
             pass
 
 
+# device bytes a word of an uploaded key holds (he_relin_key_upload)
+KEY_BYTES_PER_WORD = 24
+
+
 class RelinKey:
     """he_relin_key: evk [n_data][2][n_data+1][N] (host array) uploaded."""
 

@@ -43,6 +43,7 @@ from dataclasses import dataclass, field
 import numpy as np
 
 from . import he
+from .he import KEY_BYTES_PER_WORD
 from .synth import Rng
 
 
@@ -203,8 +204,8 @@ class Server:
             evk = np.stack([np.stack([self.rng.uniform_limbs(data + [P], N) for _ in range(2)])
                             for _ in range(n_data)])
             self.key[N] = he.RelinKey(self.ctx[N], evk)
-            # resident: key words with Shoup quotients, twiddles of n_data+1 primes, constants
-            self.static_bytes += evk.size * 16 + (n_data + 1) * N * 32
+            # resident: the key, twiddles of n_data + 1 primes
+            self.static_bytes += evk.size * KEY_BYTES_PER_WORD + (n_data + 1) * N * 32
         # Client-side input pool: pinned host ciphertext pairs per (N, level)
         # (or another server's pool over the same degrees and levels).
         self.pool = pool if pool is not None else {}

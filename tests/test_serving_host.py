@@ -13,6 +13,8 @@ compared with that function of the request's own pooled input, so a request
 routed to another slot, bucket or stride fails. The real kernels behind the
 same server are tested on the GPU by tests/test_gpu_runtime.py."""
 import contextlib
+import pathlib
+import re
 import time
 
 import numpy as np
@@ -288,3 +290,15 @@ def test_no_room_for_a_single_batch_is_an_error_not_a_hang(fake):
     with pytest.raises(MemoryError, match="budget"):
         srv.run(_reqs([(0.0, 32, 3)]))
     assert srv.cache.reserved == 0
+
+
+def test_ledger_counts_the_resident_keys(fake):
+    """The bytes held before any batch are those the header states for an
+    uploaded key, and 32 a twiddle pair."""
+    header = (pathlib.Path(__file__).parents[1] / "include" / "he.h").read_text()
+    per_word = int(re.search(r"(\d+) bytes a word in all", header).group(1))
+    fake(0.001)
+    srv = _server(degrees=(16, 32), max_level=4)
+    nd = 5
+    assert srv.static_bytes == sum(nd * 2 * (nd + 1) * N * per_word + (nd + 1) * N * 32 for N in (16, 32))
+    assert srv.ledger() == srv.static_bytes
