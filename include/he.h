@@ -189,8 +189,8 @@ he_status he_context_set_eval_shape(he_context *ctx, uint32_t log_thread_words);
  * NTT domain: digit j, component k, limbs q_0..q_L then P; it must satisfy
  * evk[j][0] + evk[j][1] s = e_j + [j = i] (P mod q_i) s^2 on limb q_i (and no
  * s^2 term on P), i.e. one RNS digit per data prime and one special prime.
- * The device copy stores each word with its Shoup quotient and once more in
- * the form of the key sums, 24 bytes a word in all. Synchronises. */
+ * The device copy stores each word in the form of the key sums with its Shoup
+ * quotient, 16 bytes a word in all (no more during the call). Synchronises. */
 he_status he_relin_key_upload(const he_context *ctx, const uint64_t *evk_host,
                               he_relin_key **out);
 he_status he_relin_key_destroy(he_relin_key *key);

@@ -651,8 +651,8 @@ struct he_context {
 
 struct he_relin_key {
     const he_context *ctx = nullptr;
-    ulonglong2 *d_evk = nullptr;       // (word, Shoup quotient): the fused mod-up
-    u64 *d_mac = nullptr;              // the multiply-accumulate's words
+    u64 *d_mac = nullptr;              // the key sums' words
+    u64 *d_sh = nullptr;               // their Shoup quotients: the fused mod-up
 };
 
 template <class T>
@@ -771,21 +771,18 @@ extern "C" he_status he_relin_key_upload(const he_context *ctx, const uint64_t *
     }
     he_relin_key *key = new he_relin_key;
     key->ctx = ctx;
-    u64 *raw = nullptr;
-    cudaError_t e = cudaMalloc(&key->d_evk, words * sizeof(ulonglong2));
-    if (e == cudaSuccess) e = cudaMalloc(&key->d_mac, words * 8);
-    if (e == cudaSuccess) e = cudaMalloc(&raw, words * 8);
-    if (e == cudaSuccess) e = cudaMemcpy(raw, evk_host, words * 8, cudaMemcpyHostToDevice);
+    cudaError_t e = cudaMalloc(&key->d_mac, words * 8);
+    if (e == cudaSuccess) e = cudaMalloc(&key->d_sh, words * 8);
+    if (e == cudaSuccess) e = cudaMemcpy(key->d_mac, evk_host, words * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess) {
-        he::k_key_prepare<<<stream_grid(words, 256), 256>>>(key->d_evk, key->d_mac, raw, words, (u32)ctx->log_n, nd,
+        he::k_key_prepare<<<stream_grid(words, 256), 256>>>(key->d_mac, key->d_sh, words, (u32)ctx->log_n, nd,
                                                             ctx->tables->d_pc, ctx->d_limb, ctx->R_special);
         e = cudaGetLastError();
         if (e == cudaSuccess) e = cudaStreamSynchronize(nullptr);
     }
-    cudaFree(raw);
     if (e != cudaSuccess) {
-        cudaFree(key->d_evk);
         cudaFree(key->d_mac);
+        cudaFree(key->d_sh);
         delete key;
         return fail(e == cudaErrorMemoryAllocation ? HE_ENOMEM : HE_ECUDA, "relin key upload: %s",
                     cudaGetErrorString(e));
@@ -798,8 +795,8 @@ extern "C" he_status he_relin_key_destroy(he_relin_key *key)
 {
     if (key) {
         cudaDeviceSynchronize();
-        cudaFree(key->d_evk);
         cudaFree(key->d_mac);
+        cudaFree(key->d_sh);
         delete key;
     }
     return HE_OK;
@@ -888,8 +885,8 @@ static he_status run_eval(const he_context *ctx, he::EvalKernel k, const he::Eva
     // and finish more per word): one product at 2^14, 7 + 1 primes 69 -> 57 us,
     // four 98 -> 97, from eight on the same within 1 %. The fused mod-up runs a
     // transform per digit in each CTA and gains only up to the transforms' own
-    // limit: at 2^14, 7 + 1 primes one product 101 -> 79 us, four 155 -> 123; at
-    // 2^15, 8 + 1 primes two 265 -> 261, but four 297 -> 383 and 32 2018 -> 2381
+    // limit: at 2^14, 7 + 1 primes one product 96 -> 72 us, four 128 -> 107; at
+    // 2^15, 8 + 1 primes two 234 -> 225, but four 267 -> 320 and 32 1800 -> 1958
     int log_e = ctx->eval_log_e.load();
     if (!log_e) {
         const u64 limit = (k == he::EK_KS_MODUP ? 1 : 2) * small_batch_words();
@@ -999,8 +996,8 @@ extern "C" he_status he_relin(uint64_t *ct_out2, const uint64_t *ct_in3, const h
     a.c2 = (u64 *)scratch;
     a.accq = a.c2 + (size_t)n * ctx->N;
     a.plift = a.accq + (size_t)2 * n * ctx->N;
-    a.evk = key->d_evk;
     a.evk_mac = key->d_mac;
+    a.evk_sh = key->d_sh;
     a.n = n;
     a.count = 1;
     a.ctx = dev_ctx(ctx);
@@ -1070,8 +1067,8 @@ static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const
     a.accq = a.c2 + (size_t)count * n * ctx->N;
     a.plift = a.accq + (size_t)count * 2 * n * ctx->N;
     a.lift2 = rescale ? a.plift + (size_t)count * 2 * ctx->N : nullptr;
-    a.evk = key->d_evk;
     a.evk_mac = key->d_mac;
+    a.evk_sh = key->d_sh;
     a.n = n;
     a.count = count;
     a.ctx = dev_ctx(ctx);

@@ -843,8 +843,11 @@ k_ks_modup(EvalArgs a)
     u64 x[Sh::E];
     for (u32 j = 0; j < n; j++) {
         if (t == j) {
+            // the NTT-domain digit times 2^-64, which its key words take off
+            const LimbConst &lc = a.ctx.limb[t];
 #pragma unroll
-            for (int e = 0; e < Sh::E; e++) x[e] = ds.d(2, j, Sh::LOG_N, last_pos<Sh>(m, tid, e), pc);
+            for (int e = 0; e < Sh::E; e++)
+                x[e] = mul_shoup_lazy4_asm(ds.d(2, j, Sh::LOG_N, last_pos<Sh>(m, tid, e), pc), lc.k2, lc.k2_sh, pc.neg_p);
         } else {
             if (j > 0) ntt_barrier<Sh>();
             const u64 *src = a.c2 + ((size_t)c * n + j) * Sh::N;
@@ -862,21 +865,29 @@ k_ks_modup(EvalArgs a)
             }
         }
         // multiply-accumulate with the key: lazy products in [0, 4p),
-        // accumulators kept in [0, 4p)
+        // accumulators kept in [0, 4p). Words and quotients come from two arrays
+        // in 256-bit loads (64 products at 2^14, 7 + 1 primes, 1278 us; with
+        // 128-bit loads 1467, with interleaved pairs in 128-bit loads 1404)
 #pragma unroll
         for (int k = 0; k < 2; k++) {
-            const ulonglong2 *key = a.evk + (((size_t)j * 2 + k) * (a.ctx.n_data + 1) + tp) * Sh::N;
+            const size_t row = (((size_t)j * 2 + k) * (a.ctx.n_data + 1) + tp) * Sh::N;
 #pragma unroll
-            for (int e = 0; e < Sh::E; e++) {
-                const ulonglong2 w = __ldg(key + last_pos<Sh>(m, tid, e));
-                const u64 prod = mul_shoup_lazy4_asm(x[e], w.x, w.y, pc.neg_p);
-                u64 &slot = acc[(k * Sh::E + e) * Sh::T + tid];
-                slot = (j == 0) ? prod : reduce_once(slot + prod, pc.four_p);
+            for (int e = 0; e < Sh::E; e += 4) {
+                const size_t at = row + last_pos<Sh>(m, tid, e);
+                u64 w[4], w_sh[4];
+                ld4_nc(a.evk_mac + at, w[0], w[1], w[2], w[3]);
+                ld4_nc(a.evk_sh + at, w_sh[0], w_sh[1], w_sh[2], w_sh[3]);
+#pragma unroll
+                for (int i = 0; i < 4; i++) {
+                    const u64 prod = mul_shoup_lazy4_asm(x[e + i], w[i], w_sh[i], pc.neg_p);
+                    u64 &slot = acc[(k * Sh::E + e + i) * Sh::T + tid];
+                    slot = (j == 0) ? prod : reduce_once(slot + prod, pc.four_p);
+                }
             }
         }
     }
     if (t < n) {
-        // (acc_k P^-1 + d_k) 2^-64, below 4 q_t
+        // (acc_k P^-1 + d_k) 2^-64, below 4 q_t (the key words hold P^-1)
         const LimbConst lc = a.ctx.limb[t];
 #pragma unroll
         for (int k = 0; k < 2; k++) {
@@ -884,19 +895,19 @@ k_ks_modup(EvalArgs a)
 #pragma unroll
             for (int e = 0; e < Sh::E; e++) {
                 const int P = last_pos<Sh>(m, tid, e);
-                const u64 s = mul_shoup_lazy4_asm(acc[(k * Sh::E + e) * Sh::T + tid], lc.k1, lc.k1_sh, pc.neg_p);
+                const u64 s = mul_shoup_lazy4_asm(acc[(k * Sh::E + e) * Sh::T + tid], lc.k2, lc.k2_sh, pc.neg_p);
                 const u64 d = mul_shoup_lazy4_asm(ds.d(k, t, Sh::LOG_N, (u32)P, pc), lc.k2, lc.k2_sh, pc.neg_p);
                 dst[P] = reduce_once(s + d, pc.four_p);
             }
         }
     } else {
-        // special prime: y_k = INTT_P(acc_k) (inputs in [0, 4p)), kept in the
-        // coefficient domain
+        // special prime: y_k = INTT_P(acc_k), kept in the coefficient domain; the
+        // sums are 2^64 acc_k there (the key words' scale)
 #pragma unroll 1
         for (int k = 0; k < 2; k++) {
             ntt_barrier<Sh>();
 #pragma unroll
-            for (int e = 0; e < Sh::E; e++) x[e] = acc[(k * Sh::E + e) * Sh::T + tid];
+            for (int e = 0; e < Sh::E; e++) x[e] = montgomery_reduce(0, acc[(k * Sh::E + e) * Sh::T + tid], pc);
             u64 *dst = a.plift + ((size_t)c * 2 + k) * Sh::N;
             auto st = [&](u32 P, u64 v) { dst[P] = v; };
             auto ld = [&](u32) -> u64 { return 0; };
@@ -1200,11 +1211,11 @@ __global__ void __launch_bounds__(256, 4) k_ks_mac_tiled(EvalArgs a, u32 groups)
     }
 }
 
-// Device words of an uploaded key, [nd][2][nd + 1][N] canonical words raw:
-// evk = (word, Shoup quotient), evk_mac = the multiply-accumulate's word. The
-// quotient floor(w 2^64 / p) comes in two steps of 32 bits: with mu =
-// floor(2^(2b+2) / p) and r < p < 2^b, r mu / 2^(2b-30) is r 2^32 / p less
-// below one, so its floor is short by at most two.
+// Device words of an uploaded key, [nd][2][nd + 1][N] canonical words in mac:
+// replaced by the key sums' words w (scaled as EvalArgs says), with their Shoup
+// quotients in sh for the fused mod-up. The quotient floor(w 2^64 / p) comes in
+// two steps of 32 bits: with mu = floor(2^(2b+2) / p) and r < p < 2^b, r mu /
+// 2^(2b-30) is r 2^32 / p less below one, so its floor is short by at most two.
 __device__ __forceinline__ u64 shoup_step(u64 &r, const PrimeConst &c)
 {
     u64 hi, lo;
@@ -1216,22 +1227,22 @@ __device__ __forceinline__ u64 shoup_step(u64 &r, const PrimeConst &c)
     return q;
 }
 
-__global__ void k_key_prepare(ulonglong2 *evk, u64 *evk_mac, const u64 *raw, u64 words, u32 log_n, u32 nd,
-                              const PrimeConst *pcs, const LimbConst *limb, u64 R_special)
+__global__ void k_key_prepare(u64 *mac, u64 *sh, u64 words, u32 log_n, u32 nd, const PrimeConst *pcs,
+                              const LimbConst *limb, u64 R_special)
 {
     stream_order();
     for (u64 e = (u64)blockIdx.x * blockDim.x + threadIdx.x; e < words; e += (u64)gridDim.x * blockDim.x) {
         const u32 t = (u32)((e >> log_n) % (nd + 1));
         const PrimeConst pc = pcs[t];
-        const u64 w = raw[e];
-        u64 r = w;
-        const u64 qh = shoup_step(r, pc);
-        const u64 ql = shoup_step(r, pc);
-        evk[e] = make_ulonglong2(w, (qh << 32) + ql);
         const u32 j = (u32)((e >> log_n) / (2 * (nd + 1)));
         u64 f = R_special;
         if (t < nd) f = j == t ? mul_mod(limb[t].Pinv, limb[t].R, pc) : limb[t].Pinv;
-        evk_mac[e] = mul_mod(w, f, pc);
+        const u64 w = mul_mod(mac[e], f, pc);
+        u64 r = w;
+        const u64 qh = shoup_step(r, pc);
+        const u64 ql = shoup_step(r, pc);
+        mac[e] = w;
+        sh[e] = (qh << 32) + ql;
     }
 }
 #endif  // HE_MISC_KERNELS

@@ -156,8 +156,9 @@ struct EvalArgs {
     u64 *accq;                  // scratch [count][2][n][N]
     u64 *plift;                 // scratch [count][2][N]
     u64 *lift2;                 // scratch [count][2][N]
-    const ulonglong2 *evk;      // [n_data][2][n_data + 1][N] (value, Shoup quotient)
-    const u64 *evk_mac;         // same order: value P^-1 mod q_i (2^64 P^-1 for digit j = i), value 2^64 mod P on the special prime
+    // key words [n_data][2][n_data + 1][N]: value P^-1 mod q_i (2^64 P^-1 for digit
+    // j = i), value 2^64 mod P on the special prime; and their Shoup quotients
+    const u64 *evk_mac, *evk_sh;
     u64 *mx;                    // expanded mod-up scratch [group][n + 1][n][N]
     u32 n;                      // limbs at the current level
     u32 count;

@@ -185,10 +185,15 @@ __host__ __device__ __forceinline__ int inv_tw_pos(int log_n, int S, int G)
 // costs the L1 what one 128-bit access did: half the requests for the same
 // words (measured 4-5 % off both transform directions at N = 2^15).
 // _cs: streaming (data read or written once per launch). Volatile: a data
-// load must not move ahead of stream_order().
+// load must not move ahead of stream_order(). _nc: read-only path, for keys.
 __device__ __forceinline__ void ld4_cs(const u64 *p, u64 &a, u64 &b, u64 &c, u64 &d)
 {
     asm volatile("ld.global.cs.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
+}
+
+__device__ __forceinline__ void ld4_nc(const u64 *p, u64 &a, u64 &b, u64 &c, u64 &d)
+{
+    asm("ld.global.nc.v4.u64 {%0, %1, %2, %3}, [%4];" : "=l"(a), "=l"(b), "=l"(c), "=l"(d) : "l"(p));
 }
 
 // A plain load: the memory clobber keeps it ordered after this thread's

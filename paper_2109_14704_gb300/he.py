@@ -459,7 +459,7 @@ class Context:
 
 
 # device bytes a word of an uploaded key holds (he_relin_key_upload)
-KEY_BYTES_PER_WORD = 24
+KEY_BYTES_PER_WORD = 16
 
 
 class RelinKey:

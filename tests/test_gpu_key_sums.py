@@ -58,3 +58,18 @@ def test_key_sums(N, n, bits, level, fill, count):
     he.mul_relin_rescale(fused, dev(ca[:1]), dev(cb[:1]), 1, key, ctx, level,
                          empty(ctx.mrr_scratch_bytes(level, 1, 0) // 8))
     assert np.array_equal(host(fused)[0], want)
+
+
+def test_key_memory():
+    """A key's device copy holds the bytes the ledgers count for it."""
+    N, n = 32768, 8
+    data, P = he.chain_primes(N, [60] + [50] * (n - 1), 60)
+    ctx = he.Context(N, data, P)
+    evk = _largest(data + [P], N, n, 2)
+    he.RelinKey(ctx, evk).close()                   # the kernels' own memory is in place
+    free = torch.cuda.mem_get_info()[0]
+    key = he.RelinKey(ctx, evk)
+    held = free - torch.cuda.mem_get_info()[0]
+    assert he.KEY_BYTES_PER_WORD == 16
+    assert evk.size * 16 <= held <= evk.size * 16 + (8 << 20), held      # two allocations, 2 MB pages
+    key.close()
