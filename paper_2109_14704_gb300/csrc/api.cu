@@ -20,6 +20,7 @@
 
 #include "../../include/he.h"
 #include "kernels.cuh"
+#include "shape_rule.h"
 
 using he::u32;
 using he::u64;
@@ -413,39 +414,7 @@ static int num_sms()
     return g_num_sms;
 }
 
-// Batches of at most this many words are small: one 512-thread CTA an SM of
-// the 8-word shapes covers them.
-static u64 small_batch_words() { return (u64)num_sms() * 4096; }
-
-// Shape of a batch of `items` limbs when none is set for the degree (0, 0: the
-// default, 16 words a thread). Small batches take 8 words a thread, in one CTA
-// up to 2^12 and in 2^12-word blocks above: twice the threads on the batch, and
-// half the chain of butterflies in each, which is what a launch costs that does
-// not fill the GPU. Above the limit the 16-word shapes' fewer exchanges win.
-// Measured against the default, forward / inverse, us:
-//   2^10: 76 limbs 6.4 / 5.8 -> 4.5 / 4.6, 608 7.9 / 7.3 -> 6.5 / 6.2
-//   2^12: 19 limbs 8.4 / 8.5 -> 7.1 / 6.9, 152 8.7 / 8.9 -> 7.1 / 7.2; equal at
-//     256, 5 % slower at 512
-//   2^13: 76 limbs 10.1 / 10.4 -> 9.0 / 8.9; up to 19 limbs four 2^11-word blocks
-//     of 16-word threads, 9.9 / 10.3 -> 8.7 / 8.5
-//   2^14: 33 limbs 10.8 / 10.1 -> 8.9 / 9.0; 2^15: 14 limbs 11.4 / 11.2 -> 9.7 / 9.5.
-//     Clusters of four and eight do not reach every SM: with more than 3/4 of
-//     the words (38 and 16 limbs) a second CTA lands on some, 13.7 / 14.4
-//     against 11.5 / 11.3. The inverse of up to 8 limbs of 2^14 is 2 % faster
-//     in the default.
-//   2^16: 2^12-word blocks in clusters of 16 at every size (one limb 17.3 -> 12.2,
-//     128 limbs 117 / 109 -> 101 / 102).
-static void auto_shape(int log_n, u32 items, bool inv, int *lb, int *le)
-{
-    const u64 words = (u64)items << log_n, small = small_batch_words();
-    if (log_n == 16) {
-        *lb = 12, *le = 4;
-    } else if (log_n == 13 && items * 8 <= (u32)num_sms()) {
-        *lb = 11, *le = 4;
-    } else if (log_n >= 14 ? words <= small / 4 * 3 && !(log_n == 14 && inv && items <= 8) : words <= small) {
-        *lb = std::min(log_n, 12), *le = 3;
-    }
-}
+static u64 small_batch_words() { return he::small_batch_words((u32)num_sms()); }
 
 // One launch of a batch of limb transforms in the shape set for the degree.
 // cuTensorMapEncodeTiled, fetched through the runtime's driver entry points
@@ -496,7 +465,10 @@ static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaSt
     int lb = g_shape_b[inv][log_n].load(), le = g_shape_e[inv][log_n].load();
     const bool persistent = g_shape_persistent[inv][log_n].load() != 0;
     const bool set = lb || le || persistent;
-    if (!set) auto_shape(log_n, a0.items, inv, &lb, &le);
+    if (!set) {
+        const bool wide = log_n == 16 && ops->max_clusters(he::kWideLogB, 4, inv) > 0;
+        he::auto_shape(log_n, a0.items, inv, (u32)num_sms(), wide, &lb, &le);
+    }
     he::NttLaunch a = a0;
     const u32 resident = (u32)std::max(ops->max_clusters(lb, le, inv), 1);
 #ifndef HE_NO_L2_PREFETCH
@@ -623,13 +595,12 @@ extern "C" he_status he_negacyclic_mul(uint64_t *c, const uint64_t *a, const uin
     L.tw_inv = tw->d_inv;
     L.pc = tw->d_pc;
     int lb = g_shape_b[0][log_n].load(), le = g_shape_e[0][log_n].load();
+    const he::DegreeOps *ops = he::degree_ops(log_n);
     if (!lb && !le) {
-        // three transforms in a row: at 2^13 the four 2^11-word blocks hold out
-        // longer (27 limbs 20.5 us against 21.9 with one 8-word-thread pair)
-        if (log_n == 13 && items * 4 <= (u64)num_sms()) lb = 11, le = 4;
-        else auto_shape(log_n, (u32)items, false, &lb, &le);
+        const bool wide = log_n == 16 && ops->negacyclic_clusters(he::kWideLogB, 4) > 0;
+        he::product_shape(log_n, (u32)items, (u32)num_sms(), wide, &lb, &le);
     }
-    HE_CUDA(he::degree_ops(log_n)->negacyclic(L, lb, le, (cudaStream_t)stream));
+    HE_CUDA(ops->negacyclic(L, lb, le, (cudaStream_t)stream));
     return HE_OK;
 }
 

@@ -74,10 +74,29 @@ struct ShapeOps {
         static std::once_flag f;
         static cudaError_t e = cudaSuccess;
         if (smem_attr(k_ntt_persistent<LOG_B, LOG_C, LOG_E, INV, OCC>, Sh::SMEM_BYTES, f, e, Sh::C) != cudaSuccess) return 0;
+        return active_clusters(k_ntt_persistent<LOG_B, LOG_C, LOG_E, INV, OCC>, Sh::SMEM_BYTES);
+    }
+
+    static int negacyclic_clusters()
+    {
+        static std::once_flag once, f;
+        static cudaError_t e = cudaSuccess;
+        static int n = 0;
+        std::call_once(once, [] {
+            if (smem_attr(k_negacyclic<LOG_B, LOG_C, LOG_E>, 2 * Sh::SMEM_BYTES, f, e, Sh::C) == cudaSuccess)
+                n = active_clusters(k_negacyclic<LOG_B, LOG_C, LOG_E>, 2 * Sh::SMEM_BYTES);
+        });
+        return n;
+    }
+
+    // Clusters of the kernel that the GPU holds at the same time.
+    template <class K>
+    static int active_clusters(K kernel, u32 smem)
+    {
         cudaLaunchConfig_t cfg = {};
         cfg.gridDim = dim3(Sh::C * 1024, 1, 1);
         cfg.blockDim = dim3(Sh::T, 1, 1);
-        cfg.dynamicSmemBytes = Sh::SMEM_BYTES;
+        cfg.dynamicSmemBytes = smem;
         cudaLaunchAttribute attr[1];
         attr[0].id = cudaLaunchAttributeClusterDimension;
         attr[0].val.clusterDim.x = Sh::C;
@@ -86,7 +105,7 @@ struct ShapeOps {
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         int n = 0;
-        if (cudaOccupancyMaxActiveClusters(&n, k_ntt_persistent<LOG_B, LOG_C, LOG_E, INV, OCC>, &cfg) != cudaSuccess) {
+        if (cudaOccupancyMaxActiveClusters(&n, kernel, &cfg) != cudaSuccess) {
             cudaGetLastError();
             return 0;
         }
@@ -234,13 +253,18 @@ struct DegreeImpl;
         });                                                                                        \
         return found ? r : cudaErrorInvalidValue;                                                  \
     }                                                                                              \
+    static int negacl_##LOG_N_(int log_b, int log_e)                                               \
+    {                                                                                              \
+        return DegreeImpl<LOG_N_>::with_shape(log_b, log_e,                                        \
+                                              [&](auto ops) { return decltype(ops)::negacyclic_clusters(); }); \
+    }                                                                                              \
     static bool has_##LOG_N_(int log_b, int log_e)                                                 \
     {                                                                                              \
         return DegreeImpl<LOG_N_>::with_shape(log_b, log_e, [&](auto) { return true; });           \
     }                                                                                              \
     extern const DegreeOps degree_ops_##LOG_N_ = {                                                 \
         LOG_N_, DegreeImpl<LOG_N_>::def_b, DegreeImpl<LOG_N_>::def_e, ntt_##LOG_N_, ntt_p_##LOG_N_,  \
-        maxcl_##LOG_N_, eval_##LOG_N_, has_##LOG_N_, nega_##LOG_N_,                                \
+        maxcl_##LOG_N_, eval_##LOG_N_, has_##LOG_N_, nega_##LOG_N_, negacl_##LOG_N_,               \
         (int)(sizeof(DegreeImpl<LOG_N_>::shapes) / sizeof(DegreeImpl<LOG_N_>::shapes[0])),         \
         DegreeImpl<LOG_N_>::shapes};                                                               \
     }

@@ -241,6 +241,8 @@ struct DegreeOps {
     bool (*has_shape)(int log_b, int log_e);
     // Fused negacyclic product in the given transform shape (0, 0 = default).
     cudaError_t (*negacyclic)(const NegaLaunch &a, int log_b, int log_e, cudaStream_t s);
+    // Its clusters that fit on the GPU together (0: the shape cannot be placed).
+    int (*negacyclic_clusters)(int log_b, int log_e);
     // Shapes built for this degree: n pairs (log_b, log_e), default first.
     int n_shapes;
     const int (*shapes)[2];
