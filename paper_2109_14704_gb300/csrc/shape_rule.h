@@ -31,7 +31,8 @@ constexpr int kWideLogB = 12;
 //     Clusters of four and eight do not reach every SM: with more than 3/4 of
 //     the words (38 and 16 limbs) a second CTA lands on some, 13.7 / 14.4
 //     against 11.5 / 11.3. The inverse of up to 8 limbs of 2^14 is 2 % faster
-//     in the default.
+//     in the default (8.25 against 8.41; 9 to 12 limbs 1 to 2 %, 16
+//     limbs 9.43 against 8.47).
 //   2^16: 2^12-word blocks in clusters of 16 at every size (one limb 17.3 -> 12.2,
 //     128 limbs 117 / 109 -> 101 / 102).
 inline void auto_shape(int log_n, uint32_t items, bool inv, uint32_t sms, bool wide, int *lb, int *le)
@@ -47,11 +48,13 @@ inline void auto_shape(int log_n, uint32_t items, bool inv, uint32_t sms, bool w
 }
 
 // The same for the fused product. Three transforms in a row: at 2^13 the four
-// 2^11-word blocks hold out longer (27 limbs 20.5 us against 21.9 with one
-// 8-word-thread pair).
+// 2^11-word blocks hold out longer, as long as each CTA has an SM of its own.
+// Clusters of four do not reach every SM: against one pair of 8-word-thread
+// blocks, us, 27 limbs 20.5 / 21.9, 36 20.7 / 22.0, but 38 23.9 / 22.0 and 57
+// 24.5 / 22.1 (of 152 SMs; 37 like 38).
 inline void product_shape(int log_n, uint32_t items, uint32_t sms, bool wide, int *lb, int *le)
 {
-    if (log_n == 13 && (uint64_t)items * 4 <= sms)
+    if (log_n == 13 && (uint64_t)items * 4 + 8 <= sms)
         *lb = 11, *le = 4;
     else
         auto_shape(log_n, items, false, sms, wide, lb, le);

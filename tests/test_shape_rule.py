@@ -47,5 +47,7 @@ def test_choices_are_built_and_portable_where_needed(tmp_path, sms):
             lb = s[0] or built[0][0]
             assert s == (0, 0) or s in built, (log_n, items, s)
             assert wide or (1 << log_n) >> lb <= 8, (log_n, items, s)
+        if log_n == 13 and not inv and product == (11, 4):
+            assert 4 * items <= sms - 8, items       # a CTA an SM, which clusters of four do not fill
         if log_n == 16:
             assert shape == ((12, 4) if wide else (0, 0))
