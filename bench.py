@@ -503,8 +503,11 @@ def run_ours(args, rank, world, local):
                 "achieved_gbs": gbs, "hbm_frac": gbs / hbm_peak,
                 "traffic": TRAFFIC.get(key)}
 
-    roof_fwd = direction_roof("forward", fwd, tune["fwd"])
-    roof_inv = direction_roof("inverse", inv, tune["inv"])
+    # the shape that ran: the one applied, or with none set the degree's default
+    # (its choice for a batch this large)
+    lb, le, occ = he.ntt_shapes(N)[0]
+    roof_fwd = direction_roof("forward", fwd, tune["applied_fwd"] or [lb, le, 0, occ])
+    roof_inv = direction_roof("inverse", inv, tune["applied_inv"] or [lb, le, 0, occ])
     dom = roof_inv if inv >= fwd else roof_fwd          # the larger share of the step
     bound_alu = dom["alu_frac"] >= dom["hbm_frac"]
     attach_rooflines(small, alu_peak, hbm_peak)
@@ -540,9 +543,8 @@ def run_ours(args, rank, world, local):
             "fwd_ms": fwd, "inv_ms": inv, "speedup_vs_naive": ms_naive / ms,
             "step_distribution": step_dist,
         },
-        "autotune": {"forward": dict(zip(("log_block", "log_thread_words", "persistent", "ctas_per_sm"), tune["fwd"])),
-                     "inverse": dict(zip(("log_block", "log_thread_words", "persistent", "ctas_per_sm"), tune["inv"])),
-                     "reps": TUNE_REPS,
+        "autotune": {"forward": _applied(tune["applied_fwd"]), "inverse": _applied(tune["applied_inv"]),
+                     "reps": TUNE_REPS, "unset_ms_fwd": tune["unset_ms_fwd"], "unset_ms_inv": tune["unset_ms_inv"],
                      "candidates": [{"shape": c["shape"], "ms_fwd": c.get("ms_fwd"), "ms_inv": c.get("ms_inv")}
                                     for c in tune["candidates"]]},
         "small_ntt": small,
@@ -604,6 +606,11 @@ def run_ours(args, rank, world, local):
         print(json.dumps(line), flush=True)
 
 
+def _applied(shape):
+    """A tuner's applied transform shape by name; None leaves each call its own choice."""
+    return dict(zip(("log_block", "log_thread_words", "persistent", "ctas_per_sm"), shape)) if shape else "by batch size"
+
+
 def _measured_peaks() -> dict:
     try:
         return json.load(open(os.path.join(ROOT, "MEASURED_PEAKS.json")))
@@ -656,8 +663,8 @@ def bench_degrees(args, stream, barrier):
         fwd, inv = statistics.median(fwd_ms), statistics.median(inv_ms)
         items = count * limbs
         rows.append({"N": N, "polys": count, "limbs": items,
-                     "shape": ({"forward": list(tuned["fwd"]), "inverse": list(tuned["inv"])} if tuned
-                               else "the headline batch's tuned shape"),
+                     "shape": ({"forward": _applied(tuned["applied_fwd"]), "inverse": _applied(tuned["applied_inv"])}
+                               if tuned else "the headline batch's tuned shape"),
                      "fwd_ms": fwd, "inv_ms": inv, "limbs_per_s": 2 * items / ((fwd + inv) / 1e3),
                      "_work": {"bfly": 2 * items * (N // 2) * log_n, "bytes": 2 * 16 * N * items,
                                "seconds": (fwd + inv) / 1e3}})
@@ -854,7 +861,7 @@ def bench_matrix(args, stream, barrier):
     res = {"workload": "32x32 element-wise, N=8192, primes 60/40/40 + 60, 1024 MulLinRS per step",
            "ms_per_step": ms, "mul_relin_rescale_per_s": count / (ms / 1e3),
            "_work": dict({k: v * count for k, v in mrr_work(L + 1, N).items()}, seconds=ms / 1e3),
-           "eval_log_thread_words": tune["log_thread_words"]}
+           "eval_log_thread_words": tune["applied"] or "by stage size"}
     del A, B, out, scratch
     # the encrypted matrix product C += A B (matMul_mxnxk): tensors
     # accumulated over k, one relin + rescale per output, add into C

@@ -8,13 +8,16 @@ them the threads per CTA; and the CTAs per SM the kernels are compiled for,
 i.e. their register budget -- the paper tuned the same knobs by hand:
 radix, SLM threshold and register slots, Sec. III-B, Sec. IV-A), each
 launched either as one cluster per limb or as a persistent grid walking the
-limbs, and keeps the fastest for each direction. Each candidate is first checked once: its
-forward output must equal the default shape's output bit for bit and its
-inverse must restore the input exactly. Candidates are timed with CUDA
+limbs, and finds the fastest for each direction. Each candidate is first
+checked once: its forward output must equal the untuned call's bit for bit and
+its inverse must restore the input exactly. Candidates are timed with CUDA
 events (forward + inverse, median of `reps` after warm-up); the fastest wins,
-ties going to the earlier candidate. Results are cached in a JSON file keyed
-by device, N, limbs and count, and applied with he_ntt_set_shape so that the
-plain he_ntt_fwd / he_ntt_inv calls use them.
+ties going to the earlier candidate. The state with no shape set, in which
+every call chooses by the size of its batch, is timed as well: a fixed shape
+holds for every later call of the degree, small ones too, so it is only
+applied where it is faster on the tuned batch by more than MARGIN. Results are
+cached in a JSON file keyed by device, N, limbs and count, and applied with
+he_ntt_set_shape so that the plain he_ntt_fwd / he_ntt_inv calls use them.
 
 For uneven batches, tune_plan compares the single mixed-degree launch with
 per-degree launches (one cluster per limb) in each degree's tuned shape.
@@ -32,6 +35,11 @@ from .synth import Rng
 
 DEFAULT_CACHE = os.environ.get(
     "HE_AUTOTUNE_CACHE", os.path.join(os.path.expanduser("~"), ".cache", "paper_2109_14704_gb300", "autotune.json"))
+
+
+# A fixed shape must be this much faster than the unset state to be applied (two
+# runs of one kernel differ by about 1 %).
+MARGIN = 0.02
 
 
 def _load_cache(path):
@@ -82,10 +90,13 @@ def tune_uniform(N: int, limbs: int, count: int, moduli=None, reps: int = 10, wa
                  cache_path: str | None = DEFAULT_CACHE, apply: bool = True, force: bool = False) -> dict:
     """Pick, separately for he_ntt_fwd and he_ntt_inv, the fastest built
     shape (words per CTA, words per thread, one cluster per limb or
-    persistent) on `count` polynomials of `limbs` limbs at degree N."""
+    persistent) on `count` polynomials of `limbs` limbs at degree N ("fwd",
+    "inv"). What is applied ("applied_fwd", "applied_inv") is that shape, or
+    None, no fixed shape, where the call's own choice is as fast within
+    MARGIN."""
     import torch
 
-    key = f"{_device_key()}|uniform3|N={N}|limbs={limbs}|count={count}"
+    key = f"{_device_key()}|uniform4|N={N}|limbs={limbs}|count={count}"
     cache = _load_cache(cache_path) if cache_path else {}
     if not force and key in cache:
         res = cache[key]
@@ -101,11 +112,13 @@ def tune_uniform(N: int, limbs: int, count: int, moduli=None, reps: int = 10, wa
     d = torch.empty_like(x_dev)
     shapes = he.ntt_shapes(N)
 
-    # reference output: the default shape
+    # reference output and times: no shape set
     he.ntt_set_shape(N, 0, 0, 0)
     d.copy_(x_dev)
     he.ntt_fwd(d, N, limbs, count, tables)
     ref = d.clone()
+    unset_f = _time(lambda: he.ntt_fwd(d, N, limbs, count, tables), reps, warmup)
+    unset_i = _time(lambda: he.ntt_inv(d, N, limbs, count, tables), reps, warmup)
 
     cands = []
     # shape = [log_block, log_thread_words, persistent, ctas_per_sm]
@@ -131,9 +144,10 @@ def tune_uniform(N: int, limbs: int, count: int, moduli=None, reps: int = 10, wa
         raise RuntimeError(f"no transform shape for N = {N} passed its check")
     bf = min(good, key=lambda c: (c["ms_fwd"], c["index"]))
     bi = min(good, key=lambda c: (c["ms_inv"], c["index"]))
-    d0 = next((c for c in good if c["index"] == 0), None)
     res = {"fwd": bf["shape"], "inv": bi["shape"], "ms_fwd": bf["ms_fwd"], "ms_inv": bi["ms_inv"],
-           "default_ms_fwd_inv": (d0["ms_fwd"] + d0["ms_inv"]) if d0 else None, "candidates": cands}
+           "unset_ms_fwd": unset_f, "unset_ms_inv": unset_i, "default_ms_fwd_inv": unset_f + unset_i,
+           "applied_fwd": bf["shape"] if bf["ms_fwd"] < unset_f * (1 - MARGIN) else None,
+           "applied_inv": bi["shape"] if bi["ms_inv"] < unset_i * (1 - MARGIN) else None, "candidates": cands}
     if cache_path:
         cache = _load_cache(cache_path)
         cache[key] = res
@@ -144,8 +158,8 @@ def tune_uniform(N: int, limbs: int, count: int, moduli=None, reps: int = 10, wa
 
 
 def _apply(N, res):
-    for direction, key in ((he.FORWARD, "fwd"), (he.INVERSE, "inv")):
-        lb, le, pers, occ = (list(res[key]) + [0])[:4]
+    for direction, key in ((he.FORWARD, "applied_fwd"), (he.INVERSE, "applied_inv")):
+        lb, le, pers, occ = res[key] or (0, 0, 0, 0)
         he.ntt_set_shape(N, lb, le, pers, direction=direction, ctas_per_sm=occ)
 
 
@@ -190,7 +204,10 @@ def tune_mul_relin_rescale(ctx, key, level: int, count: int, reps: int = 10, war
                            apply: bool = True) -> dict:
     """Pick the words per thread (radix-8 or radix-16 rounds) of a context's
     key-switching and rescale kernels for `count` MulLinRS at `level`:
-    each candidate must reproduce the default's output bit for bit."""
+    each candidate must reproduce the untuned output bit for bit. The faster
+    one is applied ("applied") where it beats the unset state, in which every
+    stage chooses by its size, by more than MARGIN; otherwise 0, the unset
+    state, stays."""
     import torch
 
     N = ctx.N
@@ -204,6 +221,7 @@ def tune_mul_relin_rescale(ctx, key, level: int, count: int, reps: int = 10, war
     ctx.set_eval_shape(0)
     he.mul_relin_rescale(out, a, b, count, key, ctx, level, scratch)
     ref = out.clone()
+    unset = _time(lambda: he.mul_relin_rescale(out, a, b, count, key, ctx, level, scratch), reps, warmup)
     cands = []
     for idx, le in enumerate((4, 3)):
         ctx.set_eval_shape(le)
@@ -215,5 +233,6 @@ def tune_mul_relin_rescale(ctx, key, level: int, count: int, reps: int = 10, war
         cands.append({"index": idx, "log_thread_words": le, "ok": ok, "ms": ms})
     good = [c for c in cands if c["ok"]]
     best = min(good, key=lambda c: (c["ms"], c["index"]))
-    ctx.set_eval_shape(best["log_thread_words"] if apply else 0)
-    return {"log_thread_words": best["log_thread_words"], "candidates": cands}
+    applied = best["log_thread_words"] if best["ms"] < unset * (1 - MARGIN) else 0
+    ctx.set_eval_shape(applied if apply else 0)
+    return {"log_thread_words": best["log_thread_words"], "applied": applied, "unset_ms": unset, "candidates": cands}

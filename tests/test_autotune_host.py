@@ -191,3 +191,31 @@ def test_mul_relin_rescale_radix_needs_the_default_output(fake, monkeypatch):
         assert res["log_thread_words"] == want, (broken, ms)
         assert [c["ok"] for c in res["candidates"]] == [broken != 4, broken != 3]
         assert ctx.set_calls[0] == 0 and ctx.set_calls[-1] == want      # default first, the choice applied
+
+
+@pytest.mark.parametrize("ms,applied", [(10.0, False), (9.9, False), (9.7, True)])
+def test_a_fixed_shape_must_beat_the_unset_state(fake, tmp_path, ms, applied):
+    """With no shape set every call chooses by its own batch: a fixed shape,
+    which holds for all later calls of the degree, is applied only if it is
+    clearly faster on the tuned batch; from the cache just the same."""
+    path = str(tmp_path / "c.json")
+    he = fake(shapes=SHAPES, ms={(_s(1), "fwd"): ms, (_s(2), "inv"): ms})
+    res = autotune.tune_uniform(1024, 2, 3, reps=2, warmup=1, cache_path=path)
+    want = [(he.FORWARD, _s(1) if applied else None), (he.INVERSE, _s(2) if applied else None)]
+    assert he.set_calls[-2:] == want and res["unset_ms_fwd"] == res["unset_ms_inv"] == 10.0
+    he = fake(shapes=SHAPES, ms={})
+    autotune.tune_uniform(1024, 2, 3, cache_path=path)
+    assert he.set_calls == want
+
+
+def test_mul_relin_rescale_keeps_the_choice_by_size(fake, monkeypatch):
+    fake(shapes=SHAPES, ms={})
+
+    def mrr(out, a, b, count, key, c, level, scratch, stream=None):
+        out.copy_(a[:, :, :level] + b[:, :, :level])
+        _Clock.t += c.ms[c.shape]
+    monkeypatch.setattr(autotune.he, "mul_relin_rescale", mrr, raising=False)
+    for ms, want in (({0: 1.0, 4: 1.0, 3: 2.0}, 0), ({0: 1.0, 4: 2.0, 3: 0.99}, 0), ({0: 1.0, 4: 0.9, 3: 2.0}, 4)):
+        ctx = _Ctx(None, ms)
+        res = autotune.tune_mul_relin_rescale(ctx, None, 2, 3, reps=2, warmup=1)
+        assert ctx.set_calls[-1] == res["applied"] == want
