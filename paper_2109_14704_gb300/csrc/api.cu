@@ -908,7 +908,6 @@ static he_status ks_mac(const he_context *ctx, const he::EvalArgs &a, u32 gs, cu
         HE_CUDA(he::launch_k(he::k_ks_mac<false, KIND>, mac_grid(tiles), he::MAC_BLOCK / 2, 0, 1, s, a, gs, tiles,
                              he::NoJobs{}));
     }
-    HE_CUDA(cudaGetLastError());
     return HE_OK;
 }
 
@@ -1293,7 +1292,6 @@ extern "C" he_status he_ct_matmul_tensor(uint64_t *t_out, const uint64_t *a, con
     else if (m > 1) HE_CUDA(launch(he::k_ct_matmul_tensor<2, 1>, 2, 1));
     else if (n > 1) HE_CUDA(launch(he::k_ct_matmul_tensor<1, 2>, 1, 2));
     else HE_CUDA(launch(he::k_ct_matmul_tensor<1, 1>, 1, 1));
-    HE_CUDA(cudaGetLastError());
     return HE_OK;
 }
 

@@ -50,7 +50,10 @@ static cudaError_t launch_k(K kernel, u32 grid, u32 block, u32 smem, u32 cluster
         attr[1].val.clusterDim.z = 1;
         cfg.numAttrs = 2;
     }
-    return cudaLaunchKernelEx(&cfg, kernel, args...);
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, args...);
+    // a refused launch is reported here and not by a later call's check as well
+    if (e != cudaSuccess) cudaGetLastError();
+    return e;
 }
 #endif
 
