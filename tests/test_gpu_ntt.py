@@ -49,22 +49,33 @@ def test_ntt_parity_every_degree(log_n):
 
 
 @pytest.mark.parametrize("log_n", [10, 12, 15])
-@pytest.mark.parametrize("offset_words", [0, 4])
-def test_forward_store_forms(log_n, offset_words):
-    """The forward transform of a uniform batch leaves by bulk tensor stores
-    when the batch is 128-byte aligned and by plain stores otherwise (a
-    32-byte aligned view 4 words into its buffer); both equal the oracle, and
-    the words around the batch are untouched."""
+@pytest.mark.parametrize("offset_words", [16, 4])
+@pytest.mark.parametrize("set_shape", [True, False])
+def test_forward_store_forms(log_n, offset_words, set_shape):
+    """The forward transform of a uniform batch with 16 words a thread leaves by
+    bulk tensor stores when the batch is 128-byte aligned and by plain stores
+    otherwise (a 32-byte aligned view 4 words into its buffer), in a set shape
+    and, with none set, above the small-batch limit; every limb equals the
+    oracle's, and the words around the batch are untouched."""
     N = 1 << log_n
-    limbs, count = 3, 3
+    limbs = 3
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    count = 3 if set_shape else sms * 4096 // (limbs * N) + 1
+    assert set_shape or count * limbs * N > sms * 4096
     qs = _moduli(N, limbs)
     tables = he.NttTables(N, qs)
-    x = np.stack([Rng(log_n * 100 + p).uniform_limbs(qs, N) for p in range(count)])
-    buf = torch.full((count * limbs * N + 8,), 777, dtype=torch.int64, device="cuda")
+    r = Rng(log_n * 100)
+    x = np.stack([r.uniform_limbs(qs, N) for _ in range(count)])
+    buf = torch.full((count * limbs * N + 32,), 777, dtype=torch.int64, device="cuda")
     d = buf[offset_words:offset_words + count * limbs * N].view(count, limbs, N)
-    assert d.data_ptr() % 128 == (0 if offset_words == 0 else 32)
+    assert d.data_ptr() % 128 == (0 if offset_words == 16 else 32)
     d.copy_(dev(x))
-    he.ntt_fwd(d, N, limbs, count, tables)
+    try:
+        if set_shape:
+            he.ntt_set_shape(N, min(log_n, 12), 4)
+        he.ntt_fwd(d, N, limbs, count, tables)
+    finally:
+        he.ntt_set_shape(N, 0, 0)
     got = host(d)
     for p in range(count):
         assert np.array_equal(got[p], oracle.ntt_fwd(x[p], qs)), p
