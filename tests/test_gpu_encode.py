@@ -337,3 +337,32 @@ def test_encrypt_seeded_matches_oracle(level):
     he.encrypt(ct2, pt, dev(keys.pk), dv, d0, d1, count, ctx, level,
                empty(ctx.encrypt_scratch_bytes(level, count) // 8))
     assert np.array_equal(host(ct2), got)
+
+
+@pytest.mark.parametrize("log_n,n,count,log_e", [(10, 3, 2, 3), (10, 3, 2, 4), (14, 2, 2, 3), (14, 2, 2, 4),
+                                                 (15, 3, 1, 3), (15, 3, 1, 4), (16, 2, 1, 3), (16, 2, 1, 4),
+                                                 (15, 3, 5, 0)])
+def test_encrypt_transform_forms(log_n, n, count, log_e):
+    """Encryption in both forms of its transforms, 8 and 16 words a thread, set
+    and (the last case, above the small-batch limit) by the batch's size: from
+    a seed and from given draws, bit for bit the oracle's."""
+    N = 1 << log_n
+    data, P = he.chain_primes(N, [60] + [50] * n, 60)     # one prime more than the level holds
+    qs = data[:n]
+    r = Rng(940 + log_n)
+    keys = ckks.Keys(N, data, P, None, np.stack([r.uniform_limbs(data, N) for _ in range(2)]), None)
+    ctx = he.Context(N, data, P)
+    ctx.set_eval_shape(log_e)
+    if not log_e:
+        assert 3 * count * n * N > 2 * 4096 * torch.cuda.get_device_properties(0).multi_processor_count
+    seed = 0xFEDC_BA98_7654_3210
+    m = [r.gaussian(N) << 20 for _ in range(count)]
+    draws = ckks.encryption_draws(seed, count, N)
+    want = np.stack([ckks.encrypt_with_draws(m[c], keys, *[d[c] for d in draws], n - 1) for c in range(count)])
+    pt = dev(np.stack([oracle.ntt_fwd(ckks.to_residues(m[c], qs), qs) for c in range(count)]))
+    sc = empty(ctx.encrypt_scratch_bytes(n - 1, count) // 8)
+    for call in (lambda ct: he.encrypt_seeded(ct, pt, dev(keys.pk), seed, count, ctx, n - 1, sc),
+                 lambda ct: he.encrypt(ct, pt, dev(keys.pk), *map(_i8, draws), count, ctx, n - 1, sc)):
+        ct = empty(count, 2, n, N)
+        call(ct)
+        assert np.array_equal(host(ct), want)
