@@ -1,6 +1,6 @@
-"""Shapes the library picks by batch size: transforms and products on both sides
-of the small-batch limit give the same words as the oracle and as a fixed
-shape, forward, inverse and back."""
+"""Shapes the library picks by batch size: transforms (forward and inverse) and
+products on both sides of every limit give the oracle's words, on batches whose
+limbs all differ, with one prime and with three."""
 import numpy as np
 import pytest
 
@@ -19,24 +19,27 @@ def test_auto_shape_sides(log_n):
     N = 1 << log_n
     sms = torch.cuda.get_device_properties(0).multi_processor_count
     limit = sms * 4096 // N
-    qs = he.primes_generate(60, 2 * N, 1)
-    t = he.NttTables(N, qs)
+    edges = [1, 8, sms // 8, (sms - 8) // 4, limit * 3 // 4, limit]
+    edges = sorted({c + d for c in edges for d in (0, 1)} - {0})
     r = Rng(log_n)
-    row = r.uniform_limbs(qs, N)
-    want_f, want_i = oracle.ntt_fwd(row, qs)[0], oracle.ntt_inv(row, qs)[0]
-    edges = [1, 8, sms // 8, limit * 3 // 4, limit]
-    for count in sorted({c + d for c in edges for d in (0, 1)} - {0}):
-        for f, want in ((he.ntt_fwd, want_f), (he.ntt_inv, want_i)):
-            d = dev(row).repeat(count, 1).contiguous()
-            f(d, N, 1, count, t)
-            got = host(d)
-            assert np.array_equal(got[0], want) and (got == want).all(), count
-        a = dev(row).repeat(count, 1).contiguous()
-        c = torch.empty_like(a)
-        he.negacyclic_mul(c, a, a, N, 1, count, t)
-        if count == 1:
-            want_c = oracle.negacyclic_mul(row, row, qs)[0]
-        assert (host(c) == want_c).all(), count
+    for limbs in (1, 3):              # limb i of the batch uses prime i mod limbs
+        qs = he.primes_generate(60, 2 * N, limbs)
+        t = he.NttTables(N, qs)
+        counts = [c // limbs for c in edges if c % limbs == 0]
+        if not counts:
+            continue
+        x, y = (np.stack([r.uniform_limbs(qs, N) for _ in range(counts[-1])]) for _ in range(2))
+        fwd = np.stack([oracle.ntt_fwd(p, qs) for p in x])
+        inv = np.stack([oracle.ntt_inv(p, qs) for p in x])
+        product = np.stack([oracle.negacyclic_mul(p, q, qs) for p, q in zip(x, y)])
+        for count in counts:
+            for f, want in ((he.ntt_fwd, fwd), (he.ntt_inv, inv)):
+                d = dev(x[:count])
+                f(d, N, limbs, count, t)
+                assert np.array_equal(host(d), want[:count]), (limbs, count)
+            c = empty(count, limbs, N)
+            he.negacyclic_mul(c, dev(x[:count]), dev(y[:count]), N, limbs, count, t)
+            assert np.array_equal(host(c), product[:count]), (limbs, count)
 
 
 @pytest.mark.parametrize("log_n", [12, 15, 16])
@@ -46,13 +49,14 @@ def test_auto_shape_fused_modup(log_n):
     data, P = he.chain_primes(N, [50] * n, 60)
     r = Rng(log_n)
     evk = np.stack([np.stack([r.uniform_limbs(data + [P], N) for _ in range(2)]) for _ in range(n)])
-    ct = np.stack([r.uniform_limbs(data, N) for _ in range(2)])
-    want = oracle.mul_relin_rescale(ct, ct, evk, data, P, n - 1)
+    limit = torch.cuda.get_device_properties(0).multi_processor_count * 4096 // N // (n + 1)
+    ca, cb = (np.stack([np.stack([r.uniform_limbs(data, N) for _ in range(2)]) for _ in range(limit + 1)])
+              for _ in range(2))
+    want = np.stack([oracle.mul_relin_rescale(a, b, evk, data, P, n - 1) for a, b in zip(ca, cb)])
     ctx = he.Context(N, data, P)
     key = he.RelinKey(ctx, evk)
-    limit = torch.cuda.get_device_properties(0).multi_processor_count * 4096 // N // (n + 1)
     for count in (limit, limit + 1):
-        a = dev(ct[None]).repeat(count, 1, 1, 1).contiguous()
         out = empty(count, 2, n - 1, N)
-        he.mul_relin_rescale(out, a, a, count, key, ctx, n - 1, empty(ctx.mrr_scratch_bytes(n - 1, count, 0) // 8))
-        assert (host(out) == want).all(), count
+        he.mul_relin_rescale(out, dev(ca[:count]), dev(cb[:count]), count, key, ctx, n - 1,
+                             empty(ctx.mrr_scratch_bytes(n - 1, count, 0) // 8))
+        assert np.array_equal(host(out), want[:count]), count
