@@ -416,7 +416,6 @@ static int num_sms()
 
 static u64 small_batch_words() { return he::small_batch_words((u32)num_sms()); }
 
-// One launch of a batch of limb transforms in the shape set for the degree.
 // cuTensorMapEncodeTiled, fetched through the runtime's driver entry points
 // (the library does not link the driver library); null if unavailable.
 typedef CUresult (*PfnEncodeTiled)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *,
@@ -459,6 +458,8 @@ static bool batch_tmap(he::NttLaunch &a, u32 N)
                CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
 }
 
+// One launch of a batch of limb transforms, in the shape set for the degree or,
+// with none set, in one for the batch's size.
 static he_status ntt_launch(const he::NttLaunch &a0, int log_n, bool inv, cudaStream_t stream)
 {
     const he::DegreeOps *ops = he::degree_ops(log_n);
@@ -885,15 +886,6 @@ static he_status plift_intt(const he_context *ctx, u64 *plift, u32 limbs, cudaSt
 // CTAs of the per-tile key multiply-accumulate: one a tile up to 16 an SM
 static u32 mac_grid(u64 tiles) { return (u32)std::max<u64>(1, std::min<u64>(tiles, (u64)num_sms() * 16)); }
 
-// Mod-up of key switching for `count` ciphertexts (a.c2 holds their
-// coefficient-domain digits): accq and plift as k_ks_modup leaves them.
-// With room for the expanded buffer (x_words at xbuf, at least one
-// ciphertext's (n + 1) n N words) the transforms run as independent plain-
-// size launches (k_ks_expand), the key products as an elementwise pass
-// (k_ks_mac); the buffer takes groups of up to kModupGroup ciphertexts, and
-// the special prime's accumulators in plift are left in the NTT domain
-// (*special_ntt = true). Otherwise the fused k_ks_modup runs, which also takes
-// them through the inverse transform.
 // The key multiply-accumulate of a uniform group of gs ciphertexts.
 template <int KIND>
 static he_status ks_mac(const he_context *ctx, const he::EvalArgs &a, u32 gs, cudaStream_t s)
@@ -922,6 +914,15 @@ static he::EvalKernel digits_kernel(const he::EvalArgs &a)
     return k == he::SRC_PAIR ? he::EK_KS_DIGITS : (k == he::SRC_THREE ? he::EK_KS_DIGITS_THREE : he::EK_KS_DIGITS_ROTATE);
 }
 
+// Mod-up of key switching for `count` ciphertexts (a.c2 holds their
+// coefficient-domain digits): accq and plift as k_ks_modup leaves them.
+// With room for the expanded buffer (x_words at xbuf, at least one
+// ciphertext's (n + 1) n N words) the transforms run as independent plain-
+// size launches (k_ks_expand), the key products as an elementwise pass
+// (k_ks_mac); the buffer takes groups of up to kModupGroup ciphertexts, and
+// the special prime's accumulators in plift are left in the NTT domain
+// (*special_ntt = true). Otherwise the fused k_ks_modup runs, which also takes
+// them through the inverse transform.
 static he_status ks_modup(const he_context *ctx, he::EvalArgs &a, u32 count, u64 *xbuf, size_t x_words,
                           bool *special_ntt, cudaStream_t s)
 {
@@ -1005,8 +1006,9 @@ extern "C" he_status he_rescale(uint64_t *ct_out, const uint64_t *ct_in, const h
 // Key switching of `count` ciphertexts whose third component is given either
 // as the tensor of a pair (ct_a, ct_b: Mul fused into the loads), as a
 // three-component input ct3, or (galois nonzero) as the rotation (sigma(c0), 0,
-// sigma(c1)) of two-component inputs ct3, gathered on the loads; then (rescale = true) RS by q_l (MulLinRS
-// kernels) or (rescale = false) the mod-down only (MulLin / Relin).
+// sigma(c1)) of two-component inputs ct3, gathered on the loads; then (rescale =
+// true) RS by q_l (MulLinRS kernels) or (rescale = false) the mod-down only
+// (MulLin / Relin).
 static he_status key_switch_common(uint64_t *ct_out, const uint64_t *ct_a, const uint64_t *ct_b, const uint64_t *ct3,
                                    uint32_t count, const he_relin_key *key, const he_context *ctx, uint32_t level,
                                    void *scratch, size_t scratch_bytes, he_stream_t stream, bool rescale,
@@ -1125,7 +1127,7 @@ static he_status mrr_jobs_pass(const he_mrr_job *jobs, u32 n_jobs, const he_reli
     u64 tot[he::JS_COUNT] = {};
     u32 pairs = 0;
     for (u32 i = 0; i < n_jobs; i++) pairs += jobs[i].count;
-    u64 *plift = w;                       // [all pairs][2][N], contiguous for one transform launch
+    u64 *plift = w;                       // [all pairs][2][N]
     w += (size_t)pairs * 2 * ctx->N;
     u64 *pl = plift;
     for (u32 i = 0; i < n_jobs; i++) {
@@ -1238,8 +1240,7 @@ extern "C" he_status he_ct_automorph(uint64_t *ct_out, const uint64_t *ct_in, ui
     if (count == 0 || components == 0) return HE_OK;
     const u64 words = (u64)count * components * (level + 1) * ctx->N;
     HE_CUDA(he::launch_k(he::k_ct_automorph, stream_grid(words, 256), 256, 0, 1, (cudaStream_t)stream, ct_out, ct_in,
-                         words,
-                                                                                  (u32)ctx->log_n, galois_elt));
+                         words, (u32)ctx->log_n, galois_elt));
     return HE_OK;
 }
 
@@ -1574,8 +1575,7 @@ static he_status encrypt_common(uint64_t *ct_out, const uint64_t *pt, const uint
     a.ctx = dev_ctx(ctx);
     if (he_status r = run_eval(ctx, he::EK_ENC_NOISE, a, 3 * count * n, s)) return r;
     HE_CUDA(he::launch_k(he::k_enc_combine, stream_grid((u64)count * n * ctx->N / 2, 256), 256, 0, 1, s, ct_out,
-                         noise,
-                         pt, pk, (u32)ctx->log_n, n, count, ctx->n_data, ctx->tables->d_pc));
+                         noise, pt, pk, (u32)ctx->log_n, n, count, ctx->n_data, ctx->tables->d_pc));
     return HE_OK;
 }
 
@@ -1604,8 +1604,7 @@ extern "C" he_status he_sample_encryption_draws(int8_t *v, int8_t *e0, int8_t *e
     if (count == 0) return HE_OK;
     if ((u64)count * N > (1ull << 40)) return fail(HE_EINVAL, "batch too large");
     HE_CUDA(he::launch_k(he::k_enc_draws, stream_grid((u64)count * N, 256), 256, 0, 1, (cudaStream_t)stream, v, e0,
-                         e1, seed,
-                                                                                        (u32)log_n, count));
+                         e1, seed, (u32)log_n, count));
     return HE_OK;
 }
 

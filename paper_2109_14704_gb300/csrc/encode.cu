@@ -279,8 +279,8 @@ __device__ __forceinline__ double mw_to_double(u64 (&v)[NW])
 // and neither products nor multi-word sums are needed: one reduction a limb
 // instead of 4 NW products and the corrections. Anything else fails at the
 // second limb with all but a 2^-30 chance and takes the general path. Bound by
-// its reads then: 64 messages of 2^15 coefficients at 8 limbs (151 MB), 205 us
-// by the general path, 44 us by this one. primes: (q_i, floor(2^64 / q_i)).
+// its reads then: 64 messages of 2^15 coefficients at 8 limbs (151 MB), 199 us
+// by the general path, 43 us by this one. primes: (q_i, floor(2^64 / q_i)).
 template <int NW>
 __global__ void __launch_bounds__(128) k_crt_compose(double *out, const u64 *coef, const u64 *tab, const u64 *primes,
                                                      u32 log_N, u32 limbs, u64 total)

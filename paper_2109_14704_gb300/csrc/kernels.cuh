@@ -59,14 +59,15 @@ __device__ __forceinline__ void tma_store_rows(const u64 (&x)[16], u32 wbase, co
 }
 
 // Forward or inverse transform of one limb stored at `data` (in place; the
-// inverse reads its input at `src`, which may be another buffer). The forward transform's last round and the inverse transform's first round
-// give each thread runs of consecutive words, which move as 32-byte quarters
-// (streaming cache hints: every word is read and written once per launch);
-// the cross-CTA columns move as single coalesced words. Stores are skipped
-// when !valid (idle sub-clusters of the mixed-degree kernel). With a tensor
-// map tm (forward, 16 words a thread, the limb block's first row row0) the
-// output leaves by bulk tensor stores instead, where the warp's rows in
-// shared memory are 1024-byte aligned (the swizzle's period).
+// inverse reads its input at `src`, which may be another buffer). The forward
+// transform's last round and the inverse transform's first round give each
+// thread runs of consecutive words, which move as 32-byte quarters (streaming
+// cache hints: every word is read and written once per launch); the cross-CTA
+// columns move as single coalesced words. Stores are skipped when !valid (idle
+// sub-clusters of the mixed-degree kernel). With a tensor map tm (forward, 16
+// words a thread, the limb block's first row row0) the output leaves by bulk
+// tensor stores instead, where the warp's rows in shared memory are 1024-byte
+// aligned (the swizzle's period).
 template <class Sh, bool INV>
 __device__ __forceinline__ void ntt_limb(u64 *smem, u32 m, u32 rbase, u64 *data, const ulonglong2 *tw,
                                          const PrimeConst &pc, const u64 *src, bool valid = true,
@@ -663,8 +664,6 @@ __device__ __forceinline__ void store_run(u64 *dst, const u64 (&x)[Sh::E], u32 m
     for (int e = 0; e < Sh::E; e += 4) st4(dst + last_pos<Sh>(m, tid, e), x[e], x[e + 1], x[e + 2], x[e + 3]);
 }
 
-// d_k[i] at position P for component k (0 or 1): from the tensor of the two
-// input ciphertexts (fused Mul) or from a 3-component input.
 // Job of a mixed-level batch that owns global item `item` of stage S (the
 // last job whose first item is not above it): its buffers and sizes go into
 // a, and the item's index within the job is returned.
@@ -695,6 +694,9 @@ __device__ __forceinline__ u32 bind_job(EvalArgs &a, const JobTable &t, int S, u
     return item - J.begin[S];
 }
 
+// The input of a key switch of one ciphertext. d(k, limb, ..., P): component k of
+// its three at position P, from the tensor of the two input ciphertexts (fused
+// Mul), from a 3-component input, or through the automorphism.
 struct DSource {
     const u64 *ct_a, *ct_b, *ct3;  // per-ciphertext bases
     size_t per;                    // n * N words per component
@@ -919,7 +921,8 @@ k_ks_modup(EvalArgs a)
 // Expanded mod-up, first half: one transform per cluster,
 //   X[g][t][j] = NTT_t(c2_j mod t)  for each digit j != t, target t in
 //   {q_0..q_l, P}, ciphertext c = c_first + g of the group,
-// left in the lazy range [0, 12t) (it only feeds Shoup products). The same
+// left in the lazy range [0, 8t + 2^32): the 128-bit key sums (MacSums::digit)
+// rely on that bound, not only on 12t, which would overflow them. The same
 // transforms as k_ks_modup, but as independent launches of the plain
 // transform's size and register budget instead of a sequence inside one
 // accumulating cluster; k_ks_mac or k_ks_mac_tiled then accumulates them.

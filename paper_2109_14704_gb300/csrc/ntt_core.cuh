@@ -488,8 +488,9 @@ __device__ __forceinline__ void fwd_cross(u64 *s, u32 tid, u32 m, u32 rbase, con
 // receives the canonical output at bit-reversed evaluation index P. After
 // the call the canonical values also remain in x[] in the last round's order
 // (see last_pos). With CANON = false the final reduction is skipped: x[] and
-// store receive values in [0, 8p + 2^32), below 12p for p >= 2^30, for
-// callers that feed them straight into a Shoup product (any 64-bit input).
+// store receive values in [0, 8p + 2^32), below 12p for p >= 2^30, for callers
+// that feed them into a Shoup product (any 64-bit input) or into the key sums
+// (MacSums::digit, which needs the range as stated).
 template <class Sh, bool CANON = true, bool ROLL = false, class Load, class Store>
 __device__ __forceinline__ void ntt_fwd_block(u64 *s, u32 m, u32 rbase, const ulonglong2 *tw,
                                               const PrimeConst &pc, Load load, Store store, u64 (&x)[Sh::E])
