@@ -240,13 +240,25 @@ def mrr_work(n: int, N: int) -> dict:
     n^2 + 5n + 2 transforms of (N/2) log2 N butterflies; N (2n^2 + 16n - 4)
     further modular products (tensor 4n, key products 2n(n+1), d P 2n,
     mod-down 2n + 2n centred reductions, rescale 2(n-1) + 2(n-1)): the method
-    as written, one transform per limb and division; the kernels share one
-    between the two divisions and run n^2 + 3n + 2. HBM bytes: the two input
+    as written, one transform per limb and division. HBM bytes: the two input
     ciphertexts read and the output written once (the resident key is not
     counted)."""
     log_n = N.bit_length() - 1
     return {"bfly": (n * n + 5 * n + 2) * (N // 2) * log_n, "products": N * (2 * n * n + 16 * n - 4),
             "bytes": (4 * n + 2 * (n - 1)) * N * 8}
+
+
+def mrr_run_work(n: int, N: int) -> dict:
+    """The work the kernels run for one MulLinRS, which its rooflines count: one
+    transform serves both divisions of a limb, so n^2 + 3n + 2 transforms
+    (digits n, expansion n^2, special prime and q_l back 4, the rest 2(n-1)); and
+    N (2n^2 + 15n - 8) further products: the digits' loads n, the key sums
+    2n + 4 a data prime (tensor terms 3, the diagonal digit 1) and 2n on the
+    special prime, the shared division 4 a word of its 2(n-1) limbs. Bytes as
+    mrr_work."""
+    log_n = N.bit_length() - 1
+    return {"bfly": (n * n + 3 * n + 2) * (N // 2) * log_n, "products": N * (2 * n * n + 15 * n - 8),
+            "bytes": mrr_work(n, N)["bytes"]}
 
 
 def roof_entry(work: dict, seconds: float, alu_peak: float, hbm_peak: float) -> dict:
@@ -515,7 +527,7 @@ def run_ours(args, rank, world, local):
     attach_rooflines(uneven, alu_peak, hbm_peak)
     attach_rooflines(matrix, alu_peak, hbm_peak)
     attach_rooflines(routines, alu_peak, hbm_peak)
-    mrr_roof = roof_entry({k: v * MRR_COUNT for k, v in mrr_work(L + 1, MRR_N).items()}, ms_mrr / 1e3,
+    mrr_roof = roof_entry({k: v * MRR_COUNT for k, v in mrr_run_work(L + 1, MRR_N).items()}, ms_mrr / 1e3,
                           alu_peak, hbm_peak)
     value = job_value(world, 2 * limbs_total, ms)
     e2e_value = job_value(world, 2 * limbs_total, ms_e2e)
@@ -561,7 +573,7 @@ def run_ours(args, rank, world, local):
             "ms_per_batch": ms_mrr,
             "batch_distribution": mrr_dist,
             "transforms_per_op": (L + 1) ** 2 + 3 * (L + 1) + 2,   # as the kernels run them
-            "work_per_op": mrr_work(L + 1, MRR_N),
+            "work_per_op": mrr_run_work(L + 1, MRR_N),
             "roofline": mrr_roof,
             "autotune": mrr_tune,
         },
@@ -860,7 +872,7 @@ def bench_matrix(args, stream, barrier):
     ms = _time_steps(step, args.steps, args.warmup, stream, barrier)
     res = {"workload": "32x32 element-wise, N=8192, primes 60/40/40 + 60, 1024 MulLinRS per step",
            "ms_per_step": ms, "mul_relin_rescale_per_s": count / (ms / 1e3),
-           "_work": dict({k: v * count for k, v in mrr_work(L + 1, N).items()}, seconds=ms / 1e3),
+           "_work": dict({k: v * count for k, v in mrr_run_work(L + 1, N).items()}, seconds=ms / 1e3),
            "eval_log_thread_words": tune["applied"] or "by stage size"}
     del A, B, out, scratch
     # the encrypted matrix product C += A B (matMul_mxnxk): tensors
@@ -932,7 +944,7 @@ def bench_routines(args, stream, barrier):
         ms = _time_steps(fn, max(3, args.steps // 2), 3, stream, barrier)
         res[name] = {"ms_per_batch": ms, "per_s": count / (ms / 1e3)}
         if name in ("mul_lin_rs", "sqr_lin_rs"):
-            res[name]["_work"] = dict({k: v * count for k, v in mrr_work(L + 1, N).items()}, seconds=ms / 1e3)
+            res[name]["_work"] = dict({k: v * count for k, v in mrr_run_work(L + 1, N).items()}, seconds=ms / 1e3)
     return res
 
 

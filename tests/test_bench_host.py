@@ -106,3 +106,21 @@ def test_mul_relin_rescale_transform_count():
             w = bench.mrr_work(n, N)
             assert w["bfly"] == stages * (N // 2) * (N.bit_length() - 1)
             assert w["bytes"] == (2 * 2 * n + 2 * (n - 1)) * N * 8
+
+
+def test_mul_relin_rescale_work_as_run():
+    """What the rooflines count, stage by stage of the kernels at n data limbs:
+    transforms of the digits (n), the expansion (n - 1 digits at each data
+    prime, n at P), the lifts of P and q_l (2 + 2) and the shared division
+    (2(n - 1)); products of the digits' loads, the key sums (per data prime 2n
+    key products, 3 tensor terms and the diagonal digit's own; 2n at P) and the
+    shared division (3 on each load, 1 after it)."""
+    for n in (2, 3, 7, 17):
+        transforms = n + n * (n - 1) + n + 4 + 2 * (n - 1)
+        products = n + n * (2 * n + 4) + 2 * n + 4 * 2 * (n - 1)
+        for N in (4096, 16384):
+            w = bench.mrr_run_work(n, N)
+            assert w["bfly"] == transforms * (N // 2) * (N.bit_length() - 1)
+            assert w["products"] == products * N
+            assert w["bytes"] == bench.mrr_work(n, N)["bytes"]
+            assert transforms == n * n + 3 * n + 2
