@@ -434,6 +434,7 @@ def run_ours(args, rank, world, local):
     gc.disable()
     try:
         ms_e2e = max_over_ranks(_time_steps(step_e2e, max(3, args.steps), max(3, args.warmup), stream, barrier))
+        e2e_dist = _distribution(_step_times(step_e2e, max(20, args.steps), stream))
     finally:
         gc.enable()
     torch.cuda.synchronize()
@@ -598,7 +599,7 @@ def run_ours(args, rank, world, local):
             "butterflies_per_launch": bfly_per_launch,
         },
         "e2e": {"value": e2e_value, "unit": UNIT, "h2d_bytes_per_step": 8 * limbs_total * N,
-                "d2h_bytes_per_step": 8 * limbs_total * N, "ms_per_step": ms_e2e,
+                "d2h_bytes_per_step": 8 * limbs_total * N, "ms_per_step": ms_e2e, "step_distribution": e2e_dist,
                 "call": "he_ntt_host(forward | inverse), pinned host buffers, 4 streams x 32-polynomial chunks",
                 "whole_batch_copies_value": world * 2 * limbs_total / (ms_serial / 1e3),
                 "host_link": {"ms_copy_in_and_out": ms_link, "ms_whole_batch_copies": ms_link_whole,
@@ -980,8 +981,14 @@ def bench_encode(args, stream, barrier):
                          barrier)
     torch.cuda.synchronize()
     err = float(((zo - z).abs().max() / z.abs().max()).item())
+    # the CRT lift as decoding meets it, on the messages' coefficients, and its
+    # general path, on uniform residues
     coef.copy_(pt)
+    he.ntt_inv(coef, N, level + 1, count, tables, stream=stream)
     ms_crt = _time_steps(lambda: enc.crt_compose(m, coef, count, level, stream=stream), steps, 3, stream, barrier)
+    coef.copy_(pt)
+    ms_crt_general = _time_steps(lambda: enc.crt_compose(m, coef, count, level, stream=stream), steps, 3, stream,
+                                 barrier)
     ms_fwd = _time_steps(lambda: he.ntt_fwd(coef, N, level + 1, count, tables, stream=stream), steps, 3, stream,
                          barrier)
     ms_inv = _time_steps(lambda: he.ntt_inv(coef, N, level + 1, count, tables, stream=stream), steps, 3, stream,
@@ -1000,6 +1007,7 @@ def bench_encode(args, stream, barrier):
         "decode": {"ms_per_batch": ms_dec, "per_s": count / (ms_dec / 1e3)},
         "round_trip_max_rel_err": err,
         "components_ms": {"ntt_fwd": ms_fwd, "ntt_inv": ms_inv, "crt_lift": ms_crt,
+                          "crt_lift_general": ms_crt_general,
                           "encode_minus_ntt": ms_fft_enc, "decode_minus_intt_crt": ms_dec - ms_inv - ms_crt},
         "fp64": {"probe_tflops": fp64_peak,
                  "encode_fft_tflops": fft_flop / (ms_fft_enc / 1e3) / 1e12,
